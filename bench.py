@@ -715,7 +715,7 @@ def extras(args, ctx, lat, b, b_dev, x_dev, solve_kw, mixed_ms, torch, bqcd):
         torch.cuda.synchronize()
         t = e0.elapsed_time(e1) / n * 1e-3
         pid = PREC_ID[prec]
-        byts = (8 * link_b(pid, recon) + 2 * SPINOR_B[pid]) * Vh
+        byts = (8 * link_b(pid, 18 if pid == 0 else recon) + 2 * SPINOR_B[pid]) * Vh  # FP64 keeps all 18 reals
         sweep[f"{prec}_r{recon}" + (f"_{arith}" if arith else "")] = {
             "GB/s": byts / t / 1e9, "GFLOP/s": 1320.0 * Vh / t / 1e9, "us": t * 1e6}
     bqcd.bq_set_recon(ctx, "double", 18)

@@ -135,7 +135,9 @@ int bq_set_params(bq_ctx *ctx, const bq_params *p);
  * (first two rows; the third is rebuilt as conj(row1 x row2)) or, for
  * BQ_PREC_SINGLE and BQ_PREC_HALF, BQ_RECON_8 (U01, U02, U10 and the phases of
  * U00 and U20; the rest rebuilt from unitarity and det U = 1, with two sine /
- * cosine evaluations, two square roots and one reciprocal per link). 12 and 8
+ * cosine evaluations, two square roots and one reciprocal per link). For
+ * BQ_PREC_DOUBLE the third row of BQ_RECON_12 is rebuilt once, when the links are
+ * packed, and kept with the other two. 12 and 8
  * are valid for SU(3) links only, so they are refused while a U(1) field is
  * set; 8 is singular where |U00| = 1, so the link packing (on the first
  * operator call) fails with BQ_ERR_ARG if a link has |U01|^2 + |U02|^2 < 1e-6

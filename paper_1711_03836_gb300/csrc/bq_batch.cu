@@ -30,6 +30,7 @@
 
 #include "bq_ms.cuh"
 #include "bq_nvtx.cuh"
+#include "bq_split.cuh"
 
 struct BArgs {
     const SysVec *sys;
@@ -105,10 +106,33 @@ __global__ void __launch_bounds__(RED_THREADS) kb_init(BArgs ba, int use_t) {
     }
 }
 
-// p = rs + beta p
+// p = rs + beta p. FP32 and FP64 vectors of one storage are flat arrays of the same layout:
+// one 16-byte word at a time, so that a small lattice has 6 or 12 times the threads and every
+// thread one load of each vector in flight.
 template <int PS, int PR>
 __global__ void __launch_bounds__(RED_THREADS) kb_update_p(BArgs ba) {
     BATCH_PROLOGUE
+    if constexpr (PS == PR) {
+        const size_t n = (PS == BQ_PREC_DOUBLE ? 12 : 6) * (size_t)Vh;
+        if constexpr (PS == BQ_PREC_DOUBLE) {
+            const double beta = scal[S_BETA];
+            double2 *p = static_cast<double2 *>(sv.p);
+            const double2 *r = static_cast<const double2 *>(sv.rs);
+            for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+                const double2 a = p[i], b = r[i];
+                p[i] = make_double2(fma(beta, a.x, b.x), fma(beta, a.y, b.y));
+            }
+        } else {
+            const float beta = (float)scal[S_BETA];
+            float4 *p = static_cast<float4 *>(sv.p);
+            const float4 *r = static_cast<const float4 *>(sv.rs);
+            for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+                const float4 a = p[i], b = r[i];
+                p[i] = make_float4(fmaf(beta, a.x, b.x), fmaf(beta, a.y, b.y), fmaf(beta, a.z, b.z), fmaf(beta, a.w, b.w));
+            }
+        }
+        return;
+    }
     using TS = typename Traits<PS>::real;
     using TR = typename Traits<PR>::real;
     const TS beta = (TS)scal[S_BETA];
@@ -751,6 +775,8 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     int maxVh = 0;
     for (int i = 0; i < nsys; i++) maxVh = ctxs[i]->Vh > maxVh ? ctxs[i]->Vh : maxVh;
     const dim3 G(red_grid(maxVh), nsys);
+    // p update: 16-byte words of the vector per thread (FP16 p against FP32 r: sites), no limit from a reduction
+    const dim3 GP(PS == PR ? (unsigned)(((PS == BQ_PREC_DOUBLE ? 12LL : 6LL) * maxVh + RED_THREADS - 1) / RED_THREADS) : G.x, nsys);
 
     // device tables: per-system vectors and scalars (the launch tables stay on the host)
     std::vector<SysVec> hs(nsys);
@@ -783,12 +809,13 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     };
     const BArgs ba_act{w->d_sys, w->d_scal, w->d_part, w->d_ticket, d_active};
     const BArgs ba_upd{w->d_sys, w->d_scal, w->d_part, w->d_ticket, d_update};
-    // one system with an FP32 or FP16-storage inner iteration: the CG vector work rides on
-    // the two A x - k D launches
-    const bool fuse = nsys == 1 && PS != BQ_PREC_DOUBLE;
+    // one system with an FP32 or FP16-storage inner iteration, or a small lattice on the FP64 units:
+    // the CG vector work rides on the two A x - k D launches
+    const bool fuse = nsys == 1 && (PS != BQ_PREC_DOUBLE || bq_use_split(ctxs[0], PS));
     CgFuse cgf{};
     if (fuse) {
-        const size_t need = 2 * (size_t)((ctxs[0]->Vh + 127) / 128);  // two values per 128-site block
+        // two values per block of 128 sites, or of 16 on a small lattice
+        const size_t need = 2 * (size_t)(bq_use_split(ctxs[0], PS) ? bq_split_grid(ctxs[0]->Vh) : (ctxs[0]->Vh + 127) / 128);
         if (w->fpart_n < need) {
             cudaFree(w->d_fpart);
             w->d_fpart = nullptr;
@@ -797,7 +824,8 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
             w->fpart_n = need;
         }
         const double sigma0 = shifts ? shifts[0] : sp->shift;
-        cgf = CgFuse{w->slot[0].p, w->slot[0].xs, w->slot[0].rs, w->d_scal, w->d_fpart, sigma0 != 0.0};
+        cgf = CgFuse{w->slot[0].p, w->slot[0].xs, w->slot[0].rs, w->d_scal, w->d_fpart, sigma0 != 0.0,
+                     w->d_ticket};
     }
     // several FP32 / FP16 systems in the shared-memory tile mapping: the same fusion inside the tile kernel
     const bool fuse_tiles = nsys > 1 && PS != BQ_PREC_DOUBLE && mapping <= -3;
@@ -855,7 +883,7 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     int it = 0;
     // one iteration of the whole batch, queued on c0->stream
     auto body = [&](double frac) -> int {
-        kb_update_p<PS, PR><<<G, RED_THREADS, 0, c0->stream>>>(ba_act);
+        kb_update_p<PS, PR><<<GP, RED_THREADS, 0, c0->stream>>>(ba_act);
         BQ_COUNT(c0);
         if (fuse) {
             const DslashUnit *u[4];

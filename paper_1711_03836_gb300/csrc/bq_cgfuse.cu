@@ -13,6 +13,7 @@
 // and reload of Ap) for two one-block launches.
 #include "bq_cgfuse.cuh"
 #include "bq_reduce.cuh"
+#include "bq_split.cuh"
 #include "bq_stencil.cuh"
 
 namespace {
@@ -54,16 +55,8 @@ __global__ void __launch_bounds__(CG_FIN_THREADS) k_cg_finish(const double *part
         for (int k = 0; k < NV; k++) s[k] += partials[k * nw + i];
     block_sum(s);
     if (threadIdx.x == 0) {
-        if constexpr (MODE == CNT_CG_MHAT) {
-            const double pap = s[0] + scal[S_SIGMA] * s[1];
-            scal[S_PAP] = pap;
-            scal[S_ALPHA] = scal[S_RR] / pap;
-        } else {
-            const double rr = scal[S_RR];
-            scal[S_RRPREV] = rr;
-            scal[S_RR] = s[0];
-            scal[S_BETA] = s[0] / rr;
-        }
+        if constexpr (MODE == CNT_CG_MHAT) cg_set_alpha(scal, s[0], s[NV - 1]);
+        else cg_set_beta(scal, s[0]);
     }
 }
 
@@ -90,7 +83,7 @@ __global__ void __launch_bounds__(128, DslashMinBlocks<PS>::value) k_dslash_cg(c
             }
         }
         cplx<T> acc[12];
-        dslash_hops<PS, RECON, MODE == CNT_CG_MHATDAG>(a, a.in, h, acc);
+        dslash_hops<PS, RECON, MODE == CNT_CG_MHATDAG, false>(a, a.in, h, acc);
         if constexpr (MODE == CNT_CG_MHAT && PS == BQ_PREC_HALF) {
             // FP16 t: the site's scale needs all twelve components before the store
             cplx<T> xv[12], o[12];
@@ -216,8 +209,9 @@ void launch_cg_r(int recon, const DslashArgs &a, const CgFuse &f, int mode, unsi
 
 int bq_dslash_cg_launch(bq_ctx *c, int ps, void *out, const void *in, const void *xin, double k, int mode,
                         const CgFuse &f) {
-    if (!(ps == BQ_PREC_SINGLE || ps == BQ_PREC_HALF) || !(mode == CNT_CG_MHAT || mode == CNT_CG_MHATDAG)) {
-        bq_set_error("fused CG step: FP32 or FP16 inner precision only");
+    const bool split = bq_use_split(c, ps);
+    if (!(split || ps == BQ_PREC_SINGLE || ps == BQ_PREC_HALF) || !(mode == CNT_CG_MHAT || mode == CNT_CG_MHATDAG)) {
+        bq_set_error("fused CG step: FP32 or FP16 inner precision, or a small lattice on the FP64 units");
         return BQ_ERR_ARG;
     }
     const int dagger = mode == CNT_CG_MHATDAG;
@@ -227,18 +221,21 @@ int bq_dslash_cg_launch(bq_ctx *c, int ps, void *out, const void *in, const void
     a.in = in;
     a.xin = xin;
     const int recon = c->links_recon[ps];
-    const unsigned grid = (unsigned)((c->Vh + 127) / 128);
+    const unsigned grid = split ? bq_split_grid(c->Vh) : (unsigned)((c->Vh + 127) / 128);
     int slot;
     BQ_TRY(bq_time_begin(c, ps, mode, &slot));
-    if (ps == BQ_PREC_SINGLE) launch_cg_r<BQ_PREC_SINGLE>(recon, a, f, mode, grid, c->stream);
+    if (split) bq_split_launch(ps, recon, a, f, dagger, EPI_XPAY, mode, c->stream);
+    else if (ps == BQ_PREC_SINGLE) launch_cg_r<BQ_PREC_SINGLE>(recon, a, f, mode, grid, c->stream);
     else launch_cg_r<BQ_PREC_HALF>(recon, a, f, mode, grid, c->stream);
     BQ_LAUNCH_CHECK();
     BQ_TRY(bq_time_end(c, slot));
     BQ_COUNT(c);
-    launch_finish(f, mode, grid, c->stream);
-    BQ_LAUNCH_CHECK();
-    BQ_COUNT(c);
-    const double sr = spinor_bytes_per_site(BQ_PREC_SINGLE);
+    if (!split) {
+        launch_finish(f, mode, grid, c->stream);
+        BQ_LAUNCH_CHECK();
+        BQ_COUNT(c);
+    }
+    const double sr = spinor_bytes_per_site(ps == BQ_PREC_DOUBLE ? BQ_PREC_DOUBLE : BQ_PREC_SINGLE);
     c->counters.dslash_launches[ps][mode]++;
     c->counters.dslash_bytes[ps][mode] += dslash_site_bytes(ps, recon, EPI_XPAY) * c->Vh;
     c->counters.dslash_flops[ps][mode] += dslash_site_flops(EPI_XPAY) * c->Vh;

@@ -87,7 +87,7 @@ __device__ __forceinline__ df dshfl(df v) {
 
 // FMT: DF_IN_PAIR / DF_X_PAIR / DF_OUT_PAIR select float-pair storage for the
 // hopped spinor, the xpay spinor and the output (FP64 otherwise)
-template <int RECON, bool DAG, int EPI, int FMT, bool PREFETCH = true>
+template <bool DAG, int EPI, int FMT, bool PREFETCH = true>
 __device__ __forceinline__ void dslash_site_df64_pair(const DslashArgs &a, const void *in, void *out, const void *xin,
                                                       const int h, const int q, const bool valid) {
     using T = df;
@@ -138,7 +138,7 @@ __device__ __forceinline__ void dslash_site_df64_pair(const DslashArgs &a, const
             prefetch_l1(pp + (size_t)(3 * jq + c) * Vh);
         }
 #pragma unroll
-        for (int e = 0; e < (RECON == 12 ? 6 : 9); e++) prefetch_l1(pl + (size_t)e * Vh);
+        for (int e = 0; e < 9; e++) prefetch_l1(pl + (size_t)e * Vh);
     };
     if (PREFETCH) prefetch_hop(0);
 #pragma unroll 1
@@ -180,22 +180,19 @@ __device__ __forceinline__ void dslash_site_df64_pair(const DslashArgs &a, const
             cplx<T> pq, pj;
             if constexpr (FMT & DF_IN_PAIR) {
                 const float4 *pp = static_cast<const float4 *>(in);
-                const float4 vq = ldg(pp + (size_t)(3 * q + c) * Vh + hn), vj = ldg(pp + (size_t)(3 * jq + c) * Vh + hn);
+                const float4 vq = ldg<true>(pp + (size_t)(3 * q + c) * Vh + hn), vj = ldg<true>(pp + (size_t)(3 * jq + c) * Vh + hn);
                 pq = {T(vq.x, vq.y), T(vq.z, vq.w)};
                 pj = {T(vj.x, vj.y), T(vj.z, vj.w)};
             } else {
-                const double2 vq = ldg(pin + (size_t)(3 * q + c) * Vh + hn), vj = ldg(pin + (size_t)(3 * jq + c) * Vh + hn);
+                const double2 vq = ldg<true>(pin + (size_t)(3 * q + c) * Vh + hn), vj = ldg<true>(pin + (size_t)(3 * jq + c) * Vh + hn);
                 pq = {df_from_double(vq.x), df_from_double(vq.y)};
                 pj = {df_from_double(vj.x), df_from_double(vj.y)};
             }
             pj = mul_ipow(pj, kq);
             hq[c] = cadd_lazy2(pq, pj);
         }
-        // U h_q (or U^dag h_q): 18-real links one row (or column) at a time; 12-real
-        // links whole, the third row rebuilt
+        // U h_q (or U^dag h_q) one row (or column) of the link at a time
         const float4 *pu = reinterpret_cast<const float4 *>(lb) + hl;
-        cplx<T> Ufull[RECON == 12 ? 9 : 1];
-        if constexpr (RECON == 12) LinkIO<BQ_PREC_DF64, 12>::load(Ufull, lb, hl, Vh);
         cplx<T> u[3];
 #pragma unroll
         for (int aa = 0; aa < 3; aa++) {
@@ -203,12 +200,8 @@ __device__ __forceinline__ void dslash_site_df64_pair(const DslashArgs &a, const
 #pragma unroll
             for (int b = 0; b < 3; b++) {
                 const int e = back ? b * 3 + aa : aa * 3 + b;
-                if constexpr (RECON == 12) {
-                    w[b] = back ? cconj(Ufull[e]) : Ufull[e];
-                } else {
-                    const float4 v = ldg(pu + (size_t)e * Vh);
-                    w[b] = {df(v.x, v.y), back ? df(-v.z, -v.w) : df(v.z, v.w)};
-                }
+                const float4 v = ldg(pu + (size_t)e * Vh);
+                w[b] = {df(v.x, v.y), back ? df(-v.z, -v.w) : df(v.z, v.w)};
             }
             // (re, im) += (w.re, w.re) (h.re, h.im) + (-w.im, w.im) (h.im, h.re), in the
             // order of the scalar chains re = w.re h.re - w.im h.im, im = w.re h.im + w.im h.re
@@ -273,14 +266,14 @@ __device__ __forceinline__ void dslash_site_df64_pair(const DslashArgs &a, const
         const float4 *px = static_cast<const float4 *>(xin) + (size_t)(6 * q) * Vh + h;
 #pragma unroll
         for (int i = 0; i < 6; i++) {
-            const float4 v = ldg(px + (size_t)i * Vh);
+            const float4 v = ldg<true>(px + (size_t)i * Vh);
             xb[i] = {T(v.x, v.y), T(v.z, v.w)};
         }
     } else {
         const double2 *px = static_cast<const double2 *>(xin) + (size_t)(6 * q) * Vh + h;
 #pragma unroll
         for (int i = 0; i < 6; i++) {
-            const double2 v = ldg(px + (size_t)i * Vh);
+            const double2 v = ldg<true>(px + (size_t)i * Vh);
             xb[i] = {df_from_double(v.x), df_from_double(v.y)};
         }
     }
@@ -313,19 +306,21 @@ __device__ __forceinline__ void dslash_site_df64_pair(const DslashArgs &a, const
     }
 }
 
-template <int RECON, bool DAG, int EPI, int FMT>
+template <bool DAG, int EPI, int FMT>
 __global__ void __launch_bounds__(128, DF64P_MIN_BLOCKS) k_dslash_df64p(const DslashArgs a) {
+    bq_pdl_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int h = t >> 1;
     const bool valid = h < a.Vh;
-    dslash_site_df64_pair<RECON, DAG, EPI, FMT>(a, a.in, a.out, a.xin, valid ? h : a.Vh - 1, t & 1, valid);
+    dslash_site_df64_pair<DAG, EPI, FMT>(a, a.in, a.out, a.xin, valid ? h : a.Vh - 1, t & 1, valid);
 }
 
 // batched launch with a lane pair per site (interleave 5): block bl takes
 // right-hand side bl % nr and the 64 sites of site block bl / nr
-template <int RECON, bool DAG, int EPI, int FMT>
+template <bool DAG, int EPI, int FMT>
 __global__ void __launch_bounds__(128, DF64P_MIN_BLOCKS) k_dslash_batch_df64p(const __grid_constant__ DslashBatchTable tab,
                                                                               const double *mask) {
+    bq_pdl_enter();
     int u = 0;
     while (u + 1 < tab.nunits && tab.block0[u + 1] <= (int)blockIdx.x) u++;
     const DslashUnit &U = tab.units[u];
@@ -336,6 +331,6 @@ __global__ void __launch_bounds__(128, DF64P_MIN_BLOCKS) k_dslash_batch_df64p(co
     const bool valid = h < U.a.Vh;
     // no L1 prefetch here: with the unit indirection it costs registers (spills) and
     // measured slower (12-rhs batch, 24^3x48: 2.8 -> 3.1 ms per launch)
-    dslash_site_df64_pair<RECON, DAG, EPI, FMT, false>(U.a, U.in[r], U.out[r], U.xin[r], valid ? h : U.a.Vh - 1,
+    dslash_site_df64_pair<DAG, EPI, FMT, false>(U.a, U.in[r], U.out[r], U.xin[r], valid ? h : U.a.Vh - 1,
                                                 (int)(threadIdx.x & 1), valid);
 }

@@ -6,7 +6,7 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include "bq_internal.cuh"
+#include "bq_split.cuh"
 #include "bq_stencil.cuh"
 
 // Batched launch: the grid is cut into units (one lattice, up to DSLASH_UNIT_RHS
@@ -27,6 +27,7 @@ struct BatchMinBlocks {
 
 template <int PREC, int RECON, bool DAG, int EPI>
 __global__ void __launch_bounds__(128, BatchMinBlocks<PREC>::value) k_dslash_batch(const __grid_constant__ DslashBatchTable tab, const double *mask) {
+    bq_pdl_enter();
     int u = 0;
     while (u + 1 < tab.nunits && tab.block0[u + 1] <= (int)blockIdx.x) u++;
     const DslashUnit &U = tab.units[u];
@@ -77,13 +78,13 @@ double dslash_site_flops(int epi) { return 1320.0 + (epi != EPI_PLAIN ? 504.0 : 
 template <int PREC, int RECON>
 static void launch_dslash_pr(const DslashArgs &a, bool dag, int epi, unsigned grid, cudaStream_t s) {
     if (dag) {
-        if (epi == EPI_PLAIN) k_dslash<PREC, RECON, true, EPI_PLAIN><<<grid, 128, 0, s>>>(a);
-        else if (epi == EPI_CLOVINV) k_dslash<PREC, RECON, true, EPI_CLOVINV><<<grid, 128, 0, s>>>(a);
-        else k_dslash<PREC, RECON, true, EPI_XPAY><<<grid, 128, 0, s>>>(a);
+        if (epi == EPI_PLAIN) bq_launch(k_dslash<PREC, RECON, true, EPI_PLAIN>, grid, 128, s, a);
+        else if (epi == EPI_CLOVINV) bq_launch(k_dslash<PREC, RECON, true, EPI_CLOVINV>, grid, 128, s, a);
+        else bq_launch(k_dslash<PREC, RECON, true, EPI_XPAY>, grid, 128, s, a);
     } else {
-        if (epi == EPI_PLAIN) k_dslash<PREC, RECON, false, EPI_PLAIN><<<grid, 128, 0, s>>>(a);
-        else if (epi == EPI_CLOVINV) k_dslash<PREC, RECON, false, EPI_CLOVINV><<<grid, 128, 0, s>>>(a);
-        else k_dslash<PREC, RECON, false, EPI_XPAY><<<grid, 128, 0, s>>>(a);
+        if (epi == EPI_PLAIN) bq_launch(k_dslash<PREC, RECON, false, EPI_PLAIN>, grid, 128, s, a);
+        else if (epi == EPI_CLOVINV) bq_launch(k_dslash<PREC, RECON, false, EPI_CLOVINV>, grid, 128, s, a);
+        else bq_launch(k_dslash<PREC, RECON, false, EPI_XPAY>, grid, 128, s, a);
     }
 }
 
@@ -106,10 +107,11 @@ int bq_dslash_launch(bq_ctx *c, int prec, void *out, const void *in, int out_par
     int slot = -1;
     BQ_TRY(bq_time_begin(c, prec, epi, &slot));
     if (prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) {  // a lane pair per site (bq_df64.cu)
-        BQ_TRY(bq_df64p_launch(recon, a, dagger, epi, (unsigned)((2LL * c->Vh + 127) / 128), c->stream));
+        BQ_TRY(bq_df64p_launch(a, dagger, epi, (unsigned)((2LL * c->Vh + 127) / 128), c->stream));
+    } else if (bq_use_split(c, prec)) {
+        bq_split_launch(prec, recon, a, CgFuse{}, dagger, epi, 0, c->stream);
     } else if (prec == BQ_PREC_DOUBLE) {
-        if (recon == 12) launch_dslash_pr<BQ_PREC_DOUBLE, 12>(a, dagger, epi, grid, c->stream);
-        else launch_dslash_pr<BQ_PREC_DOUBLE, 18>(a, dagger, epi, grid, c->stream);
+        bq_pair64_launch(a, dagger, epi, c->stream);
     } else if (prec == BQ_PREC_SINGLE) {
         if (recon == 12) launch_dslash_pr<BQ_PREC_SINGLE, 12>(a, dagger, epi, grid, c->stream);
         else if (recon == 8) launch_dslash_pr<BQ_PREC_SINGLE, 8>(a, dagger, epi, grid, c->stream);
@@ -208,13 +210,13 @@ static void launch_batch_pr(const DslashBatchTable &tab, const double *mask, int
         return;
     }
     if (dag) {
-        if (epi == EPI_PLAIN) k_dslash_batch<PREC, RECON, true, EPI_PLAIN><<<nblocks, 128, 0, s>>>(tab, mask);
-        else if (epi == EPI_CLOVINV) k_dslash_batch<PREC, RECON, true, EPI_CLOVINV><<<nblocks, 128, 0, s>>>(tab, mask);
-        else k_dslash_batch<PREC, RECON, true, EPI_XPAY><<<nblocks, 128, 0, s>>>(tab, mask);
+        if (epi == EPI_PLAIN) bq_launch(k_dslash_batch<PREC, RECON, true, EPI_PLAIN>, nblocks, 128, s, tab, mask);
+        else if (epi == EPI_CLOVINV) bq_launch(k_dslash_batch<PREC, RECON, true, EPI_CLOVINV>, nblocks, 128, s, tab, mask);
+        else bq_launch(k_dslash_batch<PREC, RECON, true, EPI_XPAY>, nblocks, 128, s, tab, mask);
     } else {
-        if (epi == EPI_PLAIN) k_dslash_batch<PREC, RECON, false, EPI_PLAIN><<<nblocks, 128, 0, s>>>(tab, mask);
-        else if (epi == EPI_CLOVINV) k_dslash_batch<PREC, RECON, false, EPI_CLOVINV><<<nblocks, 128, 0, s>>>(tab, mask);
-        else k_dslash_batch<PREC, RECON, false, EPI_XPAY><<<nblocks, 128, 0, s>>>(tab, mask);
+        if (epi == EPI_PLAIN) bq_launch(k_dslash_batch<PREC, RECON, false, EPI_PLAIN>, nblocks, 128, s, tab, mask);
+        else if (epi == EPI_CLOVINV) bq_launch(k_dslash_batch<PREC, RECON, false, EPI_CLOVINV>, nblocks, 128, s, tab, mask);
+        else bq_launch(k_dslash_batch<PREC, RECON, false, EPI_XPAY>, nblocks, 128, s, tab, mask);
     }
 }
 
@@ -258,10 +260,9 @@ int bq_dslash_batch_launch(bq_ctx *c, int prec, int recon, const DslashBatchTabl
     BQ_TRY(bq_time_begin(c, prec, epi, &slot));
     cudaStream_t s = c->stream;
     if (prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) {  // lane pairs per site (bq_df64.cu)
-        BQ_TRY(bq_df64p_batch_launch(recon, *tab, mask, nblocks, dagger, epi, s));
+        BQ_TRY(bq_df64p_batch_launch(*tab, mask, nblocks, dagger, epi, s));
     } else if (prec == BQ_PREC_DOUBLE) {
-        if (recon == 12) launch_batch_pr<BQ_PREC_DOUBLE, 12>(*tab, mask, nblocks, dagger, epi, s);
-        else launch_batch_pr<BQ_PREC_DOUBLE, 18>(*tab, mask, nblocks, dagger, epi, s);
+        launch_batch_pr<BQ_PREC_DOUBLE, 18>(*tab, mask, nblocks, dagger, epi, s);
     } else if (prec == BQ_PREC_SINGLE) {
         if (recon == 12) launch_batch_pr<BQ_PREC_SINGLE, 12>(*tab, mask, nblocks, dagger, epi, s);
         else if (recon == 8) launch_batch_pr<BQ_PREC_SINGLE, 8>(*tab, mask, nblocks, dagger, epi, s);

@@ -17,6 +17,7 @@
 // errors
 
 static thread_local char g_err[512] = "";
+thread_local int bq_plain_next = 0;
 
 void bq_set_error(const char *fmt, ...) {
     va_list ap;
@@ -186,6 +187,7 @@ extern "C" int bq_set_recon(bq_ctx *c, int prec, int recon) {
     if (c->recon[prec] != recon) {
         c->recon[prec] = recon;
         c->links_valid[prec] = 0;
+        if (prec == BQ_PREC_DOUBLE) c->links_valid[BQ_PREC_DF64] = 0;
     }
     return BQ_OK;
 }
@@ -238,7 +240,10 @@ extern "C" int bq_set_u1(bq_ctx *c, const double *A, int where) {
 // --------------------------------------------------------------------------
 // links
 
-template <int PREC, int RECON>
+// REBUILD: 12-real FP64 links, third row = conj(row 0 x row 1), rebuilt here once and stored
+// (the FP64 kernels are bound by arithmetic: rebuilding it at every hop cost the double-float
+// kernel 40 % and the FP64-unit one 20 %)
+template <int PREC, int RECON, bool REBUILD = false>
 __global__ void k_pack_links(char *dst, size_t blk, const double2 *U, const double *A, double charge, Geo g,
                              int *flag) {
     long long lex = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -259,6 +264,12 @@ __global__ void k_pack_links(char *dst, size_t blk, const double2 *U, const doub
         // 8-real links are singular where |U00| = 1 (see reconstruct8)
         if (RECON == BQ_RECON_8 && u[1].x * u[1].x + u[1].y * u[1].y + u[2].x * u[2].x + u[2].y * u[2].y < BQ_RECON8_MIN_N)
             atomicExch(flag, 1);
+        if (REBUILD) {
+            cplx<double> w[9];
+            for (int k = 0; k < 6; k++) w[k] = {u[k].x, u[k].y};
+            reconstruct_row2(w);
+            for (int k = 6; k < 9; k++) u[k] = make_double2(w[k].re, w[k].im);
+        }
         LinkIO<PREC, RECON>::store(dst + (size_t)(par * 4 + mu) * blk, h, g.Vh, u);
     }
 }
@@ -268,9 +279,10 @@ int bq_prepare_links(bq_ctx *c, int prec) {
         bq_set_error("gauge field not set");
         return BQ_ERR_STATE;
     }
-    const int rp = (prec == BQ_PREC_DF64) ? BQ_PREC_DOUBLE : prec;  // df64 pairs follow the FP64 setting
-    if (c->links_valid[prec] && c->links_recon[prec] == c->recon[rp]) return BQ_OK;
-    int recon = c->recon[rp];
+    const bool fp64 = prec == BQ_PREC_DF64 || prec == BQ_PREC_DOUBLE;  // df64 pairs follow the FP64 setting
+    const int recon = fp64 ? BQ_RECON_18 : c->recon[prec];
+    if (c->links_valid[prec] && c->links_recon[prec] == recon) return BQ_OK;
+    const bool rebuild = fp64 && c->recon[BQ_PREC_DOUBLE] == BQ_RECON_12;
     size_t blk = link_bytes_per_link(prec, recon) * (size_t)c->Vh;
     if (c->links[prec] && c->links_recon[prec] != recon) {
         cudaFree(c->links[prec]);
@@ -288,17 +300,18 @@ int bq_prepare_links(bq_ctx *c, int prec) {
         Usrc = c->U_hop;
     }
     if (recon == BQ_RECON_8) BQ_CUDA_TRY(cudaMemsetAsync(c->dev_flag, 0, sizeof(int), c->stream));
-#define PACK(P, R) k_pack_links<P, R><<<grid, 128, 0, c->stream>>>(c->links[prec], blk, Usrc, c->A_u1, q, g, c->dev_flag)
+#define PACK(P, ...) k_pack_links<P, __VA_ARGS__><<<grid, 128, 0, c->stream>>>(c->links[prec], blk, Usrc, c->A_u1, q, g, c->dev_flag)
     if (prec == BQ_PREC_DOUBLE) {
-        if (recon == 12) PACK(BQ_PREC_DOUBLE, 12); else PACK(BQ_PREC_DOUBLE, 18);
+        if (rebuild) PACK(BQ_PREC_DOUBLE, 18, true); else PACK(BQ_PREC_DOUBLE, 18);
     } else if (prec == BQ_PREC_SINGLE) {
         if (recon == 12) PACK(BQ_PREC_SINGLE, 12); else if (recon == 8) PACK(BQ_PREC_SINGLE, 8); else PACK(BQ_PREC_SINGLE, 18);
     } else if (prec == BQ_PREC_HALF) {
         if (recon == 12) PACK(BQ_PREC_HALF, 12); else if (recon == 8) PACK(BQ_PREC_HALF, 8); else PACK(BQ_PREC_HALF, 18);
     } else {
-        if (recon == 12) PACK(BQ_PREC_DF64, 12); else PACK(BQ_PREC_DF64, 18);
+        if (rebuild) PACK(BQ_PREC_DF64, 18, true); else PACK(BQ_PREC_DF64, 18);
     }
 #undef PACK
+    bq_fields_written();
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
     if (recon == BQ_RECON_8) {
@@ -584,6 +597,7 @@ extern "C" int bq_build_clover(bq_ctx *c) {
     BQ_COUNT(c);
     k_invert_clover<<<grid_for(4LL * c->Vh, 64), 64, 0, c->stream>>>((double2 *)c->clov_master, pblk, c->Vh,
                                                                      c->dev_flag);
+    bq_fields_written();
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
     int flag = 0;
@@ -675,6 +689,7 @@ extern "C" int bq_set_clover(bq_ctx *c, const double *A, int where) {
         bq_set_error("bq_set_clover: a clover block of the field has no inverse");
         return BQ_ERR_CLOVER_SINGULAR;
     }
+    bq_fields_written();
     c->clov_user = 1;
     c->clov_master_valid = 1;
     c->clov[BQ_PREC_DOUBLE] = (char *)c->clov_master;
@@ -694,6 +709,7 @@ int bq_prepare_clover(bq_ctx *c, int prec) {
         k_convert_clover<BQ_PREC_DF64><<<grid, 128, 0, c->stream>>>(c->clov[prec], (const double2 *)c->clov_master, c->Vh, 4);
     else
         k_convert_clover<BQ_PREC_HALF><<<grid, 128, 0, c->stream>>>(c->clov[prec], (const double2 *)c->clov_master, c->Vh, 4);
+    bq_fields_written();
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
     c->clov_valid[prec] = 1;

@@ -31,6 +31,32 @@ void bq_set_error(const char *fmt, ...);
         if (s_ != BQ_OK) return s_; \
     } while (0)
 
+// Launch with programmatic dependence on the stream's previous kernel: the grid is set up
+// while that kernel drains and waits inside bq_pdl_enter(), which every kernel launched here
+// calls first. In a stream this takes 2.3 us off each launch (Mhat^dag Mhat in FP32: 8^4
+// 24.6 -> 15.4 us, 20^3x40 112.6 -> 102.7 us); inside a captured graph 0.2 us. The kernels do
+// not ask for an earlier start (griddepcontrol.launch_dependents): blocks that then wait on
+// the SMs of the running kernel leave an uneven distribution behind (FP64, 12^4: 158 -> 307 us).
+// Fields written by a kernel that was not launched this way (link and clover packing) are read
+// through the read-only path, so the first launch after one is a plain one:
+// bq_fields_written() asks for that.
+extern thread_local int bq_plain_next;
+inline void bq_fields_written() { bq_plain_next = 1; }
+template <typename... P, typename... A>
+inline void bq_launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = bq_plain_next ? 0 : 1;
+    bq_plain_next = 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // the caller reads cudaGetLastError()
+}
+
 #define BQ_LAUNCH_CHECK() BQ_CUDA_TRY(cudaGetLastError())
 
 // --------------------------------------------------------------------------
@@ -156,8 +182,8 @@ struct DslashBatchTable {
 int bq_dslash_launch(bq_ctx *c, int prec, void *out, const void *in, int out_parity, int dagger, int epi,
                      const void *xin, double k, int fmt = 0);
 // double-float lane-pair kernels (bq_df64.cu); BQ_ERR_ARG for a storage combination without a kernel
-int bq_df64p_launch(int recon, const DslashArgs &a, bool dag, int epi, unsigned grid, cudaStream_t s);
-int bq_df64p_batch_launch(int recon, const DslashBatchTable &tab, const double *mask, int nblocks, bool dag, int epi,
+int bq_df64p_launch(const DslashArgs &a, bool dag, int epi, unsigned grid, cudaStream_t s);
+int bq_df64p_batch_launch(const DslashBatchTable &tab, const double *mask, int nblocks, bool dag, int epi,
                           cudaStream_t s);
 int bq_clover_launch(bq_ctx *c, int prec, void *out, const void *in, int parity, int inverse);
 int bq_mhat_launch(bq_ctx *c, int prec, void *out, const void *in, int dagger, void *tmp_odd);
@@ -204,6 +230,7 @@ struct CgFuse {
     double *scal;
     double *partials;
     int with_pnorm;  // sum |p|^2 too (the shift is nonzero)
+    unsigned int *ticket;  // small lattices (bq_split.cu): the launch's last block sums the partials
 };
 // mode CNT_CG_MHAT: out = t = A_ee p - k D_eo in (xin = p), then <p, Ap> = |t|^2 + sigma |p|^2
 //   and alpha = rr / <p, Ap>; mode CNT_CG_MHATDAG: q = A_ee^dag xin - k D_eo^dag in + sigma p

@@ -83,6 +83,20 @@ __device__ __forceinline__ double norm2_site(const cplx<T> s[12]) {
     return (double)a;
 }
 
+// the scalars of a CG step: alpha = rr / <p, Ap> with <p, Ap> = |Mhat p|^2 + sigma |p|^2 ...
+__device__ __forceinline__ void cg_set_alpha(double *scal, double tt, double pp) {
+    const double pap = tt + scal[S_SIGMA] * pp;
+    scal[S_PAP] = pap;
+    scal[S_ALPHA] = scal[S_RR] / pap;
+}
+// ... and rr, beta from the new |r|^2
+__device__ __forceinline__ void cg_set_beta(double *scal, double rr_new) {
+    const double rr = scal[S_RR];
+    scal[S_RRPREV] = rr;
+    scal[S_RR] = rr_new;
+    scal[S_BETA] = rr_new / rr;
+}
+
 struct RedArgs {
     double *partials;
     unsigned int *ticket;

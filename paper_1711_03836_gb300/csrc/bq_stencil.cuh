@@ -95,7 +95,7 @@ __device__ __forceinline__ void accumulate_scaled(cplx<T> acc[12], const cplx<T>
     }
 }
 
-template <int PREC, int RECON, int MU, int S, bool BACK, bool SCALE>
+template <int PREC, int RECON, int MU, int S, bool BACK, bool SCALE, bool FRESH>
 __device__ __forceinline__ void hop(cplx<typename Traits<PREC>::real> acc[12], const void *in, int hn,
                                     const char *lblk, int hl, int Vh, typename Traits<PREC>::real coef) {
     using T = typename Traits<PREC>::real;
@@ -106,10 +106,10 @@ __device__ __forceinline__ void hop(cplx<typename Traits<PREC>::real> acc[12], c
     T f = SCALE ? coef : T(1);
     if constexpr (PREC == BQ_PREC_HALF) {
         T n;
-        SpinorIO<PREC>::load_unscaled(psi, in, hn, Vh, n);
+        SpinorIO<PREC>::template load_unscaled<FRESH>(psi, in, hn, Vh, n);
         f *= n;
     } else {
-        SpinorIO<PREC>::load(psi, in, hn, Vh);
+        SpinorIO<PREC>::template load<FRESH>(psi, in, hn, Vh);
     }
     cplx<T> h0[3], h1[3];
     project<MU, S>(psi, h0, h1);
@@ -137,8 +137,8 @@ __device__ __forceinline__ void hop(cplx<typename Traits<PREC>::real> acc[12], c
         accumulate<MU, S>(acc, u0, u1);
 }
 
-// acc = D_hop in at output site h (the eight hops, Eq. 1 / Eq. 5)
-template <int PREC, int RECON, bool DAG>
+// acc = D_hop in at output site h (the eight hops, Eq. 1 / Eq. 5); FRESH: see ldg
+template <int PREC, int RECON, bool DAG, bool FRESH>
 __device__ __forceinline__ void dslash_hops(const DslashArgs &a, const void *in, const int h,
                                             cplx<typename Traits<PREC>::real> acc[12]) {
     using T = typename Traits<PREC>::real;
@@ -161,40 +161,40 @@ __device__ __forceinline__ void dslash_hops(const DslashArgs &a, const void *in,
 
     {
         const int xn = (x + 1 == a.L0) ? 0 : x + 1;
-        hop<PREC, RECON, 0, SF, false, false>(acc, in, h - xh + (xn >> 1), Lo, h, Vh, T(1));
+        hop<PREC, RECON, 0, SF, false, false, FRESH>(acc, in, h - xh + (xn >> 1), Lo, h, Vh, T(1));
     }
     {
         const int xn = (x == 0) ? a.L0 - 1 : x - 1;
         const int hn = h - xh + (xn >> 1);
-        hop<PREC, RECON, 0, SB, true, false>(acc, in, hn, Li, hn, Vh, T(1));
+        hop<PREC, RECON, 0, SB, true, false, FRESH>(acc, in, hn, Li, hn, Vh, T(1));
     }
     {
         const int hn = (y + 1 == a.L1) ? h - (a.L1 - 1) * sy : h + sy;
-        hop<PREC, RECON, 1, SF, false, false>(acc, in, hn, Lo + a.lblk, h, Vh, T(1));
+        hop<PREC, RECON, 1, SF, false, false, FRESH>(acc, in, hn, Lo + a.lblk, h, Vh, T(1));
     }
     {
         const int hn = (y == 0) ? h + (a.L1 - 1) * sy : h - sy;
-        hop<PREC, RECON, 1, SB, true, false>(acc, in, hn, Li + a.lblk, hn, Vh, T(1));
+        hop<PREC, RECON, 1, SB, true, false, FRESH>(acc, in, hn, Li + a.lblk, hn, Vh, T(1));
     }
     {
         const int hn = (z + 1 == a.L2) ? h - (a.L2 - 1) * sz : h + sz;
-        hop<PREC, RECON, 2, SF, false, false>(acc, in, hn, Lo + 2 * a.lblk, h, Vh, T(1));
+        hop<PREC, RECON, 2, SF, false, false, FRESH>(acc, in, hn, Lo + 2 * a.lblk, h, Vh, T(1));
     }
     {
         const int hn = (z == 0) ? h + (a.L2 - 1) * sz : h - sz;
-        hop<PREC, RECON, 2, SB, true, false>(acc, in, hn, Li + 2 * a.lblk, hn, Vh, T(1));
+        hop<PREC, RECON, 2, SB, true, false, FRESH>(acc, in, hn, Li + 2 * a.lblk, hn, Vh, T(1));
     }
     {
         const bool wrap = (t + 1 == a.L3);
         const int hn = wrap ? h - (a.L3 - 1) * st : h + st;
         const T coef = (T)(wrap ? a.cf * a.bc : a.cf);
-        hop<PREC, RECON, 3, SF, false, true>(acc, in, hn, Lo + 3 * a.lblk, h, Vh, coef);
+        hop<PREC, RECON, 3, SF, false, true, FRESH>(acc, in, hn, Lo + 3 * a.lblk, h, Vh, coef);
     }
     {
         const bool wrap = (t == 0);
         const int hn = wrap ? h + (a.L3 - 1) * st : h - st;
         const T coef = (T)(wrap ? a.cb * a.bc : a.cb);
-        hop<PREC, RECON, 3, SB, true, true>(acc, in, hn, Li + 3 * a.lblk, hn, Vh, coef);
+        hop<PREC, RECON, 3, SB, true, true, FRESH>(acc, in, hn, Li + 3 * a.lblk, hn, Vh, coef);
     }
 }
 
@@ -205,7 +205,7 @@ __device__ __forceinline__ void xpay_site(const DslashArgs &a, const void *xin, 
                                           cplx<typename Traits<PREC>::real> xv[12],
                                           cplx<typename Traits<PREC>::real> o[12]) {
     using T = typename Traits<PREC>::real;
-    SpinorIO<PREC>::load(xv, xin, h, a.Vh);
+    SpinorIO<PREC>::template load<true>(xv, xin, h, a.Vh);
     clover_apply_site<PREC>(o, xv, a.clov, h, a.Vh);
     const T k = (T)a.k;
 #pragma unroll
@@ -221,7 +221,7 @@ __device__ __forceinline__ void dslash_site(const DslashArgs &a, const void *in,
     using T = typename Traits<PREC>::real;
     const int Vh = a.Vh;
     cplx<T> acc[12];
-    dslash_hops<PREC, RECON, DAG>(a, in, h, acc);
+    dslash_hops<PREC, RECON, DAG, true>(a, in, h, acc);
     if (EPI == EPI_PLAIN) {
         SpinorIO<PREC>::store(out, h, Vh, acc);
     } else if (EPI == EPI_CLOVINV) {
@@ -266,6 +266,7 @@ struct DslashMinBlocks<BQ_PREC_DOUBLE> {  // FP64-unit bound: no cap
 };
 template <int PREC, int RECON, bool DAG, int EPI>
 __global__ void __launch_bounds__(128, DslashMinBlocks<PREC>::value) k_dslash(const DslashArgs a) {
+    bq_pdl_enter();
     const int h = blockIdx.x * blockDim.x + threadIdx.x;
     if (h >= a.Vh) return;
     dslash_any<PREC, RECON, DAG, EPI>(a, a.in, a.out, a.xin, h);

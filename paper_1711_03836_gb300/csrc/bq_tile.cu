@@ -52,7 +52,7 @@ __device__ __forceinline__ SiteNb site_neighbours(const DslashArgs &a, int h) {
 // one hop with the link already in registers (FP32 arithmetic; FP16 spinors
 // are projected and multiplied unscaled, the site's scale folded into the
 // accumulation as in hop())
-template <int PREC, int MU, int S, bool BACK, bool SCALE>
+template <int PREC, int MU, int S, bool BACK, bool SCALE, bool FRESH>
 __device__ __forceinline__ void hop_link(cplx<float> acc[12], const void *in, int hn, const cplx<float> U[9], int Vh,
                                          float coef) {
     constexpr bool FOLD = SCALE || PREC == BQ_PREC_HALF;
@@ -60,10 +60,10 @@ __device__ __forceinline__ void hop_link(cplx<float> acc[12], const void *in, in
     float f = SCALE ? coef : 1.0f;
     if constexpr (PREC == BQ_PREC_HALF) {
         float n;
-        SpinorIO<PREC>::load_unscaled(psi, in, hn, Vh, n);
+        SpinorIO<PREC>::template load_unscaled<FRESH>(psi, in, hn, Vh, n);
         f *= n;
     } else {
-        SpinorIO<PREC>::load(psi, in, hn, Vh);
+        SpinorIO<PREC>::template load<FRESH>(psi, in, hn, Vh);
     }
     cplx<float> h0[3], h1[3];
     project<MU, S>(psi, h0, h1);
@@ -213,23 +213,23 @@ __device__ __forceinline__ void dslash_site_tile(const DslashArgs &a, const Site
     for (int c = 0; c < 12; c++) acc[c] = {0.f, 0.f};
     cplx<float> U[9];
     tile_link(U, sL, 0, lane);
-    hop_link<PREC, 0, SF, false, false>(acc, in, nb.hn[0], U, Vh, 1.f);
+    hop_link<PREC, 0, SF, false, false, CGM == 0>(acc, in, nb.hn[0], U, Vh, 1.f);
     tile_link(U, sL, 1, lane);
-    hop_link<PREC, 0, SB, true, false>(acc, in, nb.hn[1], U, Vh, 1.f);
+    hop_link<PREC, 0, SB, true, false, CGM == 0>(acc, in, nb.hn[1], U, Vh, 1.f);
     tile_link(U, sL, 2, lane);
-    hop_link<PREC, 1, SF, false, false>(acc, in, nb.hn[2], U, Vh, 1.f);
+    hop_link<PREC, 1, SF, false, false, CGM == 0>(acc, in, nb.hn[2], U, Vh, 1.f);
     tile_link(U, sL, 3, lane);
-    hop_link<PREC, 1, SB, true, false>(acc, in, nb.hn[3], U, Vh, 1.f);
+    hop_link<PREC, 1, SB, true, false, CGM == 0>(acc, in, nb.hn[3], U, Vh, 1.f);
     tile_link(U, sL, 4, lane);
-    hop_link<PREC, 2, SF, false, false>(acc, in, nb.hn[4], U, Vh, 1.f);
+    hop_link<PREC, 2, SF, false, false, CGM == 0>(acc, in, nb.hn[4], U, Vh, 1.f);
     tile_link(U, sL, 5, lane);
-    hop_link<PREC, 2, SB, true, false>(acc, in, nb.hn[5], U, Vh, 1.f);
+    hop_link<PREC, 2, SB, true, false, CGM == 0>(acc, in, nb.hn[5], U, Vh, 1.f);
     const float cf = (float)(nb.t + 1 == a.L3 ? a.cf * a.bc : a.cf);
     const float cb = (float)(nb.t == 0 ? a.cb * a.bc : a.cb);
     tile_link(U, sL, 6, lane);
-    hop_link<PREC, 3, SF, false, true>(acc, in, nb.hn[6], U, Vh, cf);
+    hop_link<PREC, 3, SF, false, true, CGM == 0>(acc, in, nb.hn[6], U, Vh, cf);
     tile_link(U, sL, 7, lane);
-    hop_link<PREC, 3, SB, true, true>(acc, in, nb.hn[7], U, Vh, cb);
+    hop_link<PREC, 3, SB, true, true, CGM == 0>(acc, in, nb.hn[7], U, Vh, cb);
 
     if (EPI == EPI_PLAIN) {
         SpinorIO<PREC>::store(out, h, Vh, acc);
@@ -333,7 +333,7 @@ __device__ __forceinline__ void dslash_site_tile(const DslashArgs &a, const Site
 #pragma unroll
         for (int c = 0; c < 12; c++) src[c] = acc[c];
     } else {
-        SpinorIO<PREC>::load(src, xin, h, Vh);
+        SpinorIO<PREC>::template load<CGM == 0>(src, xin, h, Vh);
     }
 #pragma unroll
     for (int b = 0; b < 2; b++) {
@@ -368,6 +368,7 @@ __device__ __forceinline__ void dslash_site_tile(const DslashArgs &a, const Site
 template <int PREC, int RECON, bool DAG, int EPI, int MB, int CGM = 0>
 __global__ void __launch_bounds__(128, MB) k_dslash_tile(const __grid_constant__ DslashBatchTable tab,
                                                          const double *mask, const TileCg cg) {
+    bq_pdl_enter();
     __shared__ float4 sL[8 * 5 * TILE_SITES];
     __shared__ float4 sC[EPI != EPI_PLAIN ? 18 * TILE_SITES : 1];
     int u = 0;
@@ -414,11 +415,11 @@ static void launch_tile_mb(const DslashBatchTable &tab, const double *mask, int 
                            cudaStream_t s) {
     const TileCg none{};
     if (dag) {
-        if (epi == EPI_CLOVINV) k_dslash_tile<PREC, RECON, true, EPI_CLOVINV, MB><<<nblocks, 128, 0, s>>>(tab, mask, none);
-        else k_dslash_tile<PREC, RECON, true, EPI_XPAY, MB><<<nblocks, 128, 0, s>>>(tab, mask, none);
+        if (epi == EPI_CLOVINV) bq_launch(k_dslash_tile<PREC, RECON, true, EPI_CLOVINV, MB>, nblocks, 128, s, tab, mask, none);
+        else bq_launch(k_dslash_tile<PREC, RECON, true, EPI_XPAY, MB>, nblocks, 128, s, tab, mask, none);
     } else {
-        if (epi == EPI_CLOVINV) k_dslash_tile<PREC, RECON, false, EPI_CLOVINV, MB><<<nblocks, 128, 0, s>>>(tab, mask, none);
-        else k_dslash_tile<PREC, RECON, false, EPI_XPAY, MB><<<nblocks, 128, 0, s>>>(tab, mask, none);
+        if (epi == EPI_CLOVINV) bq_launch(k_dslash_tile<PREC, RECON, false, EPI_CLOVINV, MB>, nblocks, 128, s, tab, mask, none);
+        else bq_launch(k_dslash_tile<PREC, RECON, false, EPI_XPAY, MB>, nblocks, 128, s, tab, mask, none);
     }
 }
 
@@ -520,16 +521,8 @@ __global__ void __launch_bounds__(CG_FIN_BATCH_THREADS) k_cg_finish_batch(const 
     block_sum(s);
     if (threadIdx.x == 0) {
         double *scal = scal_all + (size_t)sy * S_NSCAL;
-        if constexpr (MODE == CNT_CG_MHAT) {
-            const double pap = s[0] + scal[S_SIGMA] * s[1];
-            scal[S_PAP] = pap;
-            scal[S_ALPHA] = scal[S_RR] / pap;
-        } else {
-            const double rr = scal[S_RR];
-            scal[S_RRPREV] = rr;
-            scal[S_RR] = s[0];
-            scal[S_BETA] = s[0] / rr;
-        }
+        if constexpr (MODE == CNT_CG_MHAT) cg_set_alpha(scal, s[0], s[NV - 1]);
+        else cg_set_beta(scal, s[0]);
     }
 }
 
