@@ -4,7 +4,7 @@
 // eight hops in a rolled loop, and the site split over a pair of lanes.
 #pragma once
 
-#include "bq_device.cuh"
+#include "bq_pairs.cuh"
 
 // --------------------------------------------------------------------------
 // The direction-dependent projector as data: (1 + S gamma_mu) psi has upper
@@ -38,33 +38,6 @@ __device__ __forceinline__ cplx<df> mul_ipow(cplx<df> z, int k) {
 // (spins 0, 1), lane 1 block 1 (spins 2, 3), and each applies its clover block
 // and stores its six components. Half the live state of a one-lane site, so
 // about twice the resident warps to hide the dependent double-float chains.
-
-// Lazy double-float sums of products on (real, imaginary) pairs with the packed
-// FP32 instructions of the sm_100 family (one instruction for both lanes): lane x
-// and lane y take exactly the operations of two scalar dfsum chains.
-struct dfsum2 {
-    float2 s, c;
-};
-__device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ dfsum2 dfs2_prod(float2 ah, float2 al, float2 bh, float2 bl) {
-    const float2 p = __fmul2_rn(ah, bh);
-    float2 e = __ffma2_rn(ah, bh, f2neg(p));
-    e = __ffma2_rn(ah, bl, e);
-    e = __ffma2_rn(al, bh, e);
-    return {p, e};
-}
-__device__ __forceinline__ void dfs2_add_prod(dfsum2 &z, float2 ah, float2 al, float2 bh, float2 bl) {
-    const float2 p = __fmul2_rn(ah, bh);
-    float2 e = __ffma2_rn(ah, bh, f2neg(p));
-    e = __ffma2_rn(ah, bl, e);
-    e = __ffma2_rn(al, bh, e);
-    // two-sum of z.s and p
-    const float2 t = __fadd2_rn(z.s, p);
-    const float2 bb = __fadd2_rn(t, f2neg(z.s));
-    const float2 te = __fadd2_rn(__fadd2_rn(z.s, f2neg(__fadd2_rn(t, f2neg(bb)))), __fadd2_rn(p, f2neg(bb)));
-    z.s = t;
-    z.c = __fadd2_rn(z.c, __fadd2_rn(e, te));
-}
 
 // a + b for complex double-float values without the final normalisation (add_lazy
 // on the real and the imaginary part as one pair)

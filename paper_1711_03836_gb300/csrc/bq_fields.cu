@@ -1,6 +1,6 @@
 // bq_fields.cu -- context, field upload and derived-field preparation.
 //
-//  * links: canonical FP64 U[V][4][3][3] -> native per-precision layout, with
+//  * links: the caller's FP64 U[V][4][3][3] -> [4][9][V] -> native per-precision layout, with
 //    the QCD+QED phase e^{-i Q A_mu(x)} of Eq. 5 folded into U_mu(x);
 //  * clover: A(x) = 1 + i kappa c_SW sum_{mu<nu} sigma_{mu nu} F_{mu nu}(x) of Eq. 2,
 //    built on the GPU in FP64 from the four plaquette leaves, written as two
@@ -126,6 +126,7 @@ extern "C" int bq_destroy(bq_ctx *c) {
     bq_full_free(c);
     cudaFree(c->U_canon);
     cudaFree(c->U_hop);
+    cudaFree(c->U_pair);
     cudaFree(c->A_u1);
     for (int p = 0; p < BQ_NFIELD; p++) {
         cudaFree(c->links[p]);
@@ -192,15 +193,85 @@ extern "C" int bq_set_recon(bq_ctx *c, int prec, int recon) {
     return BQ_OK;
 }
 
+// Links between the caller's layout [V][4][9] and the library's [4][9][V]: a block takes 32 sites
+// through shared memory, so that both sides are read and written along consecutive addresses.
+#define LINK_SITES 32
+template <bool IN>
+__global__ void __launch_bounds__(256) k_links_layout(double2 *dst, const double2 *src, long long V) {
+    __shared__ double2 sm[LINK_SITES][37];  // 37: the columns start in different banks
+    const long long x0 = (long long)blockIdx.x * LINK_SITES;
+    const int n = V - x0 < LINK_SITES ? (int)(V - x0) : LINK_SITES;
+    if (IN) {
+        for (int i = threadIdx.x; i < 36 * n; i += 256) sm[i / 36][i % 36] = src[x0 * 36 + i];
+    } else {
+        for (int i = threadIdx.x; i < 36 * LINK_SITES; i += 256)
+            if (i % LINK_SITES < n) sm[i % LINK_SITES][i / LINK_SITES] = src[(i / LINK_SITES) * V + x0 + i % LINK_SITES];
+    }
+    __syncthreads();
+    if (IN) {
+        for (int i = threadIdx.x; i < 36 * LINK_SITES; i += 256)
+            if (i % LINK_SITES < n) dst[(i / LINK_SITES) * V + x0 + i % LINK_SITES] = sm[i % LINK_SITES][i / LINK_SITES];
+    } else {
+        for (int i = threadIdx.x; i < 36 * n; i += 256) dst[x0 * 36 + i] = sm[i / 36][i % 36];
+    }
+}
+
+// every link entry split into float pairs (re.hi, im.hi, re.lo, im.lo), exactly but for the last
+// five bits of the low part; normalised, so that the products of two low parts which the sums
+// leave out are below 2^-50 of a term and of either sign (the truncating split alone leaves
+// 2^-48, all of one sign)
+__global__ void __launch_bounds__(256) k_split_links(float4 *dst, const double2 *src, long long n) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    const double2 v = src[i];
+    const df a = normalise(df_from_double(v.x)), b = normalise(df_from_double(v.y));
+    dst[i] = make_float4(a.hi, b.hi, a.lo, b.lo);
+}
+
+static size_t link_field_bytes(const bq_ctx *c) { return (size_t)c->V * 36 * sizeof(double2); }
+
+int bq_split_links(bq_ctx *c, const double2 *U, int thin) {
+    if (thin && c->U_pair_thin) return BQ_OK;
+    BQ_TRY(bq_alloc((void **)&c->U_pair, link_field_bytes(c)));
+    k_split_links<<<grid_for(36 * c->V, 256), 256, 0, c->stream>>>(c->U_pair, U, 36 * c->V);
+    BQ_LAUNCH_CHECK();
+    BQ_COUNT(c);
+    c->U_pair_thin = thin;
+    return BQ_OK;
+}
+
+int bq_links_out(bq_ctx *c, double *dst, const double2 *U, int where) {
+    double2 *to = (double2 *)dst;
+    if (where == BQ_HOST) {
+        BQ_TRY(bq_alloc((void **)&c->U_pair, link_field_bytes(c)));
+        c->U_pair_thin = 0;
+        to = (double2 *)c->U_pair;
+    }
+    k_links_layout<false><<<grid_for(c->V, LINK_SITES), 256, 0, c->stream>>>(to, U, c->V);
+    BQ_LAUNCH_CHECK();
+    BQ_COUNT(c);
+    if (where == BQ_HOST)
+        BQ_CUDA_TRY(cudaMemcpyAsync(dst, to, link_field_bytes(c), cudaMemcpyDeviceToHost, c->stream));
+    BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
+    return BQ_OK;
+}
+
 extern "C" int bq_set_gauge(bq_ctx *c, const double *U, int where) {
     if (!c || !U || !(where == BQ_HOST || where == BQ_DEVICE)) {
         bq_set_error("bq_set_gauge: bad arguments");
         return BQ_ERR_ARG;
     }
-    size_t bytes = (size_t)c->V * 4 * 9 * sizeof(double2);
-    BQ_TRY(bq_alloc((void **)&c->U_canon, bytes));
-    BQ_CUDA_TRY(cudaMemcpyAsync(c->U_canon, U, bytes,
-                                where == BQ_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream));
+    BQ_TRY(bq_alloc((void **)&c->U_canon, link_field_bytes(c)));
+    const double2 *src = (const double2 *)U;
+    c->U_pair_thin = 0;
+    if (where == BQ_HOST) {
+        BQ_TRY(bq_alloc((void **)&c->U_pair, link_field_bytes(c)));
+        BQ_CUDA_TRY(cudaMemcpyAsync(c->U_pair, U, link_field_bytes(c), cudaMemcpyHostToDevice, c->stream));
+        src = (const double2 *)c->U_pair;
+    }
+    k_links_layout<true><<<grid_for(c->V, LINK_SITES), 256, 0, c->stream>>>(c->U_canon, src, c->V);
+    BQ_LAUNCH_CHECK();
+    BQ_COUNT(c);
     if (where == BQ_HOST) BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
     c->have_gauge = 1;
     invalidate_derived(c, 1, 1);
@@ -254,8 +325,8 @@ __global__ void k_pack_links(char *dst, size_t blk, const double2 *U, const doub
     int h = (int)(lex >> 1);
     for (int mu = 0; mu < 4; mu++) {
         double2 u[9];
-        const double2 *src = U + (lex * 4 + mu) * 9;
-        for (int k = 0; k < 9; k++) u[k] = src[k];
+        const double2 *src = U + (long long)mu * 9 * g.V + lex;
+        for (int k = 0; k < 9; k++) u[k] = src[k * g.V];
         if (A) {
             double s, co;
             sincos(-charge * A[lex * 4 + mu], &s, &co);
@@ -331,44 +402,58 @@ int bq_prepare_links(bq_ctx *c, int prec) {
 // --------------------------------------------------------------------------
 // clover term
 
-// traceless anti-Hermitian part of the clover-leaf sum in the mu-nu plane: (Q - Q^dag)/8 - trace/3
-__device__ void field_strength(const double2 *U, const Geo &g, long long x, int mu, int nu, M3 &F) {
-    long long xpm = lex_step(g, x, mu, +1), xpn = lex_step(g, x, nu, +1);
-    long long xmm = lex_step(g, x, mu, -1), xmn = lex_step(g, x, nu, -1);
-    long long xmm_pn = lex_step(g, xmm, nu, +1), xmm_mn = lex_step(g, xmm, nu, -1);
-    long long xmn_pm = lex_step(g, xmn, mu, +1);
-    // the four leaves as paths of four links each (site, direction, daggered):
-    //   x -> x+mu -> x+mu+nu -> x+nu -> x,   x -> x+nu -> x+nu-mu -> x-mu -> x,
-    //   x -> x-mu -> x-mu-nu -> x-nu -> x,   x -> x-nu -> x-nu+mu -> x+mu -> x
-    const long long site[16] = {x, xpm, xpn, x, x, xmm_pn, xmm, xmm, xmm, xmm_mn, xmm_mn, xmn, xmn, xmn, xmn_pm, x};
-    const unsigned dir_nu = 0x5a5au;  // bit j: link j points along nu (else mu)
-    const unsigned dag = 0x936cu;     // bit j: link j enters daggered
-    // each leaf multiplied out left to right in double-float (one partial
-    // product and one link live), rounded to FP64 and summed there; the loops
-    // stay rolled so that the sixteen link loads are not all hoisted at once
-    M3 Q;
-    for (int k = 0; k < 9; k++) Q.a[k] = {0.0, 0.0};
+// F_{mu nu}(x) = (Q - Q^dag)/8 - trace/3, Q the sum of the four leaves. With n = U_nu, m = U_mu the
+// leaves pair up around the two links m(x) and m(x - mu): the sum enters only through Q - Q^dag, so
+// a leaf may be replaced by minus its adjoint, and
+//   Q - Q^dag = R - R^dag,  R = [n(x) m(x-mu+nu)^d n(x-mu)^d - n(x-nu)^d m(x-mu-nu)^d n(x-mu-nu)] m(x-mu)
+//                             - [n(x) m(x+nu) n(x+mu)^d - n(x-nu)^d m(x-nu) n(x+mu-nu)] m(x)^d:
+// ten products instead of twelve. The loop stays rolled (one partial product, one link and the
+// bracket live, one copy of the product's code). The nine independent reals of F: the imaginary
+// parts of the diagonal, then the three entries above it.
+__device__ __forceinline__ void field_strength(const float4 *P, const Geo &g, long long x, int mu, int nu, double F[9]) {
+    const long long V = g.V;
+    const long long xpm = lex_step(g, x, mu, +1), xpn = lex_step(g, x, nu, +1);
+    const long long xmm = lex_step(g, x, mu, -1), xmn = lex_step(g, x, nu, -1);
+    const long long xmm_pn = lex_step(g, xmm, nu, +1), xmm_mn = lex_step(g, xmm, nu, -1);
+    const long long xmn_pm = lex_step(g, xmn, mu, +1);
+    M3p R, D;
 #pragma unroll 1
-    for (int l = 0; l < 4; l++) {
-        M3d P = load_link_df(U, site[4 * l], (dir_nu >> (4 * l)) & 1 ? nu : mu);
-        if ((dag >> (4 * l)) & 1) P = mdag_df(P);
+    for (int half = 0; half < 2; half++) {
+        M3p A;
 #pragma unroll 1
-        for (int j = 4 * l + 1; j < 4 * l + 4; j++) {
-            const M3d L = load_link_df(U, site[j], (dir_nu >> j) & 1 ? nu : mu);
-            P = (dag >> j) & 1 ? mmul_df(P, mdag_df(L)) : mmul_df(P, L);
+        for (int st = 0; st < 5; st++) {
+            if (st == 0) A = load_link_pair(P, V, x, nu, false);
+            if (st == 2) {
+                D = A;
+                A = load_link_pair(P, V, xmn, nu, true);
+            }
+            if (st == 4) madd_pair(A, D, -1.0f);
+            // the step's link: m, n of the first path, m, n of the second, the m they share
+            const long long s = half == 0 ? (st == 0 ? xpn : st == 1 ? xpm : st == 2 ? xmn : st == 3 ? xmn_pm : x)
+                                          : (st == 0 ? xmm_pn : st == 1 ? xmm : st < 4 ? xmm_mn : xmm);
+            const int d = (st == 1 || st == 3) ? nu : mu;
+            const bool dag = st == 1 || (half == 0 ? st == 4 : (st == 0 || st == 2));
+            mmul_pair(A, load_link_pair(P, V, s, d, dag));
         }
-        for (int k = 0; k < 9; k++)
-            Q.a[k] = cadd(Q.a[k], cplx<double>{df_to_double(P.a[k].re), df_to_double(P.a[k].im)});
+        if (half == 0) R = A;
+        else madd_pair(R, A, -1.0f);
     }
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) {
-            cplx<double> q = Q.a[i * 3 + j], qt = cconj(Q.a[j * 3 + i]);
-            F.a[i * 3 + j] = cscale(0.125, csub(q, qt));
-        }
-    cplx<double> tr = cscale(1.0 / 3.0, cadd(cadd(F.a[0], F.a[4]), F.a[8]));
-    F.a[0] = csub(F.a[0], tr);
-    F.a[4] = csub(F.a[4], tr);
-    F.a[8] = csub(F.a[8], tr);
+    // (R - R^dag) / 8: reals of the diagonal drop out
+    double im[3];
+#pragma unroll
+    for (int i = 0; i < 3; i++) im[i] = 0.25 * ((double)R.hi[4 * i].y + (double)R.lo[4 * i].y);
+    const double tr = (im[0] + im[1] + im[2]) * (1.0 / 3.0);
+#pragma unroll
+    for (int i = 0; i < 3; i++) F[i] = im[i] - tr;
+#pragma unroll
+    for (int e = 0; e < 3; e++) {
+        const int i = e < 2 ? 0 : 1, j = e == 0 ? 1 : 2;
+        const float2 bh = R.hi[j * 3 + i], bl = R.lo[j * 3 + i];
+        const dfsum2 t = two_sum2(R.hi[i * 3 + j], make_float2(-bh.x, bh.y));
+        const float2 l = __fadd2_rn(t.c, __fadd2_rn(R.lo[i * 3 + j], make_float2(-bl.x, bl.y)));
+        F[3 + 2 * e] = 0.125 * ((double)t.s.x + (double)l.x);
+        F[4 + 2 * e] = 0.125 * ((double)t.s.y + (double)l.y);
+    }
 }
 
 // A(x) per site. In the chiral basis sigma_{mu nu} is block diagonal; with
@@ -379,18 +464,22 @@ __device__ void field_strength(const double2 *U, const Geo &g, long long x, int 
 // of its 32 sites into shared memory, then two threads per site (one per
 // chirality block) assemble and store the blocks.
 #define CLOVER_SITES 32
-__global__ void __launch_bounds__(6 * CLOVER_SITES) k_build_clover(double2 *master, size_t pblk, const double2 *U,
-                                                                   Geo g, double kc) {
+#ifndef CLOVER_MIN_BLOCKS
+#define CLOVER_MIN_BLOCKS 2
+#endif
+__global__ void __launch_bounds__(6 * CLOVER_SITES, CLOVER_MIN_BLOCKS) k_build_clover(double2 *master, size_t pblk,
+                                                                                      const float4 *P, Geo g, double kc) {
     // planes: 0:(0,1) 1:(0,2) 2:(0,3) 3:(1,2) 4:(1,3) 5:(2,3)
-    __shared__ double2 sF[6][9][CLOVER_SITES];
+    __shared__ double sF[6][9][CLOVER_SITES];
     const int lane = threadIdx.x % CLOVER_SITES, pl = threadIdx.x / CLOVER_SITES;
     const long long x0 = (long long)blockIdx.x * CLOVER_SITES;
     if (x0 + lane < g.V) {
         const int mu = pl < 3 ? 0 : (pl < 5 ? 1 : 2);
         const int nu = pl < 3 ? pl + 1 : (pl < 5 ? pl - 1 : 3);
-        M3 F;
-        field_strength(U, g, x0 + lane, mu, nu, F);
-        for (int k = 0; k < 9; k++) sF[pl][k][lane] = make_double2(F.a[k].re, F.a[k].im);
+        double F[9];
+        field_strength(P, g, x0 + lane, mu, nu, F);
+#pragma unroll
+        for (int k = 0; k < 9; k++) sF[pl][k][lane] = F[k];
     }
     __syncthreads();
     if (threadIdx.x >= 2 * CLOVER_SITES) return;
@@ -401,22 +490,38 @@ __global__ void __launch_bounds__(6 * CLOVER_SITES) k_build_clover(double2 *mast
     lex_coords(g, x, c);
     const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
     const int h = (int)(x >> 1);
-    const double sg = b == 0 ? 1.0 : -1.0;
+    const double sg = b == 0 ? kc : -kc;
+    // kc E1, kc E2, kc E3 (anti-Hermitian, nine reals each): E1 = +-F14 - F23, E2 = +-F24 + F13, E3 = +-F34 - F12
+    double e1[9], e2[9], e3[9];
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        e1[k] = fma(sg, sF[2][k][lane], -kc * sF[3][k][lane]);
+        e2[k] = fma(sg, sF[4][k][lane], kc * sF[1][k][lane]);
+        e3[k] = fma(sg, sF[5][k][lane], -kc * sF[0][k][lane]);
+    }
     cplx<double> B[36];
-    for (int a = 0; a < 3; a++)
-        for (int bb = 0; bb < 3; bb++) {
-            const int k = a * 3 + bb;
-            const double2 f12 = sF[0][k][lane], f13 = sF[1][k][lane], f14 = sF[2][k][lane];
-            const double2 f23 = sF[3][k][lane], f24 = sF[4][k][lane], f34 = sF[5][k][lane];
-            const cplx<double> e1 = {sg * f14.x - f23.x, sg * f14.y - f23.y};  // +-F14 - F23
-            const cplx<double> e2 = {sg * f24.x + f13.x, sg * f24.y + f13.y};  // +-F24 + F13
-            const cplx<double> e3 = {sg * f34.x - f12.x, sg * f34.y - f12.y};  // +-F34 - F12
-            const double d = (a == bb) ? 1.0 : 0.0;
-            // i kc E3, i kc (E1 - i E2) = i kc E1 + kc E2, i kc (E1 + i E2) = i kc E1 - kc E2, -i kc E3
-            B[(0 + a) * 6 + (0 + bb)] = {d - kc * e3.im, kc * e3.re};
-            B[(0 + a) * 6 + (3 + bb)] = {-kc * e1.im + kc * e2.re, kc * e1.re + kc * e2.im};
-            B[(3 + a) * 6 + (0 + bb)] = {-kc * e1.im - kc * e2.re, kc * e1.re - kc * e2.im};
-            B[(3 + a) * 6 + (3 + bb)] = {d + kc * e3.im, -kc * e3.re};
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            cplx<double> f1, f2, f3;  // entry (i, j) of each
+            if (i == j) {
+                f1 = {0.0, e1[i]};
+                f2 = {0.0, e2[i]};
+                f3 = {0.0, e3[i]};
+            } else {
+                const int r = i < j ? i : j, k = 3 + 2 * (r == 1 ? 2 : (i + j - 1));
+                const double s = i < j ? 1.0 : -1.0;  // F_ji = -conj(F_ij)
+                f1 = {s * e1[k], e1[k + 1]};
+                f2 = {s * e2[k], e2[k + 1]};
+                f3 = {s * e3[k], e3[k + 1]};
+            }
+            const double d = (i == j) ? 1.0 : 0.0;
+            // i E3, i (E1 - i E2) = i E1 + E2, i (E1 + i E2) = i E1 - E2, -i E3
+            B[(0 + i) * 6 + (0 + j)] = {d - f3.im, f3.re};
+            B[(0 + i) * 6 + (3 + j)] = {f2.re - f1.im, f1.re + f2.im};
+            B[(3 + i) * 6 + (0 + j)] = {-f1.im - f2.re, f1.re - f2.im};
+            B[(3 + i) * 6 + (3 + j)] = {d + f3.im, -f3.re};
         }
     store_herm6(master + (size_t)(par * 2 + 0) * pblk, b, h, g.Vh, B);
 }
@@ -473,7 +578,9 @@ __device__ __noinline__ bool invert6_pivoted(const double2 *src, double2 *dst, i
 // taken when every |d_j| is at least 0.1 of the block's largest entry (all
 // blocks of smooth and moderately rough fields). Otherwise Gauss-Jordan with
 // partial pivoting; a block whose pivot falls below 1e-13 of its largest entry
-// is reported as singular.
+// is reported as singular. Bound by the FP64 pipe: about 450 FP64 instructions per block,
+// 0.95 ms of the 1.08 ms at 24^3x48 (1.97 ms with hypot for the largest entry, products
+// added after rounding, and D^-1 applied inside every sum).
 __global__ void k_invert_clover(double2 *master, size_t pblk, int Vh, int *flag) {
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= 4 * Vh) return;
@@ -484,33 +591,8 @@ __global__ void k_invert_clover(double2 *master, size_t pblk, int Vh, int *flag)
     double2 *dst = master + (size_t)(par * 2 + 1) * pblk;
     cplx<double> B[36];
     load_herm6(src, b, h, Vh, B);
-    double scale = 0.0;
-    for (int k = 0; k < 36; k++) scale = fmax(scale, hypot(B[k].re, B[k].im));
-    // L D L^dag; W_ik = L_ik d_k. The loops run over fixed trip counts with
-    // guards, so that they unroll completely and every array stays in registers.
-    cplx<double> L[36], W[36];
-    double dinv[6];
-    bool fast = true;
-#pragma unroll
-    for (int j = 0; j < 6; j++) {
-        double dj = B[j * 7].re;
-#pragma unroll
-        for (int k = 0; k < 6; k++)
-            if (k < j) dj -= W[j * 6 + k].re * L[j * 6 + k].re + W[j * 6 + k].im * L[j * 6 + k].im;
-        fast = fast && fabs(dj) >= 0.1 * scale;
-        dinv[j] = 1.0 / dj;
-#pragma unroll
-        for (int i = 0; i < 6; i++)
-            if (i > j) {
-                cplx<double> t = B[i * 6 + j];
-#pragma unroll
-                for (int k = 0; k < 6; k++)
-                    if (k < j) t = csub(t, cmul(W[i * 6 + k], cconj(L[j * 6 + k])));
-                W[i * 6 + j] = t;
-                L[i * 6 + j] = cscale(dinv[j], t);
-            }
-    }
-    if (!fast) {
+    Ldl6 f;
+    if (!f.factor(B)) {
         if (!invert6_pivoted(src, dst, b, h, Vh)) atomicExch(flag, 1);
         return;
     }
@@ -521,23 +603,28 @@ __global__ void k_invert_clover(double2 *master, size_t pblk, int Vh, int *flag)
 #pragma unroll
         for (int i = 0; i < 6; i++)
             if (i > j) {
-                cplx<double> t = cscale(-1.0, L[i * 6 + j]);
+                cplx<double> t = {-f.L[i * 6 + j].re, -f.L[i * 6 + j].im};
 #pragma unroll
                 for (int k = 0; k < 6; k++)
-                    if (k > j && k < i) t = csub(t, cmul(L[i * 6 + k], X[k * 6 + j]));
+                    if (k > j && k < i) t = cfnma(f.L[i * 6 + k], X[k * 6 + j], t);
                 X[i * 6 + j] = t;
             }
-    // (A^-1)_ij = sum_{k >= max(i,j)} conj(X_ki) X_kj / d_k (X_kk = 1), upper triangle and diagonal
+    // (A^-1)_ij = sum_{k >= max(i,j)} conj(X_ki) Y_kj, Y = D^-1 X (X_kk = 1), upper triangle and
+    // (real) diagonal; row k of Y is formed once for all the sums it enters
     cplx<double> Binv[36];
 #pragma unroll
     for (int i = 0; i < 6; i++)
 #pragma unroll
         for (int j = 0; j < 6; j++)
             if (j >= i) {
-                cplx<double> t = i == j ? cplx<double>{dinv[j], 0.0} : cscale(dinv[j], cconj(X[j * 6 + i]));
+                cplx<double> t = i == j ? cplx<double>{f.dinv[j], 0.0} : cscale(f.dinv[j], cconj(X[j * 6 + i]));
 #pragma unroll
                 for (int k = 0; k < 6; k++)
-                    if (k > j) t = cadd(t, cscale(dinv[k], cmul(cconj(X[k * 6 + i]), X[k * 6 + j])));
+                    if (k > j) {
+                        const cplx<double> yk = cscale(f.dinv[k], X[k * 6 + j]);
+                        if (i == j) t.re = fma(X[k * 6 + i].re, yk.re, fma(X[k * 6 + i].im, yk.im, t.re));
+                        else t = cfmac(X[k * 6 + i], yk, t);
+                    }
                 Binv[i * 6 + j] = t;
             }
     // the inverse of a Hermitian matrix is Hermitian: keep the diagonal's real part and the upper triangle
@@ -591,7 +678,8 @@ extern "C" int bq_build_clover(bq_ctx *c) {
     Geo g = geo_of(c);
     BQ_CUDA_TRY(cudaMemsetAsync(c->dev_flag, 0, sizeof(int), c->stream));
     const unsigned nblk = (unsigned)((c->V + CLOVER_SITES - 1) / CLOVER_SITES);
-    k_build_clover<<<nblk, 6 * CLOVER_SITES, 0, c->stream>>>((double2 *)c->clov_master, pblk, c->U_canon, g,
+    BQ_TRY(bq_split_links(c, c->U_canon, 1));
+    k_build_clover<<<nblk, 6 * CLOVER_SITES, 0, c->stream>>>((double2 *)c->clov_master, pblk, c->U_pair, g,
                                                              c->params.kappa * c->params.csw);
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);

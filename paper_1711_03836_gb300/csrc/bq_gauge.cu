@@ -87,63 +87,149 @@ __device__ M3 expm_su3_ch(const M3 &X) {
     return E;
 }
 
-// one stout step for every link: C = rho sum_{nu != mu} (upper + lower staple)
-// (staple products in double-float, the rest in FP64),
+// f_j of exp(iQ) = f0 + f1 Q + f2 Q^2 by the Taylor series to order N: every power of Q is
+// a + b Q + c Q^2 by the Cayley-Hamilton theorem (Q^3 = c1 Q + c0), with real a, b, c of two
+// operations per order. Truncation below 1e-17 for eigenvalues up to 0.2 (N = 11) or 1 (N = 18).
+template <int N>
+__device__ __forceinline__ void exp_coefficients(double c0, double c1, cplx<double> f[3]) {
+    double a = 0.0, b = 0.0, c = 1.0;  // Q^2
+    f[0] = {1.0, 0.0};
+    f[1] = {0.0, 1.0};
+    f[2] = {-0.5, 0.0};
+    double inv = 0.5;
+#pragma unroll
+    for (int n = 3; n <= N; n++) {
+        const double a1 = c * c0, b1 = n == 3 ? c1 : fma(c, c1, a);  // times Q
+        c = b;
+        a = a1;
+        b = b1;
+        inv *= 1.0 / n;
+        const double s = (n & 2) ? -inv : inv;  // i^n / n!
+        if (n & 1) {
+            f[0].im = fma(s, a, f[0].im);
+            f[1].im = fma(s, b, f[1].im);
+            f[2].im = fma(s, c, f[2].im);
+        } else {
+            f[0].re = fma(s, a, f[0].re);
+            f[1].re = fma(s, b, f[1].re);
+            f[2].re = fma(s, c, f[2].re);
+        }
+    }
+}
+
+// exp(X) of a traceless anti-Hermitian X given by its nine reals (imaginary parts of the diagonal,
+// the entries 01, 02, 12): the series for eigenvalues up to 1 (2 sqrt(c1 / 3) bounds them), the
+// closed form beyond
+__device__ __forceinline__ M3 exp_antiherm(const double q[3], const cplx<double> x[3]) {
+    // Q = -iX: diagonal q, off-diagonal -i x
+    const cplx<double> q01 = {x[0].im, -x[0].re}, q02 = {x[1].im, -x[1].re}, q12 = {x[2].im, -x[2].re};
+    const double n01 = fma(q01.re, q01.re, q01.im * q01.im), n02 = fma(q02.re, q02.re, q02.im * q02.im),
+                 n12 = fma(q12.re, q12.re, q12.im * q12.im);
+    const double c1 = fma(0.5, fma(q[0], q[0], fma(q[1], q[1], q[2] * q[2])), n01 + n02 + n12);
+    if (!(c1 <= 0.75)) {
+        M3 X;
+        for (int k = 0; k < 3; k++) X.a[4 * k] = {0.0, q[k]};
+        for (int e = 0; e < 3; e++) {
+            const int i = e < 2 ? 0 : 1, j = e == 0 ? 1 : 2;
+            X.a[i * 3 + j] = x[e];
+            X.a[j * 3 + i] = {-x[e].re, x[e].im};
+        }
+        return expm_su3_ch(X);
+    }
+    // c0 = det Q
+    const cplx<double> t = cmul(q01, q12);
+    const double c0 = q[0] * fma(q[1], q[2], -n12) - fma(q[2], n01, q[1] * n02) +
+                      2.0 * fma(t.re, q02.re, t.im * q02.im);
+    cplx<double> f[3];
+    if (c1 <= 0.03) exp_coefficients<11>(c0, c1, f);
+    else exp_coefficients<18>(c0, c1, f);
+    // Q^2: diagonal, then 01 = q01 (q0 + q1) + q02 conj(q12), 02 = q02 (q0 + q2) + q01 q12,
+    // 12 = q12 (q1 + q2) + conj(q01) q02
+    const double s0 = fma(q[0], q[0], n01 + n02), s1 = fma(q[1], q[1], n01 + n12), s2 = fma(q[2], q[2], n02 + n12);
+    const cplx<double> z01 = cfmac(q12, q02, cscale(q[0] + q[1], q01));
+    const cplx<double> z02 = cfma(q01, q12, cscale(q[0] + q[2], q02));
+    const cplx<double> z12 = cfmac(q01, q02, cscale(q[1] + q[2], q12));
+    M3 E;
+    E.a[0] = {fma(f[2].re, s0, fma(f[1].re, q[0], f[0].re)), fma(f[2].im, s0, fma(f[1].im, q[0], f[0].im))};
+    E.a[4] = {fma(f[2].re, s1, fma(f[1].re, q[1], f[0].re)), fma(f[2].im, s1, fma(f[1].im, q[1], f[0].im))};
+    E.a[8] = {fma(f[2].re, s2, fma(f[1].re, q[2], f[0].re)), fma(f[2].im, s2, fma(f[1].im, q[2], f[0].im))};
+    E.a[1] = cfma(f[2], z01, cmul(f[1], q01));
+    E.a[2] = cfma(f[2], z02, cmul(f[1], q02));
+    E.a[5] = cfma(f[2], z12, cmul(f[1], q12));
+    E.a[3] = cfma(f[2], cconj(z01), cmul(f[1], cconj(q01)));
+    E.a[6] = cfma(f[2], cconj(z02), cmul(f[1], cconj(q02)));
+    E.a[7] = cfma(f[2], cconj(z12), cmul(f[1], cconj(q12)));
+    return E;
+}
+
+// one stout step for every link: C = rho sum_{nu != mu} (upper + lower staple) in double-float,
 // Omega = C U^dag, X = traceless anti-Hermitian part of Omega
 // (= i Q with Q = (i/2)(Omega^dag - Omega) - (i/6) tr(Omega^dag - Omega)),
-// U' = exp(X) U. Links are periodic in every direction.
-// three resident 128-thread blocks per SM (168 registers, no spills with the
-// staples in a rolled loop): 18 ms per step at 32^3x64; 24 ms with the staples
-// unrolled (144 bytes of spills), 30 ms at one or two blocks (255 registers)
+// U' = exp(X) U in FP64. Links are periodic in every direction. A block of four warps takes 32
+// consecutive sites, warp mu their links U_mu. Bound by the FP64 pipe and the packed FP32 products
+// together: about 430 FP64 instructions per link (Omega 90, series and Q^2 140, exp(X) 60, times
+// U 108) are 1.9 ms of the 2.45 ms at 24^3x48; three blocks per SM (168 registers).
 #ifndef STOUT_MIN_BLOCKS
 #define STOUT_MIN_BLOCKS 3
 #endif
-__global__ void __launch_bounds__(128, STOUT_MIN_BLOCKS) k_stout_step(double2 *out, const double2 *in, Geo g,
-                                                                      double rho) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= g.V * 4) return;
-    const long long x = idx >> 2;
-    const int mu = (int)(idx & 3);
-    const long long xpm = lex_step(g, x, mu, +1);
-    M3d Cd;
-    for (int k = 0; k < 9; k++) Cd.a[k] = {df(0.0f, 0.0f), df(0.0f, 0.0f)};
-    // the six staples as three-link paths, multiplied out left to right (one
-    // partial product and one link live); the loops stay rolled so that the
-    // eighteen link loads are not all hoisted at once
+__global__ void __launch_bounds__(128, STOUT_MIN_BLOCKS) k_stout_step(double2 *out, const double2 *in, const float4 *P,
+                                                                      Geo g, double rho) {
+    const long long x = (long long)blockIdx.x * 32 + (threadIdx.x & 31);
+    const int mu = threadIdx.x >> 5;
+    if (x >= g.V) return;
+    const long long V = g.V, xpm = lex_step(g, x, mu, +1);
+    M3p Cd;
+#pragma unroll
+    for (int k = 0; k < 9; k++) Cd.hi[k] = Cd.lo[k] = make_float2(0.f, 0.f);
+    // the six staples as three-link paths, multiplied out left to right; one copy of the
+    // product's code, one partial product and one link live
 #pragma unroll 1
     for (int st = 0; st < 6; st++) {
         const int nu = (st >> 1) + ((st >> 1) >= mu ? 1 : 0);  // the three directions other than mu
         const bool lower = st & 1;
         const long long xmn = lex_step(g, x, nu, -1);
         // upper: U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag; lower: U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)
-        const long long s0 = lower ? xmn : x;
         const long long s1 = lower ? xmn : lex_step(g, x, nu, +1);
         const long long s2 = lower ? lex_step(g, xmn, mu, +1) : xpm;
-        M3d P = load_link_df(in, s0, nu);
-        if (lower) P = mdag_df(P);
-        P = mmul_df(P, load_link_df(in, s1, mu));
-        const M3d L = load_link_df(in, s2, nu);
-        P = lower ? mmul_df(P, L) : mmul_df(P, mdag_df(L));
-        for (int k = 0; k < 9; k++) {
-            Cd.a[k].re = add_lazy(Cd.a[k].re, P.a[k].re);
-            Cd.a[k].im = add_lazy(Cd.a[k].im, P.a[k].im);
+        M3p A = load_link_pair(P, V, lower ? xmn : x, nu, lower);
+#pragma unroll 1
+        for (int j = 0; j < 2; j++) mmul_pair(A, load_link_pair(P, V, j ? s2 : s1, j ? nu : mu, j && !lower));
+        madd_pair(Cd, A, 1.0f);
+    }
+    // Omega = C U^dag; X from its anti-Hermitian part (diagonal: imaginary parts only)
+    const M3 U = load_link(in, V, x, mu);
+    double q[3];
+    cplx<double> xo[3];
+    {
+        M3 C;
+#pragma unroll
+        for (int k = 0; k < 9; k++)
+            C.a[k] = {(double)Cd.hi[k].x + (double)Cd.lo[k].x, (double)Cd.hi[k].y + (double)Cd.lo[k].y};
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            double s = 0.0;  // Im sum_k C_ik conj(U_ik)
+#pragma unroll
+            for (int k = 0; k < 3; k++) s = fma(C.a[i * 3 + k].im, U.a[i * 3 + k].re, fma(-C.a[i * 3 + k].re, U.a[i * 3 + k].im, s));
+            q[i] = rho * s;
+        }
+        const double tr = (q[0] + q[1] + q[2]) * (1.0 / 3.0);
+#pragma unroll
+        for (int i = 0; i < 3; i++) q[i] -= tr;
+#pragma unroll
+        for (int e = 0; e < 3; e++) {
+            const int i = e < 2 ? 0 : 1, j = e == 0 ? 1 : 2;
+            cplx<double> o = {0.0, 0.0}, p = {0.0, 0.0};  // Omega_ij, Omega_ji
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                o = cfmac(U.a[j * 3 + k], C.a[i * 3 + k], o);
+                p = cfmac(U.a[i * 3 + k], C.a[j * 3 + k], p);
+            }
+            xo[e] = {0.5 * rho * (o.re - p.re), 0.5 * rho * (o.im + p.im)};
         }
     }
-    M3 C;
-    for (int k = 0; k < 9; k++) C.a[k] = {df_to_double(normalise(Cd.a[k].re)), df_to_double(normalise(Cd.a[k].im))};
-    const M3 U = load_link(in, x, mu);
-    M3 Om = mmul(C, mdag(U));
-    M3 X;
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++)
-            X.a[i * 3 + j] = cscale(0.5 * rho, csub(Om.a[i * 3 + j], cconj(Om.a[j * 3 + i])));
-    const cplx<double> tr = cscale(1.0 / 3.0, cadd(cadd(X.a[0], X.a[4]), X.a[8]));
-    X.a[0] = csub(X.a[0], tr);
-    X.a[4] = csub(X.a[4], tr);
-    X.a[8] = csub(X.a[8], tr);
-    const M3 Un = mmul(expm_su3_ch(X), U);
-    double2 *p = out + (x * 4 + mu) * 9;
-    for (int k = 0; k < 9; k++) p[k] = make_double2(Un.a[k].re, Un.a[k].im);
+    const M3 Un = mmul(exp_antiherm(q, xo), U);
+    double2 *p = out + (long long)mu * 9 * V + x;
+    for (int k = 0; k < 9; k++) p[k * V] = make_double2(Un.a[k].re, Un.a[k].im);
 }
 
 int bq_prepare_hop_links(bq_ctx *c) {
@@ -154,13 +240,15 @@ int bq_prepare_hop_links(bq_ctx *c) {
     double2 *tmp = nullptr;
     if (c->stout_iter > 1) BQ_TRY(bq_alloc((void **)&tmp, bytes));
     const Geo g = geo_of(c);
-    const unsigned grid = grid_for(c->V * 4, 128);
+    const unsigned grid = grid_for(c->V, 32);
     // ping-pong so that the last step writes U_hop
     const double2 *src = c->U_canon;
     int status = BQ_OK;
     for (int it = 0; it < c->stout_iter; it++) {
         double2 *dst = ((c->stout_iter - 1 - it) % 2 == 0) ? c->U_hop : tmp;
-        k_stout_step<<<grid, 128, 0, c->stream>>>(dst, src, g, c->stout_rho);
+        status = bq_split_links(c, src, it == 0);
+        if (status != BQ_OK) break;
+        k_stout_step<<<grid, 128, 0, c->stream>>>(dst, src, c->U_pair, g, c->stout_rho);
         if (cudaGetLastError() != cudaSuccess) {
             bq_set_error("stout smearing launch failed");
             status = BQ_ERR_CUDA;
@@ -206,10 +294,7 @@ extern "C" int bq_get_hop_links(bq_ctx *c, double *U, int where) {
         BQ_TRY(bq_prepare_hop_links(c));
         src = c->U_hop;
     }
-    BQ_CUDA_TRY(cudaMemcpyAsync(U, src, (size_t)c->V * 4 * 9 * sizeof(double2),
-                                where == BQ_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, c->stream));
-    BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    return BQ_OK;
+    return bq_links_out(c, U, src, where);
 }
 
 // --------------------------------------------------------------------------
@@ -272,31 +357,11 @@ __global__ void __launch_bounds__(RED_THREADS) k_clover_logdet(const double2 *bl
         const int h = idx % Vh, b = idx / Vh;
         cplx<double> B[36];
         load_herm6(blk, b, h, Vh, B);
-        double scale = 0.0;
-        for (int k = 0; k < 36; k++) scale = fmax(scale, hypot(B[k].re, B[k].im));
-        cplx<double> L[36], W[36];  // W_ik = L_ik d_k
+        Ldl6 f;
+        const bool fast = f.factor(B);
         double det = 1.0;
-        bool fast = true;
 #pragma unroll
-        for (int j = 0; j < 6; j++) {
-            double dj = B[j * 7].re;
-#pragma unroll
-            for (int k = 0; k < 6; k++)
-                if (k < j) dj -= W[j * 6 + k].re * L[j * 6 + k].re + W[j * 6 + k].im * L[j * 6 + k].im;
-            fast = fast && fabs(dj) >= 0.1 * scale;
-            det *= dj;
-            const double dinv = 1.0 / dj;
-#pragma unroll
-            for (int i = 0; i < 6; i++)
-                if (i > j) {
-                    cplx<double> t = B[i * 6 + j];
-#pragma unroll
-                    for (int k = 0; k < 6; k++)
-                        if (k < j) t = csub(t, cmul(W[i * 6 + k], cconj(L[j * 6 + k])));
-                    W[i * 6 + j] = t;
-                    L[i * 6 + j] = cscale(dinv, t);
-                }
-        }
+        for (int j = 0; j < 6; j++) det *= f.d[j];
         bool neg;
         double la;
         if (fast) {

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "bq_internal.cuh"
+#include "bq_pairs.cuh"
 
 struct Geo {
     int L0, L1, L2, L3;
@@ -39,16 +40,15 @@ struct M3 {
     cplx<double> a[9];
 };
 
-__device__ __forceinline__ M3 load_link(const double2 *U, long long lex, int mu) {
+// gauge links inside the library: element k of U_mu(lex) at (mu * 9 + k) * V + lex, so that the
+// threads of a warp (consecutive sites) read consecutive addresses
+__device__ __forceinline__ M3 load_link(const double2 *U, long long V, long long lex, int mu) {
     M3 m;
-    const double2 *p = U + (lex * 4 + mu) * 9;
-    for (int k = 0; k < 9; k++) m.a[k] = {p[k].x, p[k].y};
-    return m;
-}
-__device__ __forceinline__ M3 mdag(const M3 &x) {
-    M3 m;
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) m.a[i * 3 + j] = cconj(x.a[j * 3 + i]);
+    const double2 *p = U + (long long)mu * 9 * V + lex;
+    for (int k = 0; k < 9; k++) {
+        const double2 v = p[k * V];
+        m.a[k] = {v.x, v.y};
+    }
     return m;
 }
 __device__ __forceinline__ M3 mmul(const M3 &x, const M3 &y) {
@@ -92,44 +92,119 @@ __device__ __forceinline__ void load_herm6(const double2 *blk, int b, int h, int
 }
 
 
-// 3x3 complex matrices in double-float (links split exactly into float pairs,
-// each product entry a lazy sum of six products): GB300 runs FP32 at ~60x its
-// FP64 rate, and the staple and clover-leaf products are most of the work of
-// a stout step and of the clover build
-struct M3d {
-    cplx<df> a[9];
-};
-__device__ __forceinline__ M3d load_link_df(const double2 *U, long long lex, int mu) {
-    M3d m;
-    const double2 *p = U + (lex * 4 + mu) * 9;
-    for (int k = 0; k < 9; k++) {
-        const double2 v = p[k];
-        m.a[k] = {df_from_double(v.x), df_from_double(v.y)};
+// c - a b and c - a conj(b), one FMA per real product
+__device__ __forceinline__ cplx<double> cfnma(cplx<double> a, cplx<double> b, cplx<double> c) {
+    return {fma(-a.re, b.re, fma(a.im, b.im, c.re)), fma(-a.re, b.im, fma(-a.im, b.re, c.im))};
+}
+__device__ __forceinline__ cplx<double> cfnmac(cplx<double> a, cplx<double> b, cplx<double> c) {
+    return {fma(-a.re, b.re, fma(-a.im, b.im, c.re)), fma(a.re, b.im, fma(-a.im, b.re, c.im))};
+}
+
+// B = L D L^dag of a Hermitian 6x6 block without pivoting (L unit lower triangular, D real): false
+// unless every |d_j| is at least 0.1 of the block's largest entry (compared as squares: 36 hypot calls
+// took a third of the inverse's FP64 time; a block whose squares leave the double range is refused
+// here and takes the pivoted path). The loops run over fixed trip counts with guards, so that they
+// unroll completely and every array stays in registers. W_ik = L_ik d_k.
+struct Ldl6 {
+    cplx<double> L[36];
+    double d[6], dinv[6];
+    __device__ __forceinline__ bool factor(const cplx<double> B[36]) {
+        double s2 = 0.0;
+#pragma unroll
+        for (int i = 0; i < 6; i++)
+#pragma unroll
+            for (int j = 0; j < 6; j++)
+                if (j >= i) {
+                    const cplx<double> v = B[i * 6 + j];
+                    s2 = fmax(s2, i == j ? v.re * v.re : fma(v.re, v.re, v.im * v.im));
+                }
+        bool ok = s2 > 1e-280 && s2 < 1e280;
+        cplx<double> W[36];
+#pragma unroll
+        for (int j = 0; j < 6; j++) {
+            double dj = B[j * 7].re;
+#pragma unroll
+            for (int k = 0; k < 6; k++)
+                if (k < j) dj = fma(-W[j * 6 + k].re, L[j * 6 + k].re, fma(-W[j * 6 + k].im, L[j * 6 + k].im, dj));
+            ok = ok && dj * dj >= 0.01 * s2;
+            d[j] = dj;
+            dinv[j] = 1.0 / dj;
+#pragma unroll
+            for (int i = 0; i < 6; i++)
+                if (i > j) {
+                    cplx<double> t = B[i * 6 + j];
+#pragma unroll
+                    for (int k = 0; k < 6; k++)
+                        if (k < j) t = cfnmac(W[i * 6 + k], L[j * 6 + k], t);
+                    W[i * 6 + j] = t;
+                    L[i * 6 + j] = cscale(dinv[j], t);
+                }
+        }
+        return ok;
     }
-    return m;
-}
-__device__ __forceinline__ M3d mdag_df(const M3d &x) {
-    M3d m;
+};
+
+// 3x3 complex matrices in double-float: GB300 runs FP32 at ~60x its FP64 rate, and the staple
+// and clover-leaf products are most of the work of a stout step and of the clover build. An
+// entry is a (re, im) pair of leading parts and one of low parts, and the products run on such
+// pairs with the packed FP32 instructions (one instruction for both components), each entry a
+// lazy sum of six products. The links come split (k_split_links, same order as the master
+// field, float4 (re.hi, im.hi, re.lo, im.lo)): splitting the doubles at every use took a
+// quarter of the instructions, and reading [site][4][9] links one site per thread 8 times the
+// L1 wavefronts. Against scalar sums on links split at each use (24^3x48, V = 663 552): clover
+// build 5.86 -> 2.30 ms (with ten products per plane instead of twelve), stout step
+// 5.79 -> 2.45 ms (with the exponential's series); the packed FP32 work is 1.4 ms of the first.
+struct M3p {
+    float2 hi[9], lo[9];
+};
+// U_mu(lex), or its adjoint
+__device__ __forceinline__ M3p load_link_pair(const float4 *P, long long V, long long lex, int mu, bool dag) {
+    M3p m;
+    const float4 *p = P + (long long)mu * 9 * V + lex;
+    const float sg = dag ? -1.0f : 1.0f;
+#pragma unroll
     for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) m.a[i * 3 + j] = {x.a[j * 3 + i].re, -x.a[j * 3 + i].im};
-    return m;
-}
-__device__ inline M3d mmul_df(const M3d &x, const M3d &y) {
-    M3d m;
-    for (int i = 0; i < 3; i++)
+#pragma unroll
         for (int j = 0; j < 3; j++) {
-            dfsum re = dfs_prod(x.a[i * 3].re, y.a[j].re), im = dfs_prod(x.a[i * 3].re, y.a[j].im);
-            dfs_add_prod(re, -x.a[i * 3].im, y.a[j].im);
-            dfs_add_prod(im, x.a[i * 3].im, y.a[j].re);
-            for (int k = 1; k < 3; k++) {
-                const cplx<df> p = x.a[i * 3 + k], q = y.a[k * 3 + j];
-                dfs_add_prod(re, p.re, q.re);
-                dfs_add_prod(re, -p.im, q.im);
-                dfs_add_prod(im, p.re, q.im);
-                dfs_add_prod(im, p.im, q.re);
-            }
-            m.a[i * 3 + j] = {dfs_done(re), dfs_done(im)};
+            const float4 v = p[(dag ? j * 3 + i : i * 3 + j) * V];
+            m.hi[i * 3 + j] = make_float2(v.x, sg * v.y);
+            m.lo[i * 3 + j] = make_float2(v.z, sg * v.w);
         }
     return m;
 }
-
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 swap2(float2 a) { return make_float2(a.y, a.x); }
+// x = x y, row by row
+__device__ __forceinline__ void mmul_pair(M3p &x, const M3p &y) {
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        float2 rh[3], rl[3];
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            dfsum2 z;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const float2 wh = x.hi[i * 3 + k], wl = x.lo[i * 3 + k], h = y.hi[k * 3 + j], l = y.lo[k * 3 + j];
+                if (k == 0) z = dfs2_prod(dup(wh.x), dup(wl.x), h, l);
+                else dfs2_add_prod(z, dup(wh.x), dup(wl.x), h, l);
+                dfs2_add_prod(z, make_float2(-wh.y, wh.y), make_float2(-wl.y, wl.y), swap2(h), swap2(l));
+            }
+            dfs2_done(z, rh[j], rl[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            x.hi[i * 3 + j] = rh[j];
+            x.lo[i * 3 + j] = rl[j];
+        }
+    }
+}
+// x = s x + y (s = +-1), normalised: a low part above half an ulp of its leading part would lose
+// the product of two low parts in the multiplication that follows
+__device__ __forceinline__ void madd_pair(M3p &x, const M3p &y, float s) {
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        const float2 a = __fmul2_rn(dup(s), x.hi[k]), al = __fmul2_rn(dup(s), x.lo[k]);
+        const dfsum2 t = two_sum2(a, y.hi[k]);
+        dfs2_done({t.s, __fadd2_rn(t.c, __fadd2_rn(al, y.lo[k]))}, x.hi[k], x.lo[k]);
+    }
+}

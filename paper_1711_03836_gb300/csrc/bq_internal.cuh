@@ -77,8 +77,11 @@ struct bq_ctx {
     int fp64_arith;  // BQ_FP64_NATIVE or BQ_FP64_DF64 for FP64-storage operator kernels
 
     // master fields (FP64, device)
-    double2 *U_canon;  // [V][4][9]
+    double2 *U_canon;  // [4][9][V]
     double2 *U_hop;    // stout-smeared copy for the hopping term (stout_iter > 0), same layout
+    float4 *U_pair;    // work field of the size of U_canon: links split into float pairs (same order) while
+                       // staples and leaves are formed, staging of links in the caller's layout otherwise
+    int U_pair_thin;   // U_pair holds the split of U_canon
     int U_hop_valid;
     double stout_rho;
     int stout_iter;
@@ -133,6 +136,8 @@ int bq_time_end(bq_ctx *c, int slot);
 // field preparation (bq_fields.cu)
 int bq_prepare_links(bq_ctx *c, int prec);
 int bq_prepare_clover(bq_ctx *c, int prec);
+int bq_split_links(bq_ctx *c, const double2 *U, int thin);  // U -> U_pair (bq_fields.cu)
+int bq_links_out(bq_ctx *c, double *dst, const double2 *U, int where);  // to the caller's layout
 int bq_prepare_hop_links(bq_ctx *c);  // stout-smeared canonical links of the hopping term (bq_gauge.cu)
 int bq_alloc(void **p, size_t bytes);
 int bq_pack(bq_ctx *c, void *native, const double *canon_dev, int prec);
