@@ -311,7 +311,8 @@ int bq_apply_mdagm(bq_ctx *ctx, void *out, const void *in, int precision);
  * `precision`); systems that share a context share the link and clover loads
  * of each of the four batched hopping-term launches, with the right-hand-side
  * mapping of bq_set_batch_mapping on ctx[0] (0 = shared-memory tiles for FP32
- * and FP16 storage, block-interleaved for FP64). The contexts obey the rules
+ * and FP16 storage with eight or more right-hand sides per lattice on average,
+ * else block-interleaved). The contexts obey the rules
  * of bq_solve_cg_batch (one device, same link storage and FP64 arithmetic);
  * queued on ctx[0]'s stream. No out[j] may alias an in[i]. The two
  * intermediate vectors per system are the batched solver's work vectors,

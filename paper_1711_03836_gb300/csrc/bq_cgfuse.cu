@@ -65,7 +65,7 @@ template <int PS, int RECON, int MODE, bool PN>
 __global__ void __launch_bounds__(128, DslashMinBlocks<PS>::value) k_dslash_cg(const DslashArgs a, const CgFuse f) {
     using T = typename Traits<PS>::real;
     constexpr int NV = MODE == CNT_CG_MHAT ? 2 : 1;
-    const int h = blockIdx.x * blockDim.x + threadIdx.x;
+    const int h = (gridDim.x - 1 - blockIdx.x) * 128 + threadIdx.x;  // from the last site: see k_dslash
     float v[NV];
 #pragma unroll
     for (int k = 0; k < NV; k++) v[k] = 0.f;

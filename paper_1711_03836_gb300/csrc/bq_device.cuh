@@ -125,6 +125,23 @@ __device__ __forceinline__ void bq_pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Links and clover blocks of a launch are read once per right-hand side. STREAM: without a
+// place in L1, which the neighbour spinors (read by several sites of an SM) then keep.
+template <bool STREAM>
+__device__ __forceinline__ float4 ldg_once(const float4 *p) {
+    if constexpr (!STREAM) return __ldg(p);
+    float4 v;
+    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+template <bool STREAM>
+__device__ __forceinline__ float2 ldg_once(const float2 *p) {
+    if constexpr (!STREAM) return __ldg(p);
+    float2 v;
+    asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ float2 h2f(uint32_t u) {
     __half2 h = *reinterpret_cast<__half2 *>(&u);
     return __half22float2(h);
@@ -308,11 +325,12 @@ template <int RECON>
 struct LinkIO<BQ_PREC_SINGLE, RECON> {
     using T = float;
     static constexpr int NF4 = (RECON == 12) ? 3 : 4;  // float4 chunks (2 complex each)
+    template <bool STREAM = false>
     __device__ static __forceinline__ void load(cplx<T> U[9], const char *blk, int h, int Vh) {
         const float4 *p = reinterpret_cast<const float4 *>(blk);
 #pragma unroll
         for (int k = 0; k < NF4; k++) {
-            float4 v = ldg(p + (size_t)k * Vh + h);
+            float4 v = ldg_once<STREAM>(p + (size_t)k * Vh + h);
             U[2 * k] = {v.x, v.y};
             U[2 * k + 1] = {v.z, v.w};
         }
@@ -320,7 +338,7 @@ struct LinkIO<BQ_PREC_SINGLE, RECON> {
             reconstruct_row2(U);
         } else {
             const float2 *t = reinterpret_cast<const float2 *>(p + (size_t)4 * Vh);
-            float2 v = ldg(t + h);
+            float2 v = ldg_once<STREAM>(t + h);
             U[8] = {v.x, v.y};
         }
     }
@@ -440,13 +458,14 @@ struct CloverIO<BQ_PREC_DOUBLE> {
 template <>
 struct CloverIO<BQ_PREC_SINGLE> {
     using T = float;
+    template <bool STREAM = false>
     __device__ static __forceinline__ void load_block(T d[6], cplx<T> o[15], const void *base, int b, int h,
                                                       int Vh) {
         const float4 *p = static_cast<const float4 *>(base) + (size_t)(9 * b) * Vh + h;
         float r[36];
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            float4 v = ldg(p + (size_t)k * Vh);
+            float4 v = ldg_once<STREAM>(p + (size_t)k * Vh);
             r[4 * k] = v.x;
             r[4 * k + 1] = v.y;
             r[4 * k + 2] = v.z;
@@ -719,14 +738,15 @@ __device__ __forceinline__ void herm6_apply<df>(const df d[6], const cplx<df> o[
     }
 }
 
-template <int PREC, typename T>
+template <int PREC, bool STREAM = false, typename T>
 __device__ __forceinline__ void clover_apply_site(cplx<T> out[12], const cplx<T> in[12], const void *clov, int h,
                                                   int Vh) {
 #pragma unroll
     for (int b = 0; b < 2; b++) {
         T d[6];
         cplx<T> o[15];
-        CloverIO<PREC>::load_block(d, o, clov, b, h, Vh);
+        if constexpr (STREAM) CloverIO<PREC>::template load_block<true>(d, o, clov, b, h, Vh);
+        else CloverIO<PREC>::load_block(d, o, clov, b, h, Vh);
         herm6_apply(d, o, in + 6 * b, out + 6 * b);
     }
 }

@@ -31,7 +31,9 @@ __global__ void __launch_bounds__(128, BatchMinBlocks<PREC>::value) k_dslash_bat
     int u = 0;
     while (u + 1 < tab.nunits && tab.block0[u + 1] <= (int)blockIdx.x) u++;
     const DslashUnit &U = tab.units[u];
-    const int bl = (int)blockIdx.x - tab.block0[u];
+    // the A x - k D step from the last site to the first (see k_dslash): 24^3x48 FP32, 2 / 12
+    // right-hand sides, Mhat^dag Mhat 286 -> 276 / 1414 -> 1384 us block-interleaved
+    const int bl = EPI == EPI_XPAY ? tab.block0[u + 1] - 1 - (int)blockIdx.x : (int)blockIdx.x - tab.block0[u];
     int r, h;
     if (U.interleave == 1) {  // block bl: rhs bl % nr, sites of block bl / nr (neighbours in time share the links in L2)
         r = bl % U.nr;
@@ -75,17 +77,29 @@ double dslash_site_bytes(int prec, int recon, int epi) {
 }
 double dslash_site_flops(int epi) { return 1320.0 + (epi != EPI_PLAIN ? 504.0 : 0.0) + (epi == EPI_XPAY ? 48.0 : 0.0); }
 
+// links (both parities) and the two clover fields of an operator application against L2
+static bool fields_exceed_l2(const DslashArgs &a, int recon) {
+    return (double)a.Vh * (8.0 * link_bytes_per_link(BQ_PREC_SINGLE, recon) + 2.0 * clover_bytes_per_site(BQ_PREC_SINGLE)) > 129e6;
+}
+
+template <int PREC, int RECON, bool STREAM>
+static void launch_dslash_prs(const DslashArgs &a, bool dag, int epi, unsigned grid, cudaStream_t s) {
+    if (dag) {
+        if (epi == EPI_PLAIN) bq_launch(k_dslash<PREC, RECON, true, EPI_PLAIN, STREAM>, grid, 128, s, a);
+        else if (epi == EPI_CLOVINV) bq_launch(k_dslash<PREC, RECON, true, EPI_CLOVINV, STREAM>, grid, 128, s, a);
+        else bq_launch(k_dslash<PREC, RECON, true, EPI_XPAY, STREAM>, grid, 128, s, a);
+    } else {
+        if (epi == EPI_PLAIN) bq_launch(k_dslash<PREC, RECON, false, EPI_PLAIN, STREAM>, grid, 128, s, a);
+        else if (epi == EPI_CLOVINV) bq_launch(k_dslash<PREC, RECON, false, EPI_CLOVINV, STREAM>, grid, 128, s, a);
+        else bq_launch(k_dslash<PREC, RECON, false, EPI_XPAY, STREAM>, grid, 128, s, a);
+    }
+}
 template <int PREC, int RECON>
 static void launch_dslash_pr(const DslashArgs &a, bool dag, int epi, unsigned grid, cudaStream_t s) {
-    if (dag) {
-        if (epi == EPI_PLAIN) bq_launch(k_dslash<PREC, RECON, true, EPI_PLAIN>, grid, 128, s, a);
-        else if (epi == EPI_CLOVINV) bq_launch(k_dslash<PREC, RECON, true, EPI_CLOVINV>, grid, 128, s, a);
-        else bq_launch(k_dslash<PREC, RECON, true, EPI_XPAY>, grid, 128, s, a);
-    } else {
-        if (epi == EPI_PLAIN) bq_launch(k_dslash<PREC, RECON, false, EPI_PLAIN>, grid, 128, s, a);
-        else if (epi == EPI_CLOVINV) bq_launch(k_dslash<PREC, RECON, false, EPI_CLOVINV>, grid, 128, s, a);
-        else bq_launch(k_dslash<PREC, RECON, false, EPI_XPAY>, grid, 128, s, a);
+    if constexpr (PREC == BQ_PREC_SINGLE && RECON != BQ_RECON_8) {
+        if (fields_exceed_l2(a, RECON)) return launch_dslash_prs<PREC, RECON, true>(a, dag, epi, grid, s);
     }
+    launch_dslash_prs<PREC, RECON, false>(a, dag, epi, grid, s);
 }
 
 // storage of the links and clover a launch at precision prec reads

@@ -95,7 +95,7 @@ __device__ __forceinline__ void accumulate_scaled(cplx<T> acc[12], const cplx<T>
     }
 }
 
-template <int PREC, int RECON, int MU, int S, bool BACK, bool SCALE, bool FRESH>
+template <int PREC, int RECON, int MU, int S, bool BACK, bool SCALE, bool FRESH, bool STREAM>
 __device__ __forceinline__ void hop(cplx<typename Traits<PREC>::real> acc[12], const void *in, int hn,
                                     const char *lblk, int hl, int Vh, typename Traits<PREC>::real coef) {
     using T = typename Traits<PREC>::real;
@@ -114,7 +114,8 @@ __device__ __forceinline__ void hop(cplx<typename Traits<PREC>::real> acc[12], c
     cplx<T> h0[3], h1[3];
     project<MU, S>(psi, h0, h1);
     cplx<T> U[9];
-    LinkIO<PREC, RECON>::load(U, lblk, hl, Vh);
+    if constexpr (STREAM && RECON == BQ_RECON_18) LinkIO<PREC, RECON>::template load<true>(U, lblk, hl, Vh);
+    else LinkIO<PREC, RECON>::load(U, lblk, hl, Vh);
     cplx<T> u0[3], u1[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -137,8 +138,9 @@ __device__ __forceinline__ void hop(cplx<typename Traits<PREC>::real> acc[12], c
         accumulate<MU, S>(acc, u0, u1);
 }
 
-// acc = D_hop in at output site h (the eight hops, Eq. 1 / Eq. 5); FRESH: see ldg
-template <int PREC, int RECON, bool DAG, bool FRESH>
+// acc = D_hop in at output site h (the eight hops, Eq. 1 / Eq. 5); FRESH: see ldg, STREAM: see ldg_once
+// (18-real links only: 12-real ones read that way measured 2 % slower)
+template <int PREC, int RECON, bool DAG, bool FRESH, bool STREAM = false>
 __device__ __forceinline__ void dslash_hops(const DslashArgs &a, const void *in, const int h,
                                             cplx<typename Traits<PREC>::real> acc[12]) {
     using T = typename Traits<PREC>::real;
@@ -161,52 +163,52 @@ __device__ __forceinline__ void dslash_hops(const DslashArgs &a, const void *in,
 
     {
         const int xn = (x + 1 == a.L0) ? 0 : x + 1;
-        hop<PREC, RECON, 0, SF, false, false, FRESH>(acc, in, h - xh + (xn >> 1), Lo, h, Vh, T(1));
+        hop<PREC, RECON, 0, SF, false, false, FRESH, STREAM>(acc, in, h - xh + (xn >> 1), Lo, h, Vh, T(1));
     }
     {
         const int xn = (x == 0) ? a.L0 - 1 : x - 1;
         const int hn = h - xh + (xn >> 1);
-        hop<PREC, RECON, 0, SB, true, false, FRESH>(acc, in, hn, Li, hn, Vh, T(1));
+        hop<PREC, RECON, 0, SB, true, false, FRESH, STREAM>(acc, in, hn, Li, hn, Vh, T(1));
     }
     {
         const int hn = (y + 1 == a.L1) ? h - (a.L1 - 1) * sy : h + sy;
-        hop<PREC, RECON, 1, SF, false, false, FRESH>(acc, in, hn, Lo + a.lblk, h, Vh, T(1));
+        hop<PREC, RECON, 1, SF, false, false, FRESH, STREAM>(acc, in, hn, Lo + a.lblk, h, Vh, T(1));
     }
     {
         const int hn = (y == 0) ? h + (a.L1 - 1) * sy : h - sy;
-        hop<PREC, RECON, 1, SB, true, false, FRESH>(acc, in, hn, Li + a.lblk, hn, Vh, T(1));
+        hop<PREC, RECON, 1, SB, true, false, FRESH, STREAM>(acc, in, hn, Li + a.lblk, hn, Vh, T(1));
     }
     {
         const int hn = (z + 1 == a.L2) ? h - (a.L2 - 1) * sz : h + sz;
-        hop<PREC, RECON, 2, SF, false, false, FRESH>(acc, in, hn, Lo + 2 * a.lblk, h, Vh, T(1));
+        hop<PREC, RECON, 2, SF, false, false, FRESH, STREAM>(acc, in, hn, Lo + 2 * a.lblk, h, Vh, T(1));
     }
     {
         const int hn = (z == 0) ? h + (a.L2 - 1) * sz : h - sz;
-        hop<PREC, RECON, 2, SB, true, false, FRESH>(acc, in, hn, Li + 2 * a.lblk, hn, Vh, T(1));
+        hop<PREC, RECON, 2, SB, true, false, FRESH, STREAM>(acc, in, hn, Li + 2 * a.lblk, hn, Vh, T(1));
     }
     {
         const bool wrap = (t + 1 == a.L3);
         const int hn = wrap ? h - (a.L3 - 1) * st : h + st;
         const T coef = (T)(wrap ? a.cf * a.bc : a.cf);
-        hop<PREC, RECON, 3, SF, false, true, FRESH>(acc, in, hn, Lo + 3 * a.lblk, h, Vh, coef);
+        hop<PREC, RECON, 3, SF, false, true, FRESH, STREAM>(acc, in, hn, Lo + 3 * a.lblk, h, Vh, coef);
     }
     {
         const bool wrap = (t == 0);
         const int hn = wrap ? h + (a.L3 - 1) * st : h - st;
         const T coef = (T)(wrap ? a.cb * a.bc : a.cb);
-        hop<PREC, RECON, 3, SB, true, true, FRESH>(acc, in, hn, Li + 3 * a.lblk, hn, Vh, coef);
+        hop<PREC, RECON, 3, SB, true, true, FRESH, STREAM>(acc, in, hn, Li + 3 * a.lblk, hn, Vh, coef);
     }
 }
 
 // o = A x - k acc at site h (the A_ee x - k D_eo step), x read from xin
-template <int PREC>
+template <int PREC, bool STREAM = false>
 __device__ __forceinline__ void xpay_site(const DslashArgs &a, const void *xin, const int h,
                                           const cplx<typename Traits<PREC>::real> acc[12],
                                           cplx<typename Traits<PREC>::real> xv[12],
                                           cplx<typename Traits<PREC>::real> o[12]) {
     using T = typename Traits<PREC>::real;
     SpinorIO<PREC>::template load<true>(xv, xin, h, a.Vh);
-    clover_apply_site<PREC>(o, xv, a.clov, h, a.Vh);
+    clover_apply_site<PREC, STREAM>(o, xv, a.clov, h, a.Vh);
     const T k = (T)a.k;
 #pragma unroll
     for (int c = 0; c < 12; c++) {
@@ -215,32 +217,32 @@ __device__ __forceinline__ void xpay_site(const DslashArgs &a, const void *xin, 
     }
 }
 
-template <int PREC, int RECON, bool DAG, int EPI>
+template <int PREC, int RECON, bool DAG, int EPI, bool STREAM>
 __device__ __forceinline__ void dslash_site(const DslashArgs &a, const void *in, void *out, const void *xin,
                                             const int h) {
     using T = typename Traits<PREC>::real;
     const int Vh = a.Vh;
     cplx<T> acc[12];
-    dslash_hops<PREC, RECON, DAG, true>(a, in, h, acc);
+    dslash_hops<PREC, RECON, DAG, true, STREAM>(a, in, h, acc);
     if (EPI == EPI_PLAIN) {
         SpinorIO<PREC>::store(out, h, Vh, acc);
     } else if (EPI == EPI_CLOVINV) {
         cplx<T> o[12];
-        clover_apply_site<PREC>(o, acc, a.clov, h, Vh);
+        clover_apply_site<PREC, STREAM>(o, acc, a.clov, h, Vh);
         SpinorIO<PREC>::store(out, h, Vh, o);
     } else {
         cplx<T> xv[12], o[12];
-        xpay_site<PREC>(a, xin, h, acc, xv, o);
+        xpay_site<PREC, STREAM>(a, xin, h, acc, xv, o);
         SpinorIO<PREC>::store(out, h, Vh, o);
     }
 }
 
 
-template <int PREC, int RECON, bool DAG, int EPI>
+template <int PREC, int RECON, bool DAG, int EPI, bool STREAM = false>
 __device__ __forceinline__ void dslash_any(const DslashArgs &a, const void *in, void *out, const void *xin,
                                            const int h) {
     static_assert(PREC != BQ_PREC_DF64, "double-float storage runs the lane-pair kernels of bq_df64.cuh");
-    dslash_site<PREC, RECON, DAG, EPI>(a, in, out, xin, h);
+    dslash_site<PREC, RECON, DAG, EPI, STREAM>(a, in, out, xin, h);
 }
 
 // Measured at 32^3x64: FP32 runs best at four 128-thread blocks per SM (128
@@ -264,10 +266,16 @@ template <>
 struct DslashMinBlocks<BQ_PREC_DOUBLE> {  // FP64-unit bound: no cap
     static constexpr int value = 1;
 };
-template <int PREC, int RECON, bool DAG, int EPI>
+// The launches of an operator alternate their direction over the lattice: the A x - k D step goes
+// from the last site to the first, so that it starts with the part of its input that the D_oe step
+// wrote last and L2 still holds (FP32 Mhat^dag Mhat: 24^3x48 191 -> 180 us, 32^3x64 549 -> 538 us;
+// CG iteration 242 -> 230 and 676 -> 664 us).
+// STREAM (FP32): where links and clover of an application exceed L2 (129 MB). 24^3x48 180 -> 176 us,
+// 32^3x64 538 -> 534 us, 48^3x96 with 18-real links 3367 -> 3241 us; L2-resident 16^3x32 31.1 -> 32.3 us.
+template <int PREC, int RECON, bool DAG, int EPI, bool STREAM>
 __global__ void __launch_bounds__(128, DslashMinBlocks<PREC>::value) k_dslash(const DslashArgs a) {
     bq_pdl_enter();
-    const int h = blockIdx.x * blockDim.x + threadIdx.x;
+    const int h = (EPI == EPI_XPAY ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * 128 + threadIdx.x;
     if (h >= a.Vh) return;
-    dslash_any<PREC, RECON, DAG, EPI>(a, a.in, a.out, a.xin, h);
+    dslash_any<PREC, RECON, DAG, EPI, STREAM>(a, a.in, a.out, a.xin, h);
 }

@@ -75,3 +75,25 @@ def test_fp64_links_follow_the_storage_setting(bq):  # noqa: F811
             bq.bq_apply_dhop(lat.ctx, out, src, 0, False, "double")
             assert rel(lat.unpack(out), oracle.dhop(p, links, A, psi, 0, False)) < TOL["double"], (arith, recon)
     lat.close()
+
+
+@pytest.mark.parametrize("prec", ["single", "half"])
+@pytest.mark.parametrize("counts,expect", [((1, 1), -1), ((7,), -1), ((8,), None), ((15, 1), None), ((14, 1), -1)])
+def test_default_batch_mapping(bq, prec, counts, expect):  # noqa: F811
+    """The default of the batched apply: tiles from eight right-hand sides per lattice on average."""
+    lats = [make(bq, d, recon=12, precision=prec, seed=i + 1) for i, d in enumerate([(6, 4, 6, 10), (4, 4, 4, 6)][:len(counts)])]
+    ctxs, ins, outs, want = [], [], [], []
+    for (lat, U, A, p), n in zip(lats, counts):
+        op = oracle.Operator(p, U, A)
+        for k in range(n):
+            psi = synth.gaussian_spinor(lat.Vh, k)
+            ctxs.append(lat)
+            ins.append(lat.pack(psi, prec))
+            outs.append(lat.spinor(prec))
+            want.append(op.mdagm(psi))
+    bq.bq_apply_mdagm_batch([c.ctx for c in ctxs], outs, ins, prec)
+    assert bq.bq_get_batch_mapping(ctxs[0].ctx) == (expect or {"single": -3, "half": -4}[prec])
+    for c, o, w in zip(ctxs, outs, want):
+        assert rel(c.unpack(o, prec), w) < TOL[prec]
+    for lat, *_ in lats:
+        lat.close()
