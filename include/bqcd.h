@@ -101,12 +101,13 @@ typedef struct {
  * 3 and 4 = the two A x - k D_hop steps of a single-system CG iteration with
  * the CG vector work fused in: 3 = t = Mhat p with |t|^2 and |p|^2 (so
  * <p, Ap> = |t|^2 + shift |p|^2), 4 = Mhat^dag t with the x and r updates and
- * |r|^2 (Ap itself is not stored).
+ * |r|^2 (Ap itself is not stored). Batches in a tile mapping count the same steps
+ * there; block-interleaved batches (mapping -1) count them as epilogue 2.
  * Bytes and flops are ALGORITHMIC per launch: 8 links + 1 input + 1 output
  * spinor per output site, plus the clover blocks (and the x spinor) the fused
  * epilogue reads; 1320 flops per site for D_hop, +504 per clover apply,
- * +48 for the xpay. fused_bytes holds, for buckets 3 and 4, the further bytes
- * of the fused vector work (bucket 4: p, x and r read, x and r written, minus
+ * +48 for the xpay. fused_bytes holds, for steps 3 and 4, the further bytes
+ * of the fused vector work (step 4: p, x and r read, x and r written, minus
  * the output spinor that is not stored). */
 typedef struct {
     long long launches;            /* every kernel the library launched since the last reset */

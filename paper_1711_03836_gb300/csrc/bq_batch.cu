@@ -112,42 +112,7 @@ __global__ void __launch_bounds__(RED_THREADS) kb_init(BArgs ba, int use_t) {
 template <int PS, int PR>
 __global__ void __launch_bounds__(RED_THREADS) kb_update_p(BArgs ba) {
     BATCH_PROLOGUE
-    if constexpr (PS == PR) {
-        const size_t n = (PS == BQ_PREC_DOUBLE ? 12 : 6) * (size_t)Vh;
-        if constexpr (PS == BQ_PREC_DOUBLE) {
-            const double beta = scal[S_BETA];
-            double2 *p = static_cast<double2 *>(sv.p);
-            const double2 *r = static_cast<const double2 *>(sv.rs);
-            for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-                const double2 a = p[i], b = r[i];
-                p[i] = make_double2(fma(beta, a.x, b.x), fma(beta, a.y, b.y));
-            }
-        } else {
-            const float beta = (float)scal[S_BETA];
-            float4 *p = static_cast<float4 *>(sv.p);
-            const float4 *r = static_cast<const float4 *>(sv.rs);
-            for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-                const float4 a = p[i], b = r[i];
-                p[i] = make_float4(fmaf(beta, a.x, b.x), fmaf(beta, a.y, b.y), fmaf(beta, a.z, b.z), fmaf(beta, a.w, b.w));
-            }
-        }
-        return;
-    }
-    using TS = typename Traits<PS>::real;
-    using TR = typename Traits<PR>::real;
-    const TS beta = (TS)scal[S_BETA];
-    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < Vh; h += gridDim.x * blockDim.x) {
-        cplx<TS> a[12];
-        cplx<TR> rv[12];
-        SpinorIO<PS>::load(a, sv.p, h, Vh);
-        SpinorIO<PR>::load(rv, sv.rs, h, Vh);
-#pragma unroll
-        for (int c = 0; c < 12; c++) {
-            a[c].re = fma(beta, a[c].re, (TS)rv[c].re);
-            a[c].im = fma(beta, a[c].im, (TS)rv[c].im);
-        }
-        SpinorIO<PS>::store(sv.p, h, Vh, a);
-    }
+    ms_pupdate_body<PS, PR>(sv.p, sv.rs, scal, Vh);
 }
 
 // Ap += sigma p; pAp = Re <p, Ap>; alpha = rr / pAp
@@ -269,6 +234,12 @@ __global__ void __launch_bounds__(RED_THREADS) kb_residual(BArgs ba) {
     }
 }
 
+// blocks of the p update: 16-byte words of the vector (FP16 p against FP32 r: sites), no limit from a reduction
+static unsigned p_update_grid(int ps, int pr, int Vh) {
+    if (ps != pr) return red_grid(Vh);
+    return (unsigned)(((ps == BQ_PREC_DOUBLE ? 12LL : 6LL) * Vh + RED_THREADS - 1) / RED_THREADS);
+}
+
 // --------------------------------------------------------------------------
 // workspace: per-system vectors cached in the first context, reused across calls
 
@@ -312,10 +283,10 @@ __global__ void __launch_bounds__(RED_THREADS) kbm_pupdate(BArgs ba, MSBArgs m, 
     ms_pupdate_body<PS, PR>(sv.p, ms_slot(m.ptr[sy], dst), scal, Vh);
 }
 
-// coefficients of the chunk (T iterations) of every system: one block per system
-__global__ void kbm_coef(MSBArgs m, int n, int T) {
+// coefficients of the chunk (T iterations) of every system: one block per system, one warp per shift
+__global__ void __launch_bounds__(32 * MS_MAX) kbm_coef(MSBArgs m, int T) {
     const double *mh = m.mh + (size_t)blockIdx.x * MH_TOTAL;
-    ms_coef_body(mh, m.mh + (size_t)blockIdx.x * MH_TOTAL + MH_HIST, n, T);
+    ms_coef_body(mh, m.mh + (size_t)blockIdx.x * MH_TOTAL + MH_HIST, T);
 }
 
 // apply the chunk to x_k and p_k of the systems flagged in ba.mask (grid row = system)
@@ -546,6 +517,7 @@ static int build_units(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int ma
             DslashUnit *u = &tab.units[tab.nunits];
             BQ_TRY(bq_dslash_unit_fill(c, prec, parity, dagger, epi, kk, &u->a));
             u->nr = e - s;
+            u->a.rev = bq_reverse(prec, BQ_RECON_12, epi, c->Vh, u->nr);
             u->log2R = log2_ceil(u->nr);
             u->interleave = m == -1 ? 1 : m == -2 ? 2 : m <= -3 ? 3 : 0;
             if (prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) {
@@ -775,8 +747,7 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     int maxVh = 0;
     for (int i = 0; i < nsys; i++) maxVh = ctxs[i]->Vh > maxVh ? ctxs[i]->Vh : maxVh;
     const dim3 G(red_grid(maxVh), nsys);
-    // p update: 16-byte words of the vector per thread (FP16 p against FP32 r: sites), no limit from a reduction
-    const dim3 GP(PS == PR ? (unsigned)(((PS == BQ_PREC_DOUBLE ? 12LL : 6LL) * maxVh + RED_THREADS - 1) / RED_THREADS) : G.x, nsys);
+    const dim3 GP(p_update_grid(PS, PR, maxVh), nsys);
 
     // device tables: per-system vectors and scalars (the launch tables stay on the host)
     std::vector<SysVec> hs(nsys);
@@ -827,12 +798,13 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
         cgf = CgFuse{w->slot[0].p, w->slot[0].xs, w->slot[0].rs, w->d_scal, w->d_fpart, sigma0 != 0.0,
                      w->d_ticket};
     }
-    // several FP32 / FP16 systems in the shared-memory tile mapping: the same fusion inside the tile kernel
-    const bool fuse_tiles = nsys > 1 && PS != BQ_PREC_DOUBLE && mapping <= -3;
-    TileCg tcg{};
+    // several FP32 / FP16 systems in the shared-memory tile mapping or block-interleaved: the same fusion
+    // inside those kernels, one partial per system and tile of 32 sites, or block of 128
+    const bool fuse_batch = nsys > 1 && PS != BQ_PREC_DOUBLE && (mapping <= -3 || mapping == -1);
+    BatchCg tcg{};
     double sum_vh = 0.0;
-    if (fuse_tiles) {
-        const int pstride = (maxVh + 31) / 32;
+    if (fuse_batch) {
+        const int psites = mapping == -1 ? 128 : 32, pstride = (maxVh + psites - 1) / psites;
         const size_t need = (size_t)nsys * 2 * pstride;
         if (w->fpart_n < need) {
             cudaFree(w->d_fpart);
@@ -841,7 +813,7 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
             BQ_TRY(bq_alloc((void **)&w->d_fpart, sizeof(double) * need));
             w->fpart_n = need;
         }
-        tcg = TileCg{w->d_sys, w->d_scal, w->d_fpart, pstride};
+        tcg = BatchCg{w->d_sys, w->d_scal, w->d_fpart, pstride, psites};
         for (int i = 0; i < nsys; i++) sum_vh += ctxs[i]->Vh;
     }
 
@@ -894,7 +866,7 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
             BQ_TRY(bq_dslash_cg_launch(c0, PS, nullptr, u[3]->in[0], u[3]->xin[0], u[3]->a.k, CNT_CG_MHATDAG, cgf));
             return BQ_OK;
         }
-        if (fuse_tiles) {
+        if (fuse_batch) {
             for (int k = 0; k < 4; k++) {
                 if (k == 0 || k == 2) {
                     BQ_TRY(batch_step(c0, PS, recon_s, k, &plan, nsys, d_active, frac));
@@ -906,7 +878,7 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
                 // step 3 moves p, x and r (x and r twice) in place of its output: 4 spinors of x's precision
                 const double fused = mode == CNT_CG_MHATDAG ? 4.0 * spinor_bytes_per_site(PR) * sum_vh * frac / nt : 0.0;
                 for (size_t q = 0; q < tabs.size(); q++)
-                    BQ_TRY(bq_tile_cg_launch(c0, PS, recon_s, &tabs[q], d_active, mode, tcg,
+                    BQ_TRY(bq_batch_cg_launch(c0, PS, recon_s, &tabs[q], d_active, mode, tcg,
                                              plan.bytes_all[k] * frac / nt, plan.flops_all[k] * frac / nt, fused));
                 BQ_TRY(bq_cg_finish_batch(c0, mode, tcg, d_active, nsys));
             }
@@ -1198,7 +1170,7 @@ static int ms_block_run(bq_ctx *c0, int nrhs, int n, const double *shifts, int b
     cudaStream_t s = c0->stream;
     std::vector<bq_ctx *> ctxs(nrhs, c0);
     const int Vh = c0->Vh;
-    const dim3 G(red_grid(Vh), nrhs);
+    const dim3 G(red_grid(Vh), nrhs), GP(p_update_grid(PS, PR, Vh), nrhs);
     // per (rhs, shift) solution and direction vectors
     const size_t vb = spinor_bytes_per_site(PR) * (size_t)Vh;
     if (w->ms_prec != PR || w->ms_Vh != Vh) {
@@ -1305,7 +1277,7 @@ static int ms_block_run(bq_ctx *c0, int nrhs, int n, const double *shifts, int b
     // fold the chunk's T iterations into x_k and p_k; the last residual becomes slot 0 of the next chunk
     auto flush = [&]() -> int {
         if (t == 0) return BQ_OK;
-        kbm_coef<<<nrhs, MS_MAX, 0, s>>>(mb, n, t);
+        kbm_coef<<<nrhs, 32 * n, 0, s>>>(mb, t);
         BQ_COUNT(c0);
         kbm_flush<PR><<<GF, RED_THREADS, 0, s>>>(ba_chunk, mb, n, t, slot0);
         BQ_COUNT(c0);
@@ -1322,7 +1294,7 @@ static int ms_block_run(bq_ctx *c0, int nrhs, int n, const double *shifts, int b
         const int src = (slot0 + t) % MS_SLOTS, dst = (slot0 + t + 1) % MS_SLOTS;
         kbm_residual<PS, PR><<<G, RED_THREADS, 0, s>>>(ba, mb, n, base, src, dst, t);
         BQ_COUNT(c0);
-        kbm_pupdate<PS, PR><<<G, RED_THREADS, 0, s>>>(ba, mb, dst);
+        kbm_pupdate<PS, PR><<<GP, RED_THREADS, 0, s>>>(ba, mb, dst);
         BQ_COUNT(c0);
         BQ_LAUNCH_CHECK();
         it++;

@@ -765,6 +765,7 @@ struct DslashArgs {
     double cf, cb;  // time-hop factors forward / backward (e^{+mu}, e^{-mu}, swapped for the adjoint)
     double bc;      // time boundary sign
     double k;       // xpay coefficient
+    int rev;        // run from the last site to the first (bq_reverse)
     int fmt;        // double-float kernels: spinors stored as float pairs (DF_IN_PAIR | DF_X_PAIR | DF_OUT_PAIR)
 };
 

@@ -282,7 +282,7 @@ __device__ __forceinline__ void dslash_site_df64_pair(const DslashArgs &a, const
 template <bool DAG, int EPI, int FMT>
 __global__ void __launch_bounds__(128, DF64P_MIN_BLOCKS) k_dslash_df64p(const DslashArgs a) {
     bq_pdl_enter();
-    const int t = (EPI == EPI_XPAY ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * 128 + threadIdx.x;  // see k_dslash
+    const int t = (a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * 128 + threadIdx.x;
     const int h = t >> 1;
     const bool valid = h < a.Vh;
     dslash_site_df64_pair<DAG, EPI, FMT>(a, a.in, a.out, a.xin, valid ? h : a.Vh - 1, t & 1, valid);
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(128, DF64P_MIN_BLOCKS) k_dslash_batch_df64p(co
     int u = 0;
     while (u + 1 < tab.nunits && tab.block0[u + 1] <= (int)blockIdx.x) u++;
     const DslashUnit &U = tab.units[u];
-    const int bl = EPI == EPI_XPAY ? tab.block0[u + 1] - 1 - (int)blockIdx.x : (int)blockIdx.x - tab.block0[u];
+    const int bl = U.a.rev ? tab.block0[u + 1] - 1 - (int)blockIdx.x : (int)blockIdx.x - tab.block0[u];
     const int r = bl % U.nr;
     if (mask && mask[U.sys[r]] == 0.0) return;  // the whole block: one right-hand side
     const int h = (bl / U.nr) * 64 + (int)(threadIdx.x >> 1);

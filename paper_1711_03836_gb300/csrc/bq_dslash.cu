@@ -31,9 +31,7 @@ __global__ void __launch_bounds__(128, BatchMinBlocks<PREC>::value) k_dslash_bat
     int u = 0;
     while (u + 1 < tab.nunits && tab.block0[u + 1] <= (int)blockIdx.x) u++;
     const DslashUnit &U = tab.units[u];
-    // the A x - k D step from the last site to the first (see k_dslash): 24^3x48 FP32, 2 / 12
-    // right-hand sides, Mhat^dag Mhat 286 -> 276 / 1414 -> 1384 us block-interleaved
-    const int bl = EPI == EPI_XPAY ? tab.block0[u + 1] - 1 - (int)blockIdx.x : (int)blockIdx.x - tab.block0[u];
+    const int bl = U.a.rev ? tab.block0[u + 1] - 1 - (int)blockIdx.x : (int)blockIdx.x - tab.block0[u];
     int r, h;
     if (U.interleave == 1) {  // block bl: rhs bl % nr, sites of block bl / nr (neighbours in time share the links in L2)
         r = bl % U.nr;
@@ -260,6 +258,7 @@ int bq_dslash_unit_fill(bq_ctx *c, int prec, int out_parity, int dagger, int epi
     a->cb = dagger ? ef : eb;
     a->bc = c->params.t_bc;
     a->k = k;
+    a->rev = bq_reverse(prec, c->links_recon[fs], epi, c->Vh, 1);
     a->fmt = 0;
     return BQ_OK;
 }

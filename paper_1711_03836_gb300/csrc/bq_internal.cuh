@@ -153,6 +153,17 @@ inline size_t links_block_bytes(const bq_ctx *c, int prec) {
 }
 
 
+// The launches of an operator alternate their direction over the lattice where its working set
+// (links, both clover fields, four spinors per right-hand side) exceeds L2: the A x - k D step goes
+// from the last site to the first, so that it starts with the part of its input that the D_oe step
+// wrote last and L2 still holds. FP32 Mhat^dag Mhat 24^3x48 191 -> 180 us, 32^3x64 549 -> 538 us, CG
+// iteration 242 -> 230 and 676 -> 664 us; a lattice that fits loses (16^3x32 CG 47.3 -> 49.5 us: its
+// sites change the die between launches).
+inline int bq_reverse(int prec, int recon, int epi, int Vh, int nr) {
+    return epi == EPI_XPAY && (double)Vh * (8.0 * link_bytes_per_link(prec, recon) + 2.0 * clover_bytes_per_site(prec) +
+                                            4.0 * nr * spinor_bytes_per_site(prec)) > 129e6;
+}
+
 // one unit of a batched hopping-term launch: a lattice (fields, geometry and
 // parameters in `a`) and up to DSLASH_UNIT_RHS right-hand sides
 // DSLASH_UNIT_RHS: capacity of a unit (the shared-memory tile mapping fills it);
@@ -212,18 +223,21 @@ struct SysVec {
 };
 
 // The same fusion for a batch of FP32 / FP16-storage systems in the shared-memory tile mapping
-// (bq_tile.cu): per system and tile of 32 sites one partial per value, [nsys][2][pstride]
-// with pstride >= the tiles of the largest lattice; scal [nsys][S_NSCAL]
-struct TileCg {
+// (bq_tile.cu) or block-interleaved (bq_cgfuse.cu): per system and psites = 32 (tile) or 128 (block)
+// sites one partial per value, [nsys][2][pstride] with pstride >= those of the largest lattice;
+// scal [nsys][S_NSCAL]
+struct BatchCg {
     const SysVec *sys;
     double *scal;
     double *partials;
-    int pstride;
+    int pstride, psites;
 };
-int bq_tile_cg_launch(bq_ctx *c, int prec, int recon, const DslashBatchTable *tab, const double *mask, int mode,
-                      const TileCg &cg, double site_bytes_total, double site_flops_total, double fused_bytes_total);
+int bq_batch_cg_launch(bq_ctx *c, int prec, int recon, const DslashBatchTable *tab, const double *mask, int mode,
+                       const BatchCg &cg, double site_bytes_total, double site_flops_total, double fused_bytes_total);
+void bq_interleaved_cg_launch(int prec, int recon, const DslashBatchTable &tab, const double *mask, int nblocks,
+                              int mode, const BatchCg &cg, cudaStream_t s);
 // the solver scalars of every unmasked system from the tile partials of a fused launch
-int bq_cg_finish_batch(bq_ctx *c, int mode, const TileCg &cg, const double *mask, int nsys);
+int bq_cg_finish_batch(bq_ctx *c, int mode, const BatchCg &cg, const double *mask, int nsys);
 
 // The CG vector work fused into the two A x - k D launches of one CG iteration
 // on Mhat^dag Mhat + sigma (single system, FP32 or FP16-storage inner iteration; bq_cgfuse.cu).

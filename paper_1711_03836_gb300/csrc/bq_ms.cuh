@@ -90,53 +90,75 @@ __device__ __forceinline__ void ms_residual_body(const void *Ap, const void *rsr
         SpinorIO<PR>::store(rdst, h, ra.Vh, rv);
         v[0] += norm2_site(rv);
     }
+    // the recurrences: one lane of the last block's first warp per shift (in one thread, ten shifts
+    // of dependent FP64 divisions took half of the kernel's 21 us at 16^3x32)
     double tot[1];
-    if (grid_sum(v, ra.partials, ra.ticket, tot) && threadIdx.x == 0) {
+    if (grid_sum(v, ra.partials, ra.ticket, tot) && threadIdx.x < 32) {
+        static_assert(MS_MAX <= 32, "one lane per shift");
+        const int k = threadIdx.x;
         const double rr = ra.scal[S_RR], rrn = tot[0];
         const double a = ra.scal[S_ALPHA], bta = rrn / rr;
-        ra.scal[S_RRPREV] = rr;
-        ra.scal[S_RR] = rrn;
-        ra.scal[S_BETA] = bta;
         const double ap = ms[M_APREV], bp = ms[M_BPREV];
-        int nact = 0;
-        for (int k = 0; k < n; k++) {
+        bool active = false;
+        if (k < n) {
             double *z = ms + M_ZETA * MS_MAX, *zo = ms + M_ZOLD * MS_MAX, *al = ms + M_ALPHA * MS_MAX,
                    *be = ms + M_BETA * MS_MAX, *act = ms + M_ACTIVE * MS_MAX, *upd = ms + M_UPD * MS_MAX;
+            double ha = 0.0, hb = 0.0, hz = 0.0;
             upd[k] = act[k];
-            hist_t[MH_A * MS_MAX + k] = hist_t[MH_B * MS_MAX + k] = hist_t[MH_Z * MS_MAX + k] = 0.0;
-            if (act[k] == 0.0) continue;
-            if (k == base) {
-                al[k] = a;
-                be[k] = bta;
-                act[k] = (rrn > tol2bb) ? 1.0 : 0.0;
-            } else {
-                const double sdiff = ms[M_SHIFT * MS_MAX + k] - ms[M_SHIFT * MS_MAX + base];
-                const double zk = z[k], zok = zo[k];
-                const double den = a * bp * (zok - zk) + zok * ap * (1.0 + sdiff * a);
-                const double zn = zk * zok * ap / den;
-                al[k] = a * zn / zk;
-                be[k] = bta * (zn / zk) * (zn / zk);
-                zo[k] = zk;
-                z[k] = zn;
-                act[k] = (zn * zn * rrn > tol2bb) ? 1.0 : 0.0;
+            if (act[k] != 0.0) {
+                double as = a, bs = bta, zn = 1.0;
+                if (k != base) {
+                    const double sdiff = ms[M_SHIFT * MS_MAX + k] - ms[M_SHIFT * MS_MAX + base];
+                    const double zk = z[k], zok = zo[k];
+                    const double den = a * bp * (zok - zk) + zok * ap * (1.0 + sdiff * a);
+                    zn = zk * zok * ap / den;
+                    as = a * zn / zk;
+                    bs = bta * (zn / zk) * (zn / zk);
+                    zo[k] = zk;
+                    z[k] = zn;
+                }
+                al[k] = ha = as;
+                be[k] = hb = bs;
+                hz = zn;
+                active = zn * zn * rrn > tol2bb;
+                act[k] = active ? 1.0 : 0.0;
             }
-            hist_t[MH_A * MS_MAX + k] = al[k];
-            hist_t[MH_B * MS_MAX + k] = be[k];
-            hist_t[MH_Z * MS_MAX + k] = (k == base) ? 1.0 : z[k];
-            nact += (act[k] != 0.0);
+            hist_t[MH_A * MS_MAX + k] = ha;
+            hist_t[MH_B * MS_MAX + k] = hb;
+            hist_t[MH_Z * MS_MAX + k] = hz;
         }
-        ms[M_APREV] = a;
-        ms[M_BPREV] = bta;
-        ms[M_NACTIVE] = nact;
+        const int nact = __popc(__ballot_sync(0xffffffffu, active));  // also: every lane has read the old scalars
+        if (k == 0) {
+            ra.scal[S_RRPREV] = rr;
+            ra.scal[S_RR] = rrn;
+            ra.scal[S_BETA] = bta;
+            ms[M_APREV] = a;
+            ms[M_BPREV] = bta;
+            ms[M_NACTIVE] = nact;
+        }
     }
 }
 
-// the base direction p = r + beta p
+// the base direction p = r + beta p; FP32 and FP64 vectors of one storage one 16-byte word at a time
 template <int PS, int PR>
 __device__ __forceinline__ void ms_pupdate_body(void *p, const void *r, const double *scal, int Vh) {
     using TS = typename Traits<PS>::real;
     using TR = typename Traits<PR>::real;
     const TS bt = (TS)scal[S_BETA];
+    if constexpr (PS == PR) {
+        const size_t n = (PS == BQ_PREC_DOUBLE ? 12 : 6) * (size_t)Vh;
+        for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+            if constexpr (PS == BQ_PREC_DOUBLE) {
+                const double2 a = static_cast<double2 *>(p)[i], b = static_cast<const double2 *>(r)[i];
+                static_cast<double2 *>(p)[i] = make_double2(fma(bt, a.x, b.x), fma(bt, a.y, b.y));
+            } else {
+                const float4 a = static_cast<float4 *>(p)[i], b = static_cast<const float4 *>(r)[i];
+                static_cast<float4 *>(p)[i] =
+                    make_float4(fmaf(bt, a.x, b.x), fmaf(bt, a.y, b.y), fmaf(bt, a.z, b.z), fmaf(bt, a.w, b.w));
+            }
+        }
+        return;
+    }
     for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < Vh; h += gridDim.x * blockDim.x) {
         cplx<TS> pv[12];
         cplx<TR> rv[12];
@@ -151,40 +173,47 @@ __device__ __forceinline__ void ms_pupdate_body(void *p, const void *r, const do
     }
 }
 
-// chunk coefficients of shift k (thread k) from the T rows of the history
-__device__ __forceinline__ void ms_coef_body(const double *hist, double *coef, int n, int T) {
-    const int k = threadIdx.x;
-    if (k >= n) return;
+// chunk coefficients from the T rows of the history: warp k takes shift k, its lane i - 1 the stored
+// residual R_i (one thread per shift read the history from global memory T^2 / 2 times: 62 us a chunk)
+__device__ __forceinline__ void ms_coef_body(const double *hist, double *coef, int T) {
+    static_assert(MS_CHUNK == 32, "one lane per stored residual");
+    __shared__ double sa[MS_MAX][MS_CHUNK], sb[MS_MAX][MS_CHUNK];
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double *cf = coef + (size_t)k * MH_COEF;
+    sa[k][lane] = lane < T ? hist[(lane * MH_N + MH_A) * MS_MAX + k] : 0.0;
+    sb[k][lane] = lane < T ? hist[(lane * MH_N + MH_B) * MS_MAX + k] : 0.0;
+    __syncwarp();
     // A = sum_t a_t g_t, g_{t+1} = g_t b_t
-    double g = 1.0, A = 0.0;
-    for (int t = 0; t < T; t++) {
-        A += hist[(t * MH_N + MH_A) * MS_MAX + k] * g;
-        g *= hist[(t * MH_N + MH_B) * MS_MAX + k];
+    if (lane == 0) {
+        double g = 1.0, A = 0.0;
+        for (int t = 0; t < T; t++) {
+            A += sa[k][t] * g;
+            g *= sb[k][t];
+        }
+        cf[0] = A;
+        cf[1] = g;
     }
-    cf[0] = A;
-    cf[1] = g;
     // for each stored residual R_i (i = 1..T): c_{t,i} = z_i prod_{m=i}^{t-1} b_m,
     // W_i = sum_{t=i}^{T-1} a_t c_{t,i}, C_i = c_{T,i}
-    for (int i = 1; i <= MS_CHUNK; i++) {
-        double W = 0.0, C = 0.0;
-        if (i <= T) {
-            double c = hist[((i - 1) * MH_N + MH_Z) * MS_MAX + k];  // z of r^{j0+i}, written at row i-1
-            for (int t = i; t < T; t++) {
-                W += hist[(t * MH_N + MH_A) * MS_MAX + k] * c;
-                c *= hist[(t * MH_N + MH_B) * MS_MAX + k];
-            }
-            C = c;
+    const int i = lane + 1;
+    double W = 0.0, C = 0.0;
+    if (i <= T) {
+        double c = hist[((i - 1) * MH_N + MH_Z) * MS_MAX + k];  // z of r^{j0+i}, written at row i-1
+        for (int t = i; t < T; t++) {
+            W += sa[k][t] * c;
+            c *= sb[k][t];
         }
-        cf[2 + (i - 1)] = W;
-        cf[2 + MS_CHUNK + (i - 1)] = C;
+        C = c;
     }
+    cf[2 + (i - 1)] = W;
+    cf[2 + MS_CHUNK + (i - 1)] = C;
 }
 
 // X_k += A_k P_k + sum_i W_{k,i} R_i and P_k = g_k P_k + sum_i C_{k,i} R_i for every shift,
-// groups of MS_GROUP shifts per pass; one thread per site and storage chunk (a float4 of
-// two complex components for FP32, a double2 for FP64), coefficients in shared memory
-constexpr int MS_GROUP = 8;
+// groups of GROUP shifts per pass (the residuals are read once per group; ten in FP32, 80 registers of
+// sums); one thread per site and storage chunk (a float4 of two complex components for FP32, a
+// double2 for FP64); coefficients in shared memory in the vectors' type: converting each from FP64
+// at its use kept the FP64 pipe busy for 430 of the 513 us of a 32-iteration chunk of ten shifts at 16^3x32
 
 template <int PR>
 struct MsChunk;
@@ -194,6 +223,7 @@ struct MsChunk<BQ_PREC_SINGLE> {
     using T = float;
     static constexpr int PER_SITE = 6;
     static constexpr int NR = 4;
+    static constexpr int GROUP = 10;
     __device__ static __forceinline__ void get(T v[4], const V &x) {
         v[0] = x.x;
         v[1] = x.y;
@@ -208,6 +238,7 @@ struct MsChunk<BQ_PREC_DOUBLE> {
     using T = double;
     static constexpr int PER_SITE = 12;
     static constexpr int NR = 2;
+    static constexpr int GROUP = 8;
     __device__ static __forceinline__ void get(T v[2], const V &x) {
         v[0] = x.x;
         v[1] = x.y;
@@ -221,9 +252,9 @@ __device__ __forceinline__ void ms_flush_body(const MSPtrs &ptr, const double *c
     using C = MsChunk<PR>;
     using V = typename C::V;
     using TT = typename C::T;
-    constexpr int NR = C::NR;
-    __shared__ double sc[MS_MAX * MH_COEF];
-    for (int i = threadIdx.x; i < n * MH_COEF; i += blockDim.x) sc[i] = coef[i];
+    constexpr int NR = C::NR, MS_GROUP = C::GROUP;
+    __shared__ TT sc[MS_MAX * MH_COEF];
+    for (int i = threadIdx.x; i < n * MH_COEF; i += blockDim.x) sc[i] = (TT)coef[i];
     __syncthreads();
     const long long nch = (long long)C::PER_SITE * Vh;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nch; e += (long long)gridDim.x * blockDim.x) {
@@ -236,7 +267,7 @@ __device__ __forceinline__ void ms_flush_body(const MSPtrs &ptr, const double *c
                 TT xv[NR], pv[NR];
                 C::get(xv, static_cast<const V *>(ptr.x[k])[e]);
                 C::get(pv, static_cast<const V *>(ptr.p[k])[e]);
-                const TT A = (TT)sc[k * MH_COEF], G = (TT)sc[k * MH_COEF + 1];
+                const TT A = sc[k * MH_COEF], G = sc[k * MH_COEF + 1];
 #pragma unroll
                 for (int q = 0; q < NR; q++) {
                     ax[g][q] = fma(A, pv[q], xv[q]);
@@ -262,7 +293,7 @@ __device__ __forceinline__ void ms_flush_body(const MSPtrs &ptr, const double *c
                     for (int g = 0; g < MS_GROUP; g++) {
                         const int k = k0 + g;
                         if (k >= n) continue;
-                        const TT W = (TT)sc[k * MH_COEF + 2 + (i - 1)], Cc = (TT)sc[k * MH_COEF + 2 + MS_CHUNK + (i - 1)];
+                        const TT W = sc[k * MH_COEF + 2 + (i - 1)], Cc = sc[k * MH_COEF + 2 + MS_CHUNK + (i - 1)];
 #pragma unroll
                         for (int q = 0; q < NR; q++) {
                             ax[g][q] = fma(W, rv[q], ax[g][q]);

@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(32) k_dslash_pair64(const DslashArgs a) {
     constexpr int SF = DAG ? +1 : -1;
     bq_pdl_enter();
     const int q = (int)(threadIdx.x >> 4) & 1;
-    const int hh = (EPI == EPI_XPAY ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * SPLIT_SITES + (int)(threadIdx.x & 15);
+    const int hh = (a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * SPLIT_SITES + (int)(threadIdx.x & 15);
     const bool valid = hh < a.Vh;
     const int h = valid ? hh : a.Vh - 1, Vh = a.Vh;
     const int xh = h % a.Lxh;

@@ -266,16 +266,12 @@ template <>
 struct DslashMinBlocks<BQ_PREC_DOUBLE> {  // FP64-unit bound: no cap
     static constexpr int value = 1;
 };
-// The launches of an operator alternate their direction over the lattice: the A x - k D step goes
-// from the last site to the first, so that it starts with the part of its input that the D_oe step
-// wrote last and L2 still holds (FP32 Mhat^dag Mhat: 24^3x48 191 -> 180 us, 32^3x64 549 -> 538 us;
-// CG iteration 242 -> 230 and 676 -> 664 us).
 // STREAM (FP32): where links and clover of an application exceed L2 (129 MB). 24^3x48 180 -> 176 us,
 // 32^3x64 538 -> 534 us, 48^3x96 with 18-real links 3367 -> 3241 us; L2-resident 16^3x32 31.1 -> 32.3 us.
 template <int PREC, int RECON, bool DAG, int EPI, bool STREAM>
 __global__ void __launch_bounds__(128, DslashMinBlocks<PREC>::value) k_dslash(const DslashArgs a) {
     bq_pdl_enter();
-    const int h = (EPI == EPI_XPAY ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * 128 + threadIdx.x;
+    const int h = (a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * 128 + threadIdx.x;
     if (h >= a.Vh) return;
     dslash_any<PREC, RECON, DAG, EPI, STREAM>(a, a.in, a.out, a.xin, h);
 }

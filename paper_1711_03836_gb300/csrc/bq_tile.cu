@@ -184,7 +184,7 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 template <int PREC, int RECON, bool DAG, int EPI, int CGM>
 __device__ __forceinline__ void dslash_site_tile(const DslashArgs &a, const SiteNb &nb, const void *in, void *out,
                                                  const void *xin, int h, const float4 *sL, const float4 *sC,
-                                                 int lane, const TileCg &cg, int sys, float (&v)[2]) {
+                                                 int lane, const BatchCg &cg, int sys, float (&v)[2]) {
     const int Vh = a.Vh;
     constexpr int SF = DAG ? +1 : -1;
     constexpr int SB = -SF;
@@ -367,7 +367,7 @@ __device__ __forceinline__ void dslash_site_tile(const DslashArgs &a, const Site
 // per thread 128, 96 or 80); the autotuner picks among the variants
 template <int PREC, int RECON, bool DAG, int EPI, int MB, int CGM = 0>
 __global__ void __launch_bounds__(128, MB) k_dslash_tile(const __grid_constant__ DslashBatchTable tab,
-                                                         const double *mask, const TileCg cg) {
+                                                         const double *mask, const BatchCg cg) {
     bq_pdl_enter();
     __shared__ float4 sL[8 * 5 * TILE_SITES];
     __shared__ float4 sC[EPI != EPI_PLAIN ? 18 * TILE_SITES : 1];
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(128, MB) k_dslash_tile(const __grid_constant__
 template <int PREC, int RECON, int MB>
 static void launch_tile_mb(const DslashBatchTable &tab, const double *mask, int nblocks, bool dag, int epi,
                            cudaStream_t s) {
-    const TileCg none{};
+    const BatchCg none{};
     if (dag) {
         if (epi == EPI_CLOVINV) bq_launch(k_dslash_tile<PREC, RECON, true, EPI_CLOVINV, MB>, nblocks, 128, s, tab, mask, none);
         else bq_launch(k_dslash_tile<PREC, RECON, true, EPI_XPAY, MB>, nblocks, 128, s, tab, mask, none);
@@ -451,7 +451,7 @@ void bq_tile_launch(int prec, int recon, const DslashBatchTable &tab, const doub
 
 template <int PREC, int RECON, int MB>
 static void launch_tile_cg_mb(const DslashBatchTable &tab, const double *mask, int nblocks, int mode,
-                              const TileCg &cg, cudaStream_t s) {
+                              const BatchCg &cg, cudaStream_t s) {
     if (mode == CNT_CG_MHAT)
         k_dslash_tile<PREC, RECON, false, EPI_XPAY, MB, CNT_CG_MHAT><<<nblocks, 128, 0, s>>>(tab, mask, cg);
     else
@@ -459,7 +459,7 @@ static void launch_tile_cg_mb(const DslashBatchTable &tab, const double *mask, i
 }
 
 template <int PREC, int RECON>
-static void launch_tile_cg_r(const DslashBatchTable &tab, const double *mask, int nblocks, int mode, const TileCg &cg,
+static void launch_tile_cg_r(const DslashBatchTable &tab, const double *mask, int nblocks, int mode, const BatchCg &cg,
                              cudaStream_t s) {
     // FP16 t with its norms needs the whole site in registers: at 80 registers (six blocks)
     // it spills about 200 bytes, so that step runs with five at most
@@ -471,31 +471,34 @@ static void launch_tile_cg_r(const DslashBatchTable &tab, const double *mask, in
 
 template <int PREC>
 static void launch_tile_cg_p(int recon, const DslashBatchTable &tab, const double *mask, int nblocks, int mode,
-                             const TileCg &cg, cudaStream_t s) {
+                             const BatchCg &cg, cudaStream_t s) {
     if (recon == 12) launch_tile_cg_r<PREC, 12>(tab, mask, nblocks, mode, cg, s);
     else if (recon == 8) launch_tile_cg_r<PREC, 8>(tab, mask, nblocks, mode, cg, s);
     else launch_tile_cg_r<PREC, 18>(tab, mask, nblocks, mode, cg, s);
 }
 
-int bq_tile_cg_launch(bq_ctx *c, int prec, int recon, const DslashBatchTable *tab, const double *mask, int mode,
-                      const TileCg &cg, double site_bytes_total, double site_flops_total, double fused_bytes_total) {
-    if (tab->nunits < 1 || tab->units[0].interleave != 3 || !(mode == CNT_CG_MHAT || mode == CNT_CG_MHATDAG) ||
+int bq_batch_cg_launch(bq_ctx *c, int prec, int recon, const DslashBatchTable *tab, const double *mask, int mode,
+                       const BatchCg &cg, double site_bytes_total, double site_flops_total, double fused_bytes_total) {
+    const bool tiles = tab->nunits > 0 && tab->units[0].interleave == 3;
+    if (tab->nunits < 1 || !(tiles || tab->units[0].interleave == 1) || !(mode == CNT_CG_MHAT || mode == CNT_CG_MHATDAG) ||
         !(prec == BQ_PREC_SINGLE || prec == BQ_PREC_HALF)) {
-        bq_set_error("fused CG step: FP32 / FP16 units in the shared-memory tile mapping only");
+        bq_set_error("fused CG step: FP32 / FP16 units in the shared-memory tile or block-interleaved mapping only");
         return BQ_ERR_ARG;
     }
     const int nblocks = tab->block0[tab->nunits];
+    const int bucket = tiles ? mode : (int)EPI_XPAY;  // see bq_counters
     int slot;
-    BQ_TRY(bq_time_begin(c, prec, mode, &slot));
-    if (prec == BQ_PREC_SINGLE) launch_tile_cg_p<BQ_PREC_SINGLE>(recon, *tab, mask, nblocks, mode, cg, c->stream);
+    BQ_TRY(bq_time_begin(c, prec, bucket, &slot));
+    if (!tiles) bq_interleaved_cg_launch(prec, recon, *tab, mask, nblocks, mode, cg, c->stream);
+    else if (prec == BQ_PREC_SINGLE) launch_tile_cg_p<BQ_PREC_SINGLE>(recon, *tab, mask, nblocks, mode, cg, c->stream);
     else launch_tile_cg_p<BQ_PREC_HALF>(recon, *tab, mask, nblocks, mode, cg, c->stream);
     BQ_LAUNCH_CHECK();
     BQ_TRY(bq_time_end(c, slot));
     BQ_COUNT(c);
-    c->counters.dslash_launches[prec][mode]++;
-    c->counters.dslash_bytes[prec][mode] += site_bytes_total;
-    c->counters.dslash_flops[prec][mode] += site_flops_total;
-    c->counters.fused_bytes[prec][mode] += fused_bytes_total;
+    c->counters.dslash_launches[prec][bucket]++;
+    c->counters.dslash_bytes[prec][bucket] += site_bytes_total;
+    c->counters.dslash_flops[prec][bucket] += site_flops_total;
+    c->counters.fused_bytes[prec][bucket] += fused_bytes_total;
     return BQ_OK;
 }
 
@@ -504,12 +507,12 @@ int bq_tile_cg_launch(bq_ctx *c, int prec, int recon, const DslashBatchTable *ta
 constexpr int CG_FIN_BATCH_THREADS = 1024;
 template <int MODE>
 __global__ void __launch_bounds__(CG_FIN_BATCH_THREADS) k_cg_finish_batch(const SysVec *sys, const double *partials,
-                                                                          int pstride, double *scal_all,
+                                                                          int pstride, int psites, double *scal_all,
                                                                           const double *mask) {
     constexpr int NV = MODE == CNT_CG_MHAT ? 2 : 1;
     const int sy = blockIdx.x;
     if (mask && mask[sy] == 0.0) return;
-    const int nt = (sys[sy].Vh + 31) / 32;
+    const int nt = (sys[sy].Vh + psites - 1) / psites;
     const double *pt = partials + (size_t)sy * 2 * pstride;
     double s[NV];
 #pragma unroll
@@ -526,12 +529,12 @@ __global__ void __launch_bounds__(CG_FIN_BATCH_THREADS) k_cg_finish_batch(const 
     }
 }
 
-int bq_cg_finish_batch(bq_ctx *c, int mode, const TileCg &cg, const double *mask, int nsys) {
+int bq_cg_finish_batch(bq_ctx *c, int mode, const BatchCg &cg, const double *mask, int nsys) {
     if (mode == CNT_CG_MHAT)
-        k_cg_finish_batch<CNT_CG_MHAT><<<nsys, CG_FIN_BATCH_THREADS, 0, c->stream>>>(cg.sys, cg.partials, cg.pstride,
+        k_cg_finish_batch<CNT_CG_MHAT><<<nsys, CG_FIN_BATCH_THREADS, 0, c->stream>>>(cg.sys, cg.partials, cg.pstride, cg.psites,
                                                                                   cg.scal, mask);
     else
-        k_cg_finish_batch<CNT_CG_MHATDAG><<<nsys, CG_FIN_BATCH_THREADS, 0, c->stream>>>(cg.sys, cg.partials, cg.pstride,
+        k_cg_finish_batch<CNT_CG_MHATDAG><<<nsys, CG_FIN_BATCH_THREADS, 0, c->stream>>>(cg.sys, cg.partials, cg.pstride, cg.psites,
                                                                                      cg.scal, mask);
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
