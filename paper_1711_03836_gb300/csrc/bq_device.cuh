@@ -595,27 +595,17 @@ __device__ __forceinline__ df normalise(df a) { return fast_two_sum(a.hi, a.lo);
 
 // exact split of an IEEE double into hi (its leading 24 significant bits,
 // truncated) and lo (the next 29 bits rounded to 24), with integer operations
-// only; |d| outside [2^-126, 2^128) maps to 0 / infinity
+// only: hi is the double's bits rebased and shifted as one 64-bit word, lo its
+// low 29 bits times hi's power of two; |d| outside [2^-126, 2^128) maps to
+// 0 / infinity
 __device__ __forceinline__ df df_from_double(double d) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(d);
-    const unsigned h32 = (unsigned)(u >> 32), l32 = (unsigned)u;
-    const unsigned sign = h32 & 0x80000000u;
-    const int e = (int)((h32 >> 20) & 0x7ffu);
-    const int ef = e - 896;  // biased float exponent of hi (1023 - 127)
-    const unsigned m23 = ((h32 & 0xfffffu) << 3) | (l32 >> 29);
-    const int el = e - 948;  // biased float exponent of 2^(e - 1075), the weight of the lowest bit
-    const float scale = (el >= 1) ? __uint_as_float((unsigned)el << 23) : 0.0f;
-    float lo = __fmul_rn(__uint2float_rn(l32 & 0x1fffffffu), scale);
-    lo = __uint_as_float(__float_as_uint(lo) | sign);
-    float hi = __uint_as_float(sign | ((unsigned)ef << 23) | m23);
-    if (ef < 1) {
-        hi = 0.0f;
-        lo = 0.0f;
-    } else if (ef > 254) {
-        hi = __uint_as_float(sign | 0x7f800000u);
-        lo = 0.0f;
-    }
-    return df(hi, lo);
+    const unsigned h32 = (unsigned)__double2hiint(d), l32 = (unsigned)__double2loint(d);
+    const unsigned a = h32 & 0x7fffffffu;  // biased exponents 1023 (double) and 127 (float): 896 apart
+    const unsigned hb = __funnelshift_l(l32, a - (896u << 20), 3) | (h32 & 0x80000000u);
+    const float lo = __fmul_rn(__fmul_rn(__uint2float_rn(l32 & 0x1fffffffu), 0x1p-52f), __uint_as_float(hb & 0xff800000u));
+    if (a - (897u << 20) >= (254u << 20))
+        return df(a < (1023u << 20) ? 0.0f : __uint_as_float((h32 & 0x80000000u) | 0x7f800000u), 0.0f);
+    return df(__uint_as_float(hb), lo);
 }
 __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
 
