@@ -14,7 +14,10 @@
 // components w, w + 4, w + 8 for the sum, the clover rows and the stores, so no
 // arithmetic is repeated: against one thread per site only 72 additions (the sums
 // over the four warps) come on top of 1128 operations. FP64 Mhat^dag Mhat at 8^4:
-// 158 us with one thread per site, 86 with two, 36 with eight; FP32 15.4 -> 14.1 us.
+// 158 us with one thread per site, 86 with two, 34 with eight; FP32 15.4 -> 13.4 us.
+// Both hops' loads are issued before either's arithmetic (two resident blocks per SM are
+// enough here; with the second hop's loads after the first's arithmetic 36 and 14.1 us;
+// the clover rows' loads before the hops as well: 36 us).
 //
 // What bounds the FP64 launches: an FP64 warp instruction holds its scheduler's FP64
 // pipe for about 64 cycles, so a launch takes whole rounds of (instructions per thread)
@@ -108,48 +111,63 @@ struct CloverRow {
     }
 };
 
-// one hop of half spinor q: up += f u, low += f times the lower spin that u feeds (FU, FL: set instead of
-// added); f = the time-hop coefficient and the site's FP16 scale, one multiplier of the accumulating FMAs
+// One hop of half spinor q, its loads apart from its arithmetic so that a thread can have several
+// hops' loads in flight. apply: up += f u, low += f times the lower spin that u feeds (FU, FL: set
+// instead of added); f = the time-hop coefficient and the site's FP16 scale, one multiplier of the
+// accumulating FMAs.
+template <int PREC, int RECON, int MU, int S, bool BACK>
+struct HalfHop {
+    using T = typename Traits<PREC>::real;
+    cplx<T> p[3], pj[3], U[9];
+    T f;
+    __device__ __forceinline__ void load(const void *in, int hn, const char *lblk, int hl, int Vh, int q, T coef) {
+        const int jq = MU < 2 ? 3 - q : 2 + q;
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            p[c] = load_comp<PREC>(in, 3 * q + c, hn, Vh);
+            pj[c] = load_comp<PREC>(in, 3 * jq + c, hn, Vh);
+        }
+        f = MU == 3 ? coef : T(1);
+        if (PREC == BQ_PREC_HALF) f *= load_scale<PREC>(in, hn, Vh);
+        LinkIO<PREC, RECON>::load(U, lblk, hl, Vh);
+    }
+    template <bool FU, bool FL>
+    __device__ __forceinline__ void apply(cplx<T> up[3], cplx<T> low[3], int q) const {
+        constexpr bool SCALED = PREC == BQ_PREC_HALF || MU == 3;
+        // the sign of the projector's off-diagonal factor differs between the halves for mu = y, z
+        const T s = (MU == 0) ? T(-S) : (MU == 3) ? T(S) : (q ? T(S) : T(-S));
+        cplx<T> h[3];
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            if (MU == 0 || MU == 2)  // p + i s pj
+                h[c] = {fma(-s, pj[c].im, p[c].re), fma(s, pj[c].re, p[c].im)};
+            else
+                h[c] = {fma(s, pj[c].re, p[c].re), fma(s, pj[c].im, p[c].im)};
+        }
+        // the lower spin takes i S u (x), s u (y), -i s u (z), S u (t)
+        const T g = (MU == 0) ? T(S) : (MU == 2) ? -s : s;
+        const T gf = SCALED ? g * f : g;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            cplx<T> u = BACK ? cmulc(U[a], h[0]) : cmul(U[a * 3], h[0]);
+#pragma unroll
+            for (int b = 1; b < 3; b++) u = BACK ? cfmac(U[b * 3 + a], h[b], u) : cfma(U[a * 3 + b], h[b], u);
+            const cplx<T> l = (MU == 0 || MU == 2) ? cplx<T>{-u.im, u.re} : u;
+            if (FU) up[a] = SCALED ? cscale(f, u) : u;
+            else up[a] = SCALED ? cplx<T>{fma(f, u.re, up[a].re), fma(f, u.im, up[a].im)} : cadd(up[a], u);
+            if (FL) low[a] = cscale(gf, l);
+            else low[a] = {fma(gf, l.re, low[a].re), fma(gf, l.im, low[a].im)};
+        }
+    }
+};
 template <int PREC, int RECON, int MU, int S, bool BACK, bool FU, bool FL>
 __device__ __forceinline__ void half_hop(cplx<typename Traits<PREC>::real> up[3],
                                          cplx<typename Traits<PREC>::real> low[3], const void *in, int hn,
                                          const char *lblk, int hl, int Vh, int q,
                                          typename Traits<PREC>::real coef) {
-    using T = typename Traits<PREC>::real;
-    constexpr bool SCALED = PREC == BQ_PREC_HALF || MU == 3;
-    const int jq = MU < 2 ? 3 - q : 2 + q;
-    // the sign of the projector's off-diagonal factor differs between the halves for mu = y, z
-    const T s = (MU == 0) ? T(-S) : (MU == 3) ? T(S) : (q ? T(S) : T(-S));
-    cplx<T> p[3], pj[3], U[9], h[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        p[c] = load_comp<PREC>(in, 3 * q + c, hn, Vh);
-        pj[c] = load_comp<PREC>(in, 3 * jq + c, hn, Vh);
-    }
-    T f = MU == 3 ? coef : T(1);
-    if (PREC == BQ_PREC_HALF) f *= load_scale<PREC>(in, hn, Vh);
-    LinkIO<PREC, RECON>::load(U, lblk, hl, Vh);
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        if (MU == 0 || MU == 2)  // p + i s pj
-            h[c] = {fma(-s, pj[c].im, p[c].re), fma(s, pj[c].re, p[c].im)};
-        else
-            h[c] = {fma(s, pj[c].re, p[c].re), fma(s, pj[c].im, p[c].im)};
-    }
-    // the lower spin takes i S u (x), s u (y), -i s u (z), S u (t)
-    const T g = (MU == 0) ? T(S) : (MU == 2) ? -s : s;
-    const T gf = SCALED ? g * f : g;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        cplx<T> u = BACK ? cmulc(U[a], h[0]) : cmul(U[a * 3], h[0]);
-#pragma unroll
-        for (int b = 1; b < 3; b++) u = BACK ? cfmac(U[b * 3 + a], h[b], u) : cfma(U[a * 3 + b], h[b], u);
-        const cplx<T> l = (MU == 0 || MU == 2) ? cplx<T>{-u.im, u.re} : u;
-        if (FU) up[a] = SCALED ? cscale(f, u) : u;
-        else up[a] = SCALED ? cplx<T>{fma(f, u.re, up[a].re), fma(f, u.im, up[a].im)} : cadd(up[a], u);
-        if (FL) low[a] = cscale(gf, l);
-        else low[a] = {fma(gf, l.re, low[a].re), fma(gf, l.im, low[a].im)};
-    }
+    HalfHop<PREC, RECON, MU, S, BACK> x;
+    x.load(in, hn, lblk, hl, Vh, q, coef);
+    x.template apply<FU, FL>(up, low, q);
 }
 
 template <int PREC, int RECON, bool DAG, int MU>
@@ -160,13 +178,17 @@ __device__ __forceinline__ void two_hops(cplx<typename Traits<PREC>::real> up[3]
     constexpr int SF = DAG ? +1 : -1;
     const char *Lo = a.links + (size_t)a.parity * 4 * a.lblk + MU * a.lblk;
     const char *Li = a.links + (size_t)(1 - a.parity) * 4 * a.lblk + MU * a.lblk;
-    half_hop<PREC, RECON, MU, SF, false, true, true>(up, low, a.in, hf, Lo, h, a.Vh, q, cf);
-    half_hop<PREC, RECON, MU, -SF, true, false, false>(up, low, a.in, hb, Li, hb, a.Vh, q, cb);
+    HalfHop<PREC, RECON, MU, SF, false> fwd;
+    HalfHop<PREC, RECON, MU, -SF, true> back;
+    fwd.load(a.in, hf, Lo, h, a.Vh, q, cf);
+    back.load(a.in, hb, Li, hb, a.Vh, q, cb);
+    fwd.template apply<true, true>(up, low, q);
+    back.template apply<false, false>(up, low, q);
 }
 
 // MODE 0, or the CG-fused steps of bq_cgfuse.cu (CNT_CG_MHAT / CNT_CG_MHATDAG, EPI_XPAY)
 template <int PREC, int RECON, bool DAG, int EPI, int MODE>
-__global__ void __launch_bounds__(128) k_dslash_split(const DslashArgs a, const CgFuse f) {
+__global__ void __launch_bounds__(128, 2) k_dslash_split(const DslashArgs a, const CgFuse f) {
     bq_pdl_enter();
     using T = typename Traits<PREC>::real;
     __shared__ T sp[4][24][SPLIT_SITES];                                   // partial spinors of the four warps
