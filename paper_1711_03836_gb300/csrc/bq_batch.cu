@@ -421,17 +421,17 @@ int bq_batch_reserve(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int pr) 
         if (sl->b) continue;
         const size_t v64 = spinor_bytes_per_site(BQ_PREC_DOUBLE) * (size_t)Vh;
         const size_t vr = spinor_bytes_per_site(pr) * (size_t)Vh, vs = spinor_bytes_per_site(ps) * (size_t)Vh;
-        BQ_TRY(bq_alloc((void **)&sl->b, v64));
-        BQ_TRY(bq_alloc((void **)&sl->x, v64));
-        BQ_TRY(bq_alloc((void **)&sl->r, v64));
-        BQ_TRY(bq_alloc((void **)&sl->t, v64));
-        BQ_TRY(bq_alloc((void **)&sl->to_d, v64));
-        BQ_TRY(bq_alloc((void **)&sl->rs, vr));
-        BQ_TRY(bq_alloc((void **)&sl->xs, vr));
-        BQ_TRY(bq_alloc((void **)&sl->p, vs));
-        BQ_TRY(bq_alloc((void **)&sl->Ap, vs));
-        BQ_TRY(bq_alloc((void **)&sl->to_s, vs));
-        BQ_TRY(bq_alloc((void **)&sl->te_s, vs));
+        BQ_TRY(bq_alloc((void **)&sl->b, v64, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->x, v64, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->r, v64, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->t, v64, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->to_d, v64, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->rs, vr, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->xs, vr, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->p, vs, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->Ap, vs, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->to_s, vs, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->te_s, vs, ctxs[s]));
         sl->Vh = Vh;
         sl->ps = ps;
         sl->pr = pr;
@@ -1189,12 +1189,12 @@ static int ms_block_run(bq_ctx *c0, int nrhs, int n, const double *shifts, int b
             hp[r].x[k] = hp[r].p[k] = nullptr;
             if (k >= n) continue;
             char **xv = &w->ms_vec[((size_t)r * MS_MAX + k) * 2], **pv = xv + 1;
-            BQ_TRY(bq_alloc((void **)xv, vb));
-            BQ_TRY(bq_alloc((void **)pv, vb));
+            BQ_TRY(bq_alloc((void **)xv, vb, c0));
+            BQ_TRY(bq_alloc((void **)pv, vb, c0));
             hp[r].x[k] = *xv;
             hp[r].p[k] = *pv;
         }
-        BQ_TRY(bq_alloc((void **)&w->ms_hist[r], vb * MS_SLOTS));
+        BQ_TRY(bq_alloc((void **)&w->ms_hist[r], vb * MS_SLOTS, c0));
         hp[r].hist = w->ms_hist[r];
         hp[r].hstride = (long long)vb;
     }

@@ -42,9 +42,17 @@ extern "C" const char *bq_strerror(int s) {
     }
 }
 
-int bq_alloc(void **p, size_t bytes) {
+int bq_alloc(void **p, size_t bytes, bq_ctx *c) {
     if (*p) return BQ_OK;
     cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
+    if (e != cudaSuccess && c && c->U_pair && cudaStreamSynchronize(c->stream) == cudaSuccess) {
+        // the links' work field is only needed while a configuration is prepared: give it back and try again
+        cudaGetLastError();
+        cudaFree(c->U_pair);
+        c->U_pair = nullptr;
+        c->U_pair_thin = 0;
+        e = cudaMalloc(p, bytes ? bytes : 16);
+    }
     if (e != cudaSuccess) {
         *p = nullptr;
         bq_set_error("cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
@@ -295,7 +303,7 @@ extern "C" int bq_set_u1(bq_ctx *c, const double *A, int where) {
             return BQ_ERR_ARG;
         }
     size_t bytes = (size_t)c->V * 4 * sizeof(double);
-    BQ_TRY(bq_alloc((void **)&c->A_u1, bytes));
+    BQ_TRY(bq_alloc((void **)&c->A_u1, bytes, c));
     BQ_CUDA_TRY(cudaMemcpyAsync(c->A_u1, A, bytes,
                                 where == BQ_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream));
     if (where == BQ_HOST) BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -359,7 +367,7 @@ int bq_prepare_links(bq_ctx *c, int prec) {
         cudaFree(c->links[prec]);
         c->links[prec] = nullptr;
     }
-    BQ_TRY(bq_alloc((void **)&c->links[prec], blk * 8));
+    BQ_TRY(bq_alloc((void **)&c->links[prec], blk * 8, c));
     c->links_recon[prec] = recon;
     Geo g = geo_of(c);
     unsigned grid = grid_for(c->V, 128);
@@ -674,7 +682,7 @@ extern "C" int bq_build_clover(bq_ctx *c) {
     }
     c->clov_user = 0;  // building from the links replaces a caller-supplied field
     size_t pblk = (size_t)36 * c->Vh;  // double2 per (parity, inverse) block
-    BQ_TRY(bq_alloc((void **)&c->clov_master, sizeof(double2) * pblk * 4));
+    BQ_TRY(bq_alloc((void **)&c->clov_master, sizeof(double2) * pblk * 4, c));
     Geo g = geo_of(c);
     BQ_CUDA_TRY(cudaMemsetAsync(c->dev_flag, 0, sizeof(int), c->stream));
     const unsigned nblk = (unsigned)((c->V + CLOVER_SITES - 1) / CLOVER_SITES);
@@ -733,7 +741,7 @@ extern "C" int bq_set_clover(bq_ctx *c, const double *A, int where) {
     c->clov_user = 0;
     invalidate_derived(c, 0, 1);
     const size_t pblk = (size_t)36 * c->Vh;
-    BQ_TRY(bq_alloc((void **)&c->clov_master, sizeof(double2) * pblk * 4));
+    BQ_TRY(bq_alloc((void **)&c->clov_master, sizeof(double2) * pblk * 4, c));
     Geo g = geo_of(c);
     // host data goes through a bounded device staging buffer, 2^20 sites (604 MB) at a time
     const long long chunk = where == BQ_HOST ? (c->V < (1LL << 20) ? c->V : (1LL << 20)) : c->V;
@@ -789,7 +797,7 @@ extern "C" int bq_set_clover(bq_ctx *c, const double *A, int where) {
 int bq_prepare_clover(bq_ctx *c, int prec) {
     if (!c->clov_master_valid) BQ_TRY(bq_build_clover(c));
     if (c->clov_valid[prec]) return BQ_OK;
-    BQ_TRY(bq_alloc((void **)&c->clov[prec], clover_bytes_per_site(prec) * (size_t)c->Vh * 4));
+    BQ_TRY(bq_alloc((void **)&c->clov[prec], clover_bytes_per_site(prec) * (size_t)c->Vh * 4, c));
     unsigned grid = grid_for(4LL * c->Vh, 128);
     if (prec == BQ_PREC_SINGLE)
         k_convert_clover<BQ_PREC_SINGLE><<<grid, 128, 0, c->stream>>>(c->clov[prec], (const double2 *)c->clov_master, c->Vh, 4);
@@ -864,7 +872,7 @@ extern "C" int bq_spinor_pack(bq_ctx *c, void *native, const double *canon, int 
     }
     const double *src = canon;
     if (where == BQ_HOST) {
-        BQ_TRY(bq_alloc((void **)&c->canon_stage, (size_t)c->Vh * 192));
+        BQ_TRY(bq_alloc((void **)&c->canon_stage, (size_t)c->Vh * 192, c));
         BQ_CUDA_TRY(cudaMemcpyAsync(c->canon_stage, canon, (size_t)c->Vh * 192, cudaMemcpyHostToDevice, c->stream));
         src = c->canon_stage;
     }
@@ -877,7 +885,7 @@ extern "C" int bq_spinor_unpack(bq_ctx *c, double *canon, const void *native, in
         return BQ_ERR_ARG;
     }
     if (where == BQ_DEVICE) return bq_unpack(c, canon, native, prec);
-    BQ_TRY(bq_alloc((void **)&c->canon_stage, (size_t)c->Vh * 192));
+    BQ_TRY(bq_alloc((void **)&c->canon_stage, (size_t)c->Vh * 192, c));
     BQ_TRY(bq_unpack(c, c->canon_stage, native, prec));
     BQ_CUDA_TRY(cudaMemcpyAsync(canon, c->canon_stage, (size_t)c->Vh * 192, cudaMemcpyDeviceToHost, c->stream));
     BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));

@@ -139,7 +139,7 @@ int bq_prepare_clover(bq_ctx *c, int prec);
 int bq_split_links(bq_ctx *c, const double2 *U, int thin);  // U -> U_pair (bq_fields.cu)
 int bq_links_out(bq_ctx *c, double *dst, const double2 *U, int where);  // to the caller's layout
 int bq_prepare_hop_links(bq_ctx *c);  // stout-smeared canonical links of the hopping term (bq_gauge.cu)
-int bq_alloc(void **p, size_t bytes);
+int bq_alloc(void **p, size_t bytes, bq_ctx *c = nullptr);  // c: its work field is given back if memory is short
 int bq_pack(bq_ctx *c, void *native, const double *canon_dev, int prec);
 int bq_unpack(bq_ctx *c, double *canon_dev, const void *native, int prec);
 
