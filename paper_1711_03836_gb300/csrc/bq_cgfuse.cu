@@ -41,6 +41,27 @@ __device__ __forceinline__ void block_partials(float (&v)[NV], double *partials,
             partials[k * stride + at] = (double)(((ws[k][0] + ws[k][1]) + ws[k][2]) + ws[k][3]);
 }
 
+// The same for the block-interleaved batch, whose sums were FP64 before they moved into the hopping
+// launches: the warp and block sums run in double-float (48 bits; the FP64 pipe would take a 5-step
+// chain of 64-cycle additions per warp and value).
+template <int NV>
+__device__ __forceinline__ void block_partials_df(float (&v)[NV], double *partials, int stride, int at) {
+    __shared__ df ws[NV][4];
+    const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
+#pragma unroll
+    for (int k = 0; k < NV; k++) {
+        df t(v[k], 0.0f);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            t = t + df(__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o));
+        if (lane == 0) ws[k][wid] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < NV; k++) partials[k * stride + at] = df_to_double(((ws[k][0] + ws[k][1]) + ws[k][2]) + ws[k][3]);
+}
+
 // the solver scalars from the block partials of a fused launch (one block of CG_FIN_THREADS)
 constexpr int CG_FIN_THREADS = 1024;
 template <int MODE>
@@ -217,7 +238,7 @@ __global__ void __launch_bounds__(128, DslashMinBlocks<PS>::value) k_dslash_batc
     if (h < U.a.Vh)
         cg_site<PS, RECON, MODE, true>(
             U.a, CgVec{U.in[r], U.xin[r], sv.p, U.out[r], sv.xs, sv.rs, cg.scal + (size_t)sys * S_NSCAL}, h, v);
-    block_partials(v, cg.partials + (size_t)sys * 2 * cg.pstride, cg.pstride, blk);
+    block_partials_df(v, cg.partials + (size_t)sys * 2 * cg.pstride, cg.pstride, blk);
 }
 
 template <int PS, int RECON>
