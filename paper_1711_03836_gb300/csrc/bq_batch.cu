@@ -795,8 +795,9 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
             w->fpart_n = need;
         }
         const double sigma0 = shifts ? shifts[0] : sp->shift;
-        cgf = CgFuse{w->slot[0].p, w->slot[0].xs, w->slot[0].rs, w->d_scal, w->d_fpart, sigma0 != 0.0,
-                     w->d_ticket};
+        // the eight-thread kernels read the shift on the device; for the others its being zero picks the kernel
+        cgf = CgFuse{w->slot[0].p, w->slot[0].xs, w->slot[0].rs, w->d_scal, w->d_fpart,
+                     sigma0 != 0.0 && !bq_use_split(ctxs[0], PS), w->d_ticket};
     }
     // several FP32 / FP16 systems in the shared-memory tile mapping or block-interleaved: the same fusion
     // inside those kernels, one partial per system and tile of 32 sites, or block of 128
@@ -897,14 +898,15 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     // describe one launch of the graph
     GraphRun *gp = nullptr;
     if (c0->use_graphs) {
-        // everything the captured launches depend on: tables, vectors, grid, timing mode
+        // everything the captured launches depend on: tables, vectors, kernels, grid, timing mode
         unsigned long long sig = 1469598103934665603ull;
         for (int step = 0; step < 4; step++)
             sig = fnv(sig, w->tables[step].data(), sizeof(DslashBatchTable) * w->tables[step].size());
         sig = fnv(sig, hs.data(), sizeof(SysVec) * nsys);
-        const long long misc[11] = {nsys, PS, PR, check, c0->timing, (long long)(uintptr_t)w->d_sys,
+        const long long misc[13] = {nsys, PS, PR, check, c0->timing, (long long)(uintptr_t)w->d_sys,
                                     (long long)(uintptr_t)w->d_scal, (long long)(uintptr_t)w->d_flags,
-                                    (long long)(uintptr_t)w->d_part, G.x, (long long)(uintptr_t)w->d_fpart};
+                                    (long long)(uintptr_t)w->d_part, G.x, (long long)(uintptr_t)w->d_fpart,
+                                    (long long)(uintptr_t)w->d_ticket, cgf.with_pnorm};
         sig = fnv(sig, misc, sizeof misc);
         if (!(w->graph.exec && w->graph_sig == sig && w->graph_gen == c0->counter_gen)) {
             drop_graph(c0, &w->graph);

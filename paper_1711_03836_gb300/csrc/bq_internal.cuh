@@ -248,7 +248,7 @@ struct CgFuse {
     void *xs, *rs;  // iterated solution and residual, FP32
     double *scal;
     double *partials;
-    int with_pnorm;  // sum |p|^2 too (the shift is nonzero)
+    int with_pnorm;  // sum |p|^2 too (the shift is nonzero); the eight-thread kernels read the shift instead
     unsigned int *ticket;  // small lattices (bq_split.cu): the launch's last block sums the partials
 };
 // mode CNT_CG_MHAT: out = t = A_ee p - k D_eo in (xin = p), then <p, Ap> = |t|^2 + sigma |p|^2

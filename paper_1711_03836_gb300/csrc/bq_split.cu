@@ -198,6 +198,9 @@ __global__ void __launch_bounds__(128, 2) k_dslash_split(const DslashArgs a, con
     const int hh = blockIdx.x * SPLIT_SITES + sl;
     const bool valid = hh < a.Vh;
     const int h = valid ? hh : a.Vh - 1, Vh = a.Vh;
+    // |p|^2 enters <p, Ap> only with a shift: decided here, so that a captured launch holds for every shift
+    bool with_pnorm = false;
+    if constexpr (MODE == CNT_CG_MHAT) with_pnorm = f.scal[S_SIGMA] != 0.0;
 
     const int xh = h % a.Lxh;
     int r = h / a.Lxh;
@@ -302,7 +305,7 @@ __global__ void __launch_bounds__(128, 2) k_dslash_split(const DslashArgs a, con
 #pragma unroll
             for (int k = 0; k < 3; k++) {
                 v[0] = fma(o[k], o[k], v[0]);
-                if (f.with_pnorm) {
+                if (with_pnorm) {
                     const T x = sx[2 * (4 * k + w) + q][sl];
                     v[NV - 1] = fma(x, x, v[NV - 1]);
                 }
