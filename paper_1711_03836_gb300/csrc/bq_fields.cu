@@ -203,25 +203,55 @@ extern "C" int bq_set_recon(bq_ctx *c, int prec, int recon) {
 
 // Links between the caller's layout [V][4][9] and the library's [4][9][V]: a block takes 32 sites
 // through shared memory, so that both sides are read and written along consecutive addresses.
+// WIDE: the caller's links lie on a 16-byte boundary; otherwise they go one double at a time.
 #define LINK_SITES 32
-template <bool IN>
-__global__ void __launch_bounds__(256) k_links_layout(double2 *dst, const double2 *src, long long V) {
+template <bool IN, bool WIDE>
+__global__ void __launch_bounds__(256) k_links_layout(double2 *lib, double *user, long long V) {
     __shared__ double2 sm[LINK_SITES][37];  // 37: the columns start in different banks
     const long long x0 = (long long)blockIdx.x * LINK_SITES;
     const int n = V - x0 < LINK_SITES ? (int)(V - x0) : LINK_SITES;
+    user += x0 * 72;
     if (IN) {
-        for (int i = threadIdx.x; i < 36 * n; i += 256) sm[i / 36][i % 36] = src[x0 * 36 + i];
+        for (int i = threadIdx.x; i < 36 * n; i += 256)
+            sm[i / 36][i % 36] = WIDE ? reinterpret_cast<const double2 *>(user)[i] : make_double2(user[2 * i], user[2 * i + 1]);
     } else {
         for (int i = threadIdx.x; i < 36 * LINK_SITES; i += 256)
-            if (i % LINK_SITES < n) sm[i % LINK_SITES][i / LINK_SITES] = src[(i / LINK_SITES) * V + x0 + i % LINK_SITES];
+            if (i % LINK_SITES < n) sm[i % LINK_SITES][i / LINK_SITES] = lib[(i / LINK_SITES) * V + x0 + i % LINK_SITES];
     }
     __syncthreads();
     if (IN) {
         for (int i = threadIdx.x; i < 36 * LINK_SITES; i += 256)
-            if (i % LINK_SITES < n) dst[(i / LINK_SITES) * V + x0 + i % LINK_SITES] = sm[i % LINK_SITES][i / LINK_SITES];
+            if (i % LINK_SITES < n) lib[(i / LINK_SITES) * V + x0 + i % LINK_SITES] = sm[i % LINK_SITES][i / LINK_SITES];
     } else {
-        for (int i = threadIdx.x; i < 36 * n; i += 256) dst[x0 * 36 + i] = sm[i / 36][i % 36];
+        for (int i = threadIdx.x; i < 36 * n; i += 256) {
+            const double2 v = sm[i / 36][i % 36];
+            if (WIDE) {
+                reinterpret_cast<double2 *>(user)[i] = v;
+            } else {
+                user[2 * i] = v.x;
+                user[2 * i + 1] = v.y;
+            }
+        }
     }
+}
+
+template <bool IN>
+static void launch_links_layout(bq_ctx *c, double2 *lib, double *user) {
+    const unsigned grid = grid_for(c->V, LINK_SITES);
+    if ((uintptr_t)user % sizeof(double2) == 0) k_links_layout<IN, true><<<grid, 256, 0, c->stream>>>(lib, user, c->V);
+    else k_links_layout<IN, false><<<grid, 256, 0, c->stream>>>(lib, user, c->V);
+}
+
+// a caller's BQ_DEVICE links that a kernel of this context can take as they lie: doubles on this device.
+// Others (another device's memory, an address that is no multiple of eight) go through a copy.
+static bool links_direct(const bq_ctx *c, const void *p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (uintptr_t)p % sizeof(double) == 0 &&
+           (at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == c->device));
 }
 
 // every link entry split into float pairs (re.hi, im.hi, re.lo, im.lo), exactly but for the last
@@ -249,17 +279,19 @@ int bq_split_links(bq_ctx *c, const double2 *U, int thin) {
 }
 
 int bq_links_out(bq_ctx *c, double *dst, const double2 *U, int where) {
-    double2 *to = (double2 *)dst;
-    if (where == BQ_HOST) {
+    double *to = dst;
+    const bool copy = where == BQ_HOST || !links_direct(c, dst);
+    if (copy) {
         BQ_TRY(bq_alloc((void **)&c->U_pair, link_field_bytes(c)));
         c->U_pair_thin = 0;
-        to = (double2 *)c->U_pair;
+        to = (double *)c->U_pair;
     }
-    k_links_layout<false><<<grid_for(c->V, LINK_SITES), 256, 0, c->stream>>>(to, U, c->V);
+    launch_links_layout<false>(c, const_cast<double2 *>(U), to);
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
-    if (where == BQ_HOST)
-        BQ_CUDA_TRY(cudaMemcpyAsync(dst, to, link_field_bytes(c), cudaMemcpyDeviceToHost, c->stream));
+    if (copy)
+        BQ_CUDA_TRY(cudaMemcpyAsync(dst, to, link_field_bytes(c),
+                                    where == BQ_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, c->stream));
     BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
     return BQ_OK;
 }
@@ -270,14 +302,15 @@ extern "C" int bq_set_gauge(bq_ctx *c, const double *U, int where) {
         return BQ_ERR_ARG;
     }
     BQ_TRY(bq_alloc((void **)&c->U_canon, link_field_bytes(c)));
-    const double2 *src = (const double2 *)U;
+    double *src = const_cast<double *>(U);
     c->U_pair_thin = 0;
-    if (where == BQ_HOST) {
+    if (where == BQ_HOST || !links_direct(c, U)) {
         BQ_TRY(bq_alloc((void **)&c->U_pair, link_field_bytes(c)));
-        BQ_CUDA_TRY(cudaMemcpyAsync(c->U_pair, U, link_field_bytes(c), cudaMemcpyHostToDevice, c->stream));
-        src = (const double2 *)c->U_pair;
+        BQ_CUDA_TRY(cudaMemcpyAsync(c->U_pair, U, link_field_bytes(c),
+                                    where == BQ_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream));
+        src = (double *)c->U_pair;
     }
-    k_links_layout<true><<<grid_for(c->V, LINK_SITES), 256, 0, c->stream>>>(c->U_canon, src, c->V);
+    launch_links_layout<true>(c, c->U_canon, src);
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
     if (where == BQ_HOST) BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
