@@ -160,7 +160,14 @@ int bq_set_fp64_arith(bq_ctx *ctx, int mode);
 int bq_set_cuda_graphs(bq_ctx *ctx, int enable);
 
 /* Gauge links in canonical layout U[V][4][3][3] complex FP64, from host or
- * device memory (where = BQ_HOST / BQ_DEVICE). Copied; derived fields rebuilt lazily. */
+ * device memory (where = BQ_HOST / BQ_DEVICE; any address: links on a 16-byte
+ * boundary of the context's device are read fastest, others on an 8-byte
+ * boundary one double at a time, all else through a buffer of at most 151 MB
+ * that the context keeps, as it does for host links). Copied; derived fields
+ * rebuilt lazily. Beside the fields themselves (links, smeared links, clover,
+ * and the packed links and clover of each storage in use) preparing a
+ * configuration holds no memory: what it needs meanwhile lies in fields that
+ * are out of date, or is allocated for the call if there is room. */
 int bq_set_gauge(bq_ctx *ctx, const double *U, int where);
 
 /* U(1) angles A[V][4] (Eq. 5), or NULL to remove the U(1) field. */
@@ -231,7 +238,9 @@ int bq_set_stout(bq_ctx *ctx, double rho, int n_iter);
 
 /* Copy the links the hopping term uses (smeared when bq_set_stout is on,
  * otherwise the gauge field as set) in the canonical layout [V][4][3][3]
- * complex into U (host or device). BQ_ERR_STATE without a gauge field. */
+ * complex into U (host or device; any address, as for bq_set_gauge). Device
+ * memory serves as work space first, so that U holds nothing defined if the
+ * call fails. BQ_ERR_STATE without a gauge field. */
 int bq_get_hop_links(bq_ctx *ctx, double *U, int where);
 
 /* log det of the clover term (Eq. 2) summed over the sites of one parity:

@@ -421,17 +421,17 @@ int bq_batch_reserve(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int pr) 
         if (sl->b) continue;
         const size_t v64 = spinor_bytes_per_site(BQ_PREC_DOUBLE) * (size_t)Vh;
         const size_t vr = spinor_bytes_per_site(pr) * (size_t)Vh, vs = spinor_bytes_per_site(ps) * (size_t)Vh;
-        BQ_TRY(bq_alloc((void **)&sl->b, v64, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->x, v64, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->r, v64, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->t, v64, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->to_d, v64, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->rs, vr, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->xs, vr, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->p, vs, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->Ap, vs, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->to_s, vs, ctxs[s]));
-        BQ_TRY(bq_alloc((void **)&sl->te_s, vs, ctxs[s]));
+        BQ_TRY(bq_alloc((void **)&sl->b, v64));
+        BQ_TRY(bq_alloc((void **)&sl->x, v64));
+        BQ_TRY(bq_alloc((void **)&sl->r, v64));
+        BQ_TRY(bq_alloc((void **)&sl->t, v64));
+        BQ_TRY(bq_alloc((void **)&sl->to_d, v64));
+        BQ_TRY(bq_alloc((void **)&sl->rs, vr));
+        BQ_TRY(bq_alloc((void **)&sl->xs, vr));
+        BQ_TRY(bq_alloc((void **)&sl->p, vs));
+        BQ_TRY(bq_alloc((void **)&sl->Ap, vs));
+        BQ_TRY(bq_alloc((void **)&sl->to_s, vs));
+        BQ_TRY(bq_alloc((void **)&sl->te_s, vs));
         sl->Vh = Vh;
         sl->ps = ps;
         sl->pr = pr;
@@ -1026,7 +1026,10 @@ int bq_batch_prepare(int nsys, bq_ctx *const *ctxs, int ps) {
         BQ_TRY(bq_prepare_links(c, ps));
         BQ_TRY(bq_prepare_clover(c, ps));
         // field preparation ran on this context's stream; the batch runs on ctx[0]'s
-        if (c->stream != ctxs[0]->stream) BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
+        if (c->stream != ctxs[0]->stream) {
+            c->read_elsewhere = 1;
+            BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
+        }
     }
     return BQ_OK;
 }
@@ -1191,12 +1194,12 @@ static int ms_block_run(bq_ctx *c0, int nrhs, int n, const double *shifts, int b
             hp[r].x[k] = hp[r].p[k] = nullptr;
             if (k >= n) continue;
             char **xv = &w->ms_vec[((size_t)r * MS_MAX + k) * 2], **pv = xv + 1;
-            BQ_TRY(bq_alloc((void **)xv, vb, c0));
-            BQ_TRY(bq_alloc((void **)pv, vb, c0));
+            BQ_TRY(bq_alloc((void **)xv, vb));
+            BQ_TRY(bq_alloc((void **)pv, vb));
             hp[r].x[k] = *xv;
             hp[r].p[k] = *pv;
         }
-        BQ_TRY(bq_alloc((void **)&w->ms_hist[r], vb * MS_SLOTS, c0));
+        BQ_TRY(bq_alloc((void **)&w->ms_hist[r], vb * MS_SLOTS));
         hp[r].hist = w->ms_hist[r];
         hp[r].hstride = (long long)vb;
     }

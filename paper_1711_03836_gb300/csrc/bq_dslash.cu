@@ -329,8 +329,8 @@ int bq_mdagm_launch(bq_ctx *c, int prec, void *out, const void *in, void *tmp_od
 
 int bq_workspace(bq_ctx *c, int prec) {
     size_t b = spinor_bytes_per_site(prec) * (size_t)c->Vh;
-    BQ_TRY(bq_alloc((void **)&c->tmp_odd[prec], b, c));
-    BQ_TRY(bq_alloc((void **)&c->tmp_even[prec], b, c));
+    BQ_TRY(bq_alloc((void **)&c->tmp_odd[prec], b));
+    BQ_TRY(bq_alloc((void **)&c->tmp_even[prec], b));
     return BQ_OK;
 }
 

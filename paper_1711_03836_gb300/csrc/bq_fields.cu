@@ -42,18 +42,11 @@ extern "C" const char *bq_strerror(int s) {
     }
 }
 
-int bq_alloc(void **p, size_t bytes, bq_ctx *c) {
+int bq_alloc(void **p, size_t bytes) {
     if (*p) return BQ_OK;
     cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
-    if (e != cudaSuccess && c && c->U_pair && cudaStreamSynchronize(c->stream) == cudaSuccess) {
-        // the links' work field is only needed while a configuration is prepared: give it back and try again
-        cudaGetLastError();
-        cudaFree(c->U_pair);
-        c->U_pair = nullptr;
-        c->U_pair_thin = 0;
-        e = cudaMalloc(p, bytes ? bytes : 16);
-    }
     if (e != cudaSuccess) {
+        cudaGetLastError();  // reported here, not by the next launch
         *p = nullptr;
         bq_set_error("cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
         return BQ_ERR_NOMEM;
@@ -134,7 +127,6 @@ extern "C" int bq_destroy(bq_ctx *c) {
     bq_full_free(c);
     cudaFree(c->U_canon);
     cudaFree(c->U_hop);
-    cudaFree(c->U_pair);
     cudaFree(c->A_u1);
     for (int p = 0; p < BQ_NFIELD; p++) {
         cudaFree(c->links[p]);
@@ -146,6 +138,7 @@ extern "C" int bq_destroy(bq_ctx *c) {
     }
     cudaFree(c->clov_master);
     cudaFree(c->canon_stage);
+    cudaFree(c->link_stage);
     cudaFree(c->red_partials);
     cudaFree(c->red_ticket);
     cudaFree(c->dev_flag);
@@ -205,11 +198,12 @@ extern "C" int bq_set_recon(bq_ctx *c, int prec, int recon) {
 // through shared memory, so that both sides are read and written along consecutive addresses.
 // WIDE: the caller's links lie on a 16-byte boundary; otherwise they go one double at a time.
 #define LINK_SITES 32
+// Here `lib` and `user` point at the first of n_sites sites.
 template <bool IN, bool WIDE>
-__global__ void __launch_bounds__(256) k_links_layout(double2 *lib, double *user, long long V) {
+__global__ void __launch_bounds__(256) k_links_layout(double2 *lib, double *user, long long V, long long n_sites) {
     __shared__ double2 sm[LINK_SITES][37];  // 37: the columns start in different banks
     const long long x0 = (long long)blockIdx.x * LINK_SITES;
-    const int n = V - x0 < LINK_SITES ? (int)(V - x0) : LINK_SITES;
+    const int n = n_sites - x0 < LINK_SITES ? (int)(n_sites - x0) : LINK_SITES;
     user += x0 * 72;
     if (IN) {
         for (int i = threadIdx.x; i < 36 * n; i += 256)
@@ -235,16 +229,17 @@ __global__ void __launch_bounds__(256) k_links_layout(double2 *lib, double *user
     }
 }
 
+// sites x0 .. x0 + n - 1; `user` holds just these
 template <bool IN>
-static void launch_links_layout(bq_ctx *c, double2 *lib, double *user) {
-    const unsigned grid = grid_for(c->V, LINK_SITES);
-    if ((uintptr_t)user % sizeof(double2) == 0) k_links_layout<IN, true><<<grid, 256, 0, c->stream>>>(lib, user, c->V);
-    else k_links_layout<IN, false><<<grid, 256, 0, c->stream>>>(lib, user, c->V);
+static void launch_links_layout(bq_ctx *c, double2 *lib, double *user, long long x0, long long n) {
+    const unsigned grid = grid_for(n, LINK_SITES);
+    if ((uintptr_t)user % sizeof(double2) == 0) k_links_layout<IN, true><<<grid, 256, 0, c->stream>>>(lib + x0, user, c->V, n);
+    else k_links_layout<IN, false><<<grid, 256, 0, c->stream>>>(lib + x0, user, c->V, n);
 }
 
 // a caller's BQ_DEVICE links that a kernel of this context can take as they lie: doubles on this device.
 // Others (another device's memory, an address that is no multiple of eight) go through a copy.
-static bool links_direct(const bq_ctx *c, const void *p) {
+bool bq_links_direct(const bq_ctx *c, const void *p) {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
@@ -254,44 +249,92 @@ static bool links_direct(const bq_ctx *c, const void *p) {
            (at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == c->device));
 }
 
-// every link entry split into float pairs (re.hi, im.hi, re.lo, im.lo), exactly but for the last
-// five bits of the low part; normalised, so that the products of two low parts which the sums
-// leave out are below 2^-50 of a term and of either sign (the truncating split alone leaves
-// 2^-48, all of one sign)
-__global__ void __launch_bounds__(256) k_split_links(float4 *dst, const double2 *src, long long n) {
-    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-    if (i >= n) return;
-    const double2 v = src[i];
-    const df a = normalise(df_from_double(v.x)), b = normalise(df_from_double(v.y));
-    dst[i] = make_float4(a.hi, b.hi, a.lo, b.lo);
-}
-
 static size_t link_field_bytes(const bq_ctx *c) { return (size_t)c->V * 36 * sizeof(double2); }
 
-int bq_split_links(bq_ctx *c, const double2 *U, int thin) {
-    if (thin && c->U_pair_thin) return BQ_OK;
-    BQ_TRY(bq_alloc((void **)&c->U_pair, link_field_bytes(c)));
-    k_split_links<<<grid_for(36 * c->V, 256), 256, 0, c->stream>>>(c->U_pair, U, 36 * c->V);
+// every link entry split into float pairs; block y = 0 takes mu = 0 and 1, y = 1 the others
+__global__ void __launch_bounds__(256) k_split_links(float4 *dst, long long gap, const double2 *src, long long n) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i < n) dst[i + blockIdx.y * (n + gap)] = split_entry(src[i + blockIdx.y * n]);
+}
+
+// The split needs 576 bytes a site, but only while staples and leaves are formed. It is put where a field
+// of the context lies that has to be made anew before its next use anyway, so that no memory is held
+// for it: the clover blocks of FP32 or double-float storage, the FP64 or double-float links, or the
+// inverse blocks of the clover master (two of 288 bytes a site, hence the gap). A batch that runs on another
+// stream than the context's may still read such a field: then only what the caller rebuilds now.
+PairLinks bq_split_place(const bq_ctx *c, bool build) {
+    if (c->thin.p) return c->thin;
+    if (!c->read_elsewhere) {
+        for (int p : {(int)BQ_PREC_SINGLE, (int)BQ_PREC_DF64})
+            if (c->clov[p] && !c->clov_valid[p]) return {(const float4 *)c->clov[p], 0};
+        for (int p : {(int)BQ_PREC_DOUBLE, (int)BQ_PREC_DF64})
+            if (c->links[p] && !c->links_valid[p]) return {(const float4 *)c->links[p], 0};
+    }
+    const long long pblk = 36LL * c->Vh;
+    if (c->clov_master && (build || (!c->clov_master_valid && !c->read_elsewhere)))
+        return {(const float4 *)c->clov_master + pblk, pblk};
+    return {nullptr, 0};
+}
+
+int bq_split_links(bq_ctx *c, const double2 *U, PairLinks to, bool keep) {
+    const bool thin = U == c->U_canon;
+    if (thin && to.p == c->thin.p) return BQ_OK;
+    c->thin.p = nullptr;
+    const dim3 grid(grid_for(18 * c->V, 256), 2);
+    k_split_links<<<grid, 256, 0, c->stream>>>(const_cast<float4 *>(to.p), to.gap, U, 18 * c->V);
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
-    c->U_pair_thin = thin;
+    if (thin && keep) c->thin = to;
+    return BQ_OK;
+}
+
+// Links between the caller's memory, where no kernel can reach it (host, another device), and the library's
+// field, in a place where split links could lie (whole) or through a buffer of up to 2^18 sites (151 MB), or
+// less where that does not fit. The context keeps that buffer: allocating it for each call took 0.1 to 0.4 ms,
+// as long as copying the links of a small lattice.
+template <bool IN>
+static int links_through_copies(bq_ctx *c, double2 *lib, double *user, int where) {
+    const PairLinks place = bq_split_place(c, false);
+    double *stage = place.gap ? nullptr : reinterpret_cast<double *>(const_cast<float4 *>(place.p));
+    long long chunk = c->V;
+    if (stage) {
+        c->thin.p = nullptr;
+    } else {
+        if (!c->link_stage) {
+            long long n = c->V < (1LL << 18) ? c->V : (1LL << 18);
+            while (bq_alloc((void **)&c->link_stage, (size_t)n * 72 * sizeof(double)) != BQ_OK) {
+                if (n <= LINK_SITES) return BQ_ERR_NOMEM;
+                n = (n / 2 + LINK_SITES - 1) / LINK_SITES * LINK_SITES;
+            }
+            c->link_stage_sites = n;
+        }
+        stage = c->link_stage;
+        chunk = c->link_stage_sites;
+    }
+    const cudaMemcpyKind kind = where != BQ_HOST ? cudaMemcpyDeviceToDevice : IN ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
+    cudaError_t e = cudaSuccess;
+    for (long long x0 = 0; x0 < c->V && e == cudaSuccess; x0 += chunk) {
+        const long long n = c->V - x0 < chunk ? c->V - x0 : chunk;
+        const size_t bytes = (size_t)n * 72 * sizeof(double);
+        if (IN) e = cudaMemcpyAsync(stage, user + 72 * x0, bytes, kind, c->stream);
+        if (e == cudaSuccess) {
+            launch_links_layout<IN>(c, lib, stage, x0, n);
+            e = cudaGetLastError();
+        }
+        BQ_COUNT(c);
+        if (!IN && e == cudaSuccess) e = cudaMemcpyAsync(user + 72 * x0, stage, bytes, kind, c->stream);
+    }
+    const cudaError_t e2 = cudaStreamSynchronize(c->stream);
+    BQ_CUDA_TRY(e);
+    BQ_CUDA_TRY(e2);
     return BQ_OK;
 }
 
 int bq_links_out(bq_ctx *c, double *dst, const double2 *U, int where) {
-    double *to = dst;
-    const bool copy = where == BQ_HOST || !links_direct(c, dst);
-    if (copy) {
-        BQ_TRY(bq_alloc((void **)&c->U_pair, link_field_bytes(c)));
-        c->U_pair_thin = 0;
-        to = (double *)c->U_pair;
-    }
-    launch_links_layout<false>(c, const_cast<double2 *>(U), to);
+    if (where == BQ_HOST || !bq_links_direct(c, dst)) return links_through_copies<false>(c, const_cast<double2 *>(U), dst, where);
+    launch_links_layout<false>(c, const_cast<double2 *>(U), dst, 0, c->V);
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
-    if (copy)
-        BQ_CUDA_TRY(cudaMemcpyAsync(dst, to, link_field_bytes(c),
-                                    where == BQ_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, c->stream));
     BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
     return BQ_OK;
 }
@@ -302,20 +345,16 @@ extern "C" int bq_set_gauge(bq_ctx *c, const double *U, int where) {
         return BQ_ERR_ARG;
     }
     BQ_TRY(bq_alloc((void **)&c->U_canon, link_field_bytes(c)));
-    double *src = const_cast<double *>(U);
-    c->U_pair_thin = 0;
-    if (where == BQ_HOST || !links_direct(c, U)) {
-        BQ_TRY(bq_alloc((void **)&c->U_pair, link_field_bytes(c)));
-        BQ_CUDA_TRY(cudaMemcpyAsync(c->U_pair, U, link_field_bytes(c),
-                                    where == BQ_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream));
-        src = (double *)c->U_pair;
-    }
-    launch_links_layout<true>(c, c->U_canon, src);
-    BQ_LAUNCH_CHECK();
-    BQ_COUNT(c);
-    if (where == BQ_HOST) BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    c->have_gauge = 1;
+    c->thin.p = nullptr;
     invalidate_derived(c, 1, 1);
+    if (where == BQ_HOST || !bq_links_direct(c, U)) {
+        BQ_TRY(links_through_copies<true>(c, c->U_canon, const_cast<double *>(U), where));
+    } else {
+        launch_links_layout<true>(c, c->U_canon, const_cast<double *>(U), 0, c->V);
+        BQ_LAUNCH_CHECK();
+        BQ_COUNT(c);
+    }
+    c->have_gauge = 1;
     return BQ_OK;
 }
 
@@ -336,7 +375,7 @@ extern "C" int bq_set_u1(bq_ctx *c, const double *A, int where) {
             return BQ_ERR_ARG;
         }
     size_t bytes = (size_t)c->V * 4 * sizeof(double);
-    BQ_TRY(bq_alloc((void **)&c->A_u1, bytes, c));
+    BQ_TRY(bq_alloc((void **)&c->A_u1, bytes));
     BQ_CUDA_TRY(cudaMemcpyAsync(c->A_u1, A, bytes,
                                 where == BQ_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream));
     if (where == BQ_HOST) BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -400,7 +439,7 @@ int bq_prepare_links(bq_ctx *c, int prec) {
         cudaFree(c->links[prec]);
         c->links[prec] = nullptr;
     }
-    BQ_TRY(bq_alloc((void **)&c->links[prec], blk * 8, c));
+    BQ_TRY(bq_alloc((void **)&c->links[prec], blk * 8));
     c->links_recon[prec] = recon;
     Geo g = geo_of(c);
     unsigned grid = grid_for(c->V, 128);
@@ -411,6 +450,7 @@ int bq_prepare_links(bq_ctx *c, int prec) {
         BQ_TRY(bq_prepare_hop_links(c));
         Usrc = c->U_hop;
     }
+    if (c->thin.p == (const float4 *)c->links[prec]) c->thin.p = nullptr;
     if (recon == BQ_RECON_8) BQ_CUDA_TRY(cudaMemsetAsync(c->dev_flag, 0, sizeof(int), c->stream));
 #define PACK(P, ...) k_pack_links<P, __VA_ARGS__><<<grid, 128, 0, c->stream>>>(c->links[prec], blk, Usrc, c->A_u1, q, g, c->dev_flag)
     if (prec == BQ_PREC_DOUBLE) {
@@ -451,7 +491,7 @@ int bq_prepare_links(bq_ctx *c, int prec) {
 // ten products instead of twelve. The loop stays rolled (one partial product, one link and the
 // bracket live, one copy of the product's code). The nine independent reals of F: the imaginary
 // parts of the diagonal, then the three entries above it.
-__device__ __forceinline__ void field_strength(const float4 *P, const Geo &g, long long x, int mu, int nu, double F[9]) {
+__device__ __forceinline__ void field_strength(const PairLinks &P, const Geo &g, long long x, int mu, int nu, double F[9]) {
     const long long V = g.V;
     const long long xpm = lex_step(g, x, mu, +1), xpn = lex_step(g, x, nu, +1);
     const long long xmm = lex_step(g, x, mu, -1), xmn = lex_step(g, x, nu, -1);
@@ -509,7 +549,7 @@ __device__ __forceinline__ void field_strength(const float4 *P, const Geo &g, lo
 #define CLOVER_MIN_BLOCKS 2
 #endif
 __global__ void __launch_bounds__(6 * CLOVER_SITES, CLOVER_MIN_BLOCKS) k_build_clover(double2 *master, size_t pblk,
-                                                                                      const float4 *P, Geo g, double kc) {
+                                                                                      PairLinks P, Geo g, double kc) {
     // planes: 0:(0,1) 1:(0,2) 2:(0,3) 3:(1,2) 4:(1,3) 5:(2,3)
     __shared__ double sF[6][9][CLOVER_SITES];
     const int lane = threadIdx.x % CLOVER_SITES, pl = threadIdx.x / CLOVER_SITES;
@@ -715,15 +755,17 @@ extern "C" int bq_build_clover(bq_ctx *c) {
     }
     c->clov_user = 0;  // building from the links replaces a caller-supplied field
     size_t pblk = (size_t)36 * c->Vh;  // double2 per (parity, inverse) block
-    BQ_TRY(bq_alloc((void **)&c->clov_master, sizeof(double2) * pblk * 4, c));
+    BQ_TRY(bq_alloc((void **)&c->clov_master, sizeof(double2) * pblk * 4));
     Geo g = geo_of(c);
     BQ_CUDA_TRY(cudaMemsetAsync(c->dev_flag, 0, sizeof(int), c->stream));
     const unsigned nblk = (unsigned)((c->V + CLOVER_SITES - 1) / CLOVER_SITES);
-    BQ_TRY(bq_split_links(c, c->U_canon, 1));
-    k_build_clover<<<nblk, 6 * CLOVER_SITES, 0, c->stream>>>((double2 *)c->clov_master, pblk, c->U_pair, g,
+    const PairLinks P = bq_split_place(c, true);
+    BQ_TRY(bq_split_links(c, c->U_canon, P, true));
+    k_build_clover<<<nblk, 6 * CLOVER_SITES, 0, c->stream>>>((double2 *)c->clov_master, pblk, P, g,
                                                              c->params.kappa * c->params.csw);
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
+    if (c->thin.gap) c->thin.p = nullptr;  // the inverse goes where the split links lie
     k_invert_clover<<<grid_for(4LL * c->Vh, 64), 64, 0, c->stream>>>((double2 *)c->clov_master, pblk, c->Vh,
                                                                      c->dev_flag);
     bq_fields_written();
@@ -773,8 +815,9 @@ extern "C" int bq_set_clover(bq_ctx *c, const double *A, int where) {
     }
     c->clov_user = 0;
     invalidate_derived(c, 0, 1);
+    if (c->thin.gap) c->thin.p = nullptr;  // the split links lie in the master's inverse blocks
     const size_t pblk = (size_t)36 * c->Vh;
-    BQ_TRY(bq_alloc((void **)&c->clov_master, sizeof(double2) * pblk * 4, c));
+    BQ_TRY(bq_alloc((void **)&c->clov_master, sizeof(double2) * pblk * 4));
     Geo g = geo_of(c);
     // host data goes through a bounded device staging buffer, 2^20 sites (604 MB) at a time
     const long long chunk = where == BQ_HOST ? (c->V < (1LL << 20) ? c->V : (1LL << 20)) : c->V;
@@ -830,7 +873,8 @@ extern "C" int bq_set_clover(bq_ctx *c, const double *A, int where) {
 int bq_prepare_clover(bq_ctx *c, int prec) {
     if (!c->clov_master_valid) BQ_TRY(bq_build_clover(c));
     if (c->clov_valid[prec]) return BQ_OK;
-    BQ_TRY(bq_alloc((void **)&c->clov[prec], clover_bytes_per_site(prec) * (size_t)c->Vh * 4, c));
+    BQ_TRY(bq_alloc((void **)&c->clov[prec], clover_bytes_per_site(prec) * (size_t)c->Vh * 4));
+    if (c->thin.p == (const float4 *)c->clov[prec]) c->thin.p = nullptr;
     unsigned grid = grid_for(4LL * c->Vh, 128);
     if (prec == BQ_PREC_SINGLE)
         k_convert_clover<BQ_PREC_SINGLE><<<grid, 128, 0, c->stream>>>(c->clov[prec], (const double2 *)c->clov_master, c->Vh, 4);
@@ -905,7 +949,7 @@ extern "C" int bq_spinor_pack(bq_ctx *c, void *native, const double *canon, int 
     }
     const double *src = canon;
     if (where == BQ_HOST) {
-        BQ_TRY(bq_alloc((void **)&c->canon_stage, (size_t)c->Vh * 192, c));
+        BQ_TRY(bq_alloc((void **)&c->canon_stage, (size_t)c->Vh * 192));
         BQ_CUDA_TRY(cudaMemcpyAsync(c->canon_stage, canon, (size_t)c->Vh * 192, cudaMemcpyHostToDevice, c->stream));
         src = c->canon_stage;
     }
@@ -918,7 +962,7 @@ extern "C" int bq_spinor_unpack(bq_ctx *c, double *canon, const void *native, in
         return BQ_ERR_ARG;
     }
     if (where == BQ_DEVICE) return bq_unpack(c, canon, native, prec);
-    BQ_TRY(bq_alloc((void **)&c->canon_stage, (size_t)c->Vh * 192, c));
+    BQ_TRY(bq_alloc((void **)&c->canon_stage, (size_t)c->Vh * 192));
     BQ_TRY(bq_unpack(c, c->canon_stage, native, prec));
     BQ_CUDA_TRY(cudaMemcpyAsync(canon, c->canon_stage, (size_t)c->Vh * 192, cudaMemcpyDeviceToHost, c->stream));
     BQ_CUDA_TRY(cudaStreamSynchronize(c->stream));

@@ -497,8 +497,8 @@ int full_work(bq_ctx *c, int pin, FullWork **out) {
     const size_t b64 = spinor_bytes_per_site(BQ_PREC_DOUBLE) * (size_t)c->Vh;
     const size_t bin = spinor_bytes_per_site(pin) * (size_t)c->Vh;
     char **d64[] = {&w->be, &w->bo, &w->xe, &w->xo, &w->bh, &w->r, &w->to, &w->te, &w->ye};
-    for (auto p : d64) BQ_TRY(bq_alloc((void **)p, b64, c));
-    for (auto p : din) BQ_TRY(bq_alloc((void **)p, bin, c));
+    for (auto p : d64) BQ_TRY(bq_alloc((void **)p, b64));
+    for (auto p : din) BQ_TRY(bq_alloc((void **)p, bin));
     *out = w;
     return BQ_OK;
 }
@@ -769,7 +769,7 @@ extern "C" int bq_trace_samples(bq_ctx *c, int nnoise, const double *const *eta_
     auto alloc = [&](char **p) -> int {
         if (used == pool.size()) {
             char *q = nullptr;
-            BQ_TRY(bq_alloc((void **)&q, b64, c));
+            BQ_TRY(bq_alloc((void **)&q, b64));
             pool.push_back(q);
         }
         *p = pool[used++];

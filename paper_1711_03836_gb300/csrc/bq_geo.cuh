@@ -157,16 +157,32 @@ struct Ldl6 {
 struct M3p {
     float2 hi[9], lo[9];
 };
+// a link entry as (re.hi, im.hi, re.lo, im.lo), exactly but for the last five bits of the low parts;
+// normalised, so that the products of two low parts which the sums leave out are below 2^-50 of a
+// term and of either sign (the truncating split alone leaves 2^-48, all of one sign)
+__device__ __forceinline__ float4 split_entry(double2 v) {
+    const df a = normalise(df_from_double(v.x)), b = normalise(df_from_double(v.y));
+    return make_float4(a.hi, b.hi, a.lo, b.lo);
+}
+// the links of one direction: split beforehand, or split at each use where there was no memory to hold that
+__device__ __forceinline__ const float4 *links_of(const PairLinks &P, long long V, int mu) {
+    return P.p + (long long)mu * 9 * V + (mu >= 2 ? P.gap : 0);
+}
+__device__ __forceinline__ const double2 *links_of(const double2 *U, long long V, int mu) {
+    return U + (long long)mu * 9 * V;
+}
+__device__ __forceinline__ float4 split_entry(float4 v) { return v; }
 // U_mu(lex), or its adjoint
-__device__ __forceinline__ M3p load_link_pair(const float4 *P, long long V, long long lex, int mu, bool dag) {
+template <typename LINKS>
+__device__ __forceinline__ M3p load_link_pair(const LINKS &P, long long V, long long lex, int mu, bool dag) {
     M3p m;
-    const float4 *p = P + (long long)mu * 9 * V + lex;
+    const auto *p = links_of(P, V, mu) + lex;
     const float sg = dag ? -1.0f : 1.0f;
 #pragma unroll
     for (int i = 0; i < 3; i++)
 #pragma unroll
         for (int j = 0; j < 3; j++) {
-            const float4 v = p[(dag ? j * 3 + i : i * 3 + j) * V];
+            const float4 v = split_entry(p[(dag ? j * 3 + i : i * 3 + j) * V]);
             m.hi[i * 3 + j] = make_float2(v.x, sg * v.y);
             m.lo[i * 3 + j] = make_float2(v.z, sg * v.w);
         }

@@ -66,6 +66,13 @@ enum { BQ_NPREC = 3, BQ_NFIELD = 4 };  // field storages: the three precisions +
 
 struct BatchWork;   // defined in the batched solver translation unit
 
+// Links split into float pairs, float4 (re.hi, im.hi, re.lo, im.lo): entry k of U_mu(x) at
+// p[(mu * 9 + k) * V + x], from mu = 2 on `gap` further
+struct PairLinks {
+    const float4 *p;
+    long long gap;
+};
+
 struct bq_ctx {
     int L[4];
     int Vh;
@@ -79,9 +86,8 @@ struct bq_ctx {
     // master fields (FP64, device)
     double2 *U_canon;  // [4][9][V]
     double2 *U_hop;    // stout-smeared copy for the hopping term (stout_iter > 0), same layout
-    float4 *U_pair;    // work field of the size of U_canon: links split into float pairs (same order) while
-                       // staples and leaves are formed, staging of links in the caller's layout otherwise
-    int U_pair_thin;   // U_pair holds the split of U_canon
+    PairLinks thin;    // the field in whose place the split of U_canon lies (bq_split_links; p null: none)
+    int read_elsewhere;  // a batch on another stream has read the derived fields
     int U_hop_valid;
     double stout_rho;
     int stout_iter;
@@ -102,6 +108,8 @@ struct bq_ctx {
     char *tmp_odd[BQ_NPREC];
     char *tmp_even[BQ_NPREC];
     double *canon_stage;           // [Vh][12] complex staging for pack/unpack of host data
+    double *link_stage;            // links of link_stage_sites sites between the caller's memory and the library's
+    long long link_stage_sites;
     double *red_partials;          // block partial sums of reductions
     unsigned int *red_ticket;      // last-block ticket
     int *dev_flag;                 // device error flag (singular clover etc.)
@@ -136,10 +144,16 @@ int bq_time_end(bq_ctx *c, int slot);
 // field preparation (bq_fields.cu)
 int bq_prepare_links(bq_ctx *c, int prec);
 int bq_prepare_clover(bq_ctx *c, int prec);
-int bq_split_links(bq_ctx *c, const double2 *U, int thin);  // U -> U_pair (bq_fields.cu)
+// A place for split links in memory that holds no valid field (p null: there is none), or where the split of
+// U_canon lies already. build: the clover term is about to be built, so that the blocks of its inverse hold nothing.
+PairLinks bq_split_place(const bq_ctx *c, bool build);
+// U split into `to`; keep: `to` is a field of the context, where the split of U_canon may be found again
+int bq_split_links(bq_ctx *c, const double2 *U, PairLinks to, bool keep);
+bool bq_links_direct(const bq_ctx *c, const void *p);  // a kernel can take the caller's links as they lie
 int bq_links_out(bq_ctx *c, double *dst, const double2 *U, int where);  // to the caller's layout
-int bq_prepare_hop_links(bq_ctx *c);  // stout-smeared canonical links of the hopping term (bq_gauge.cu)
-int bq_alloc(void **p, size_t bytes, bq_ctx *c = nullptr);  // c: its work field is given back if memory is short
+// stout-smeared links of the hopping term (bq_gauge.cu); lent: memory of the size of the links to use meanwhile
+int bq_prepare_hop_links(bq_ctx *c, float4 *lent = nullptr);
+int bq_alloc(void **p, size_t bytes);
 int bq_pack(bq_ctx *c, void *native, const double *canon_dev, int prec);
 int bq_unpack(bq_ctx *c, double *canon_dev, const void *native, int prec);
 
