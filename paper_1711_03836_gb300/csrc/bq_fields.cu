@@ -17,7 +17,6 @@
 // errors
 
 static thread_local char g_err[512] = "";
-thread_local int bq_plain_next = 0;
 
 void bq_set_error(const char *fmt, ...) {
     va_list ap;
@@ -425,6 +424,16 @@ __global__ void k_pack_links(char *dst, size_t blk, const double2 *U, const doub
     }
 }
 
+// An empty kernel, launched in the ordinary way, so that it starts when the kernels before it have ended:
+// a launch with programmatic dependence on it can only start after that.
+__global__ void k_fields_written() {}
+int bq_fields_written(bq_ctx *c) {
+    k_fields_written<<<1, 1, 0, c->stream>>>();
+    BQ_LAUNCH_CHECK();
+    BQ_COUNT(c);
+    return BQ_OK;
+}
+
 int bq_prepare_links(bq_ctx *c, int prec) {
     if (!c->have_gauge) {
         bq_set_error("gauge field not set");
@@ -463,9 +472,9 @@ int bq_prepare_links(bq_ctx *c, int prec) {
         if (rebuild) PACK(BQ_PREC_DF64, 18, true); else PACK(BQ_PREC_DF64, 18);
     }
 #undef PACK
-    bq_fields_written();
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
+    BQ_TRY(bq_fields_written(c));
     if (recon == BQ_RECON_8) {
         int flag = 0;
         BQ_CUDA_TRY(cudaMemcpyAsync(&flag, c->dev_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -768,7 +777,6 @@ extern "C" int bq_build_clover(bq_ctx *c) {
     if (c->thin.gap) c->thin.p = nullptr;  // the inverse goes where the split links lie
     k_invert_clover<<<grid_for(4LL * c->Vh, 64), 64, 0, c->stream>>>((double2 *)c->clov_master, pblk, c->Vh,
                                                                      c->dev_flag);
-    bq_fields_written();
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
     int flag = 0;
@@ -861,7 +869,6 @@ extern "C" int bq_set_clover(bq_ctx *c, const double *A, int where) {
         bq_set_error("bq_set_clover: a clover block of the field has no inverse");
         return BQ_ERR_CLOVER_SINGULAR;
     }
-    bq_fields_written();
     c->clov_user = 1;
     c->clov_master_valid = 1;
     c->clov[BQ_PREC_DOUBLE] = (char *)c->clov_master;
@@ -882,9 +889,9 @@ int bq_prepare_clover(bq_ctx *c, int prec) {
         k_convert_clover<BQ_PREC_DF64><<<grid, 128, 0, c->stream>>>(c->clov[prec], (const double2 *)c->clov_master, c->Vh, 4);
     else
         k_convert_clover<BQ_PREC_HALF><<<grid, 128, 0, c->stream>>>(c->clov[prec], (const double2 *)c->clov_master, c->Vh, 4);
-    bq_fields_written();
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
+    BQ_TRY(bq_fields_written(c));
     c->clov_valid[prec] = 1;
     return BQ_OK;
 }

@@ -37,11 +37,9 @@ void bq_set_error(const char *fmt, ...);
 // 24.6 -> 15.4 us, 20^3x40 112.6 -> 102.7 us); inside a captured graph 0.2 us. The kernels do
 // not ask for an earlier start (griddepcontrol.launch_dependents): blocks that then wait on
 // the SMs of the running kernel leave an uneven distribution behind (FP64, 12^4: 158 -> 307 us).
-// Fields written by a kernel that was not launched this way (link and clover packing) are read
-// through the read-only path, so the first launch after one is a plain one:
-// bq_fields_written() asks for that.
-extern thread_local int bq_plain_next;
-inline void bq_fields_written() { bq_plain_next = 1; }
+// Links and clover blocks are read through the read-only path, whose loads may be scheduled ahead
+// of bq_pdl_enter(): after the kernels that write them, bq_fields_written() keeps every later
+// launch, by whichever context or thread, behind their end.
 template <typename... P, typename... A>
 inline void bq_launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args) {
     cudaLaunchAttribute at;
@@ -52,8 +50,7 @@ inline void bq_launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStrea
     cfg.blockDim = dim3(block);
     cfg.stream = s;
     cfg.attrs = &at;
-    cfg.numAttrs = bq_plain_next ? 0 : 1;
-    bq_plain_next = 0;
+    cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // the caller reads cudaGetLastError()
 }
 
@@ -144,6 +141,7 @@ int bq_time_end(bq_ctx *c, int slot);
 // field preparation (bq_fields.cu)
 int bq_prepare_links(bq_ctx *c, int prec);
 int bq_prepare_clover(bq_ctx *c, int prec);
+int bq_fields_written(bq_ctx *c);  // see bq_launch
 // A place for split links in memory that holds no valid field (p null: there is none), or where the split of
 // U_canon lies already. build: the clover term is about to be built, so that the blocks of its inverse hold nothing.
 PairLinks bq_split_place(const bq_ctx *c, bool build);
