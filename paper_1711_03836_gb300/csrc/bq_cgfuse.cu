@@ -41,25 +41,21 @@ __device__ __forceinline__ void block_partials(float (&v)[NV], double *partials,
             partials[k * stride + at] = (double)(((ws[k][0] + ws[k][1]) + ws[k][2]) + ws[k][3]);
 }
 
-// The same for the block-interleaved batch, whose sums were FP64 before they moved into the hopping
-// launches: the warp and block sums run in double-float (48 bits; the FP64 pipe would take a 5-step
-// chain of 64-cycle additions per warp and value).
+// The same in FP64 (batches in the block-interleaved mapping, whose sums run in FP64 as in their separate
+// kernels): one warp per value reads the block's 128 terms from shared memory, eight FP64 additions
+// in place of the twenty that five shuffle steps in each of the four warps would take.
 template <int NV>
-__device__ __forceinline__ void block_partials_df(float (&v)[NV], double *partials, int stride, int at) {
-    __shared__ df ws[NV][4];
+__device__ __forceinline__ void block_partials_fp64(const float (&v)[NV], double *partials, int stride, int at) {
+    __shared__ float sv[NV][128];
     const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-        df t(v[k], 0.0f);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            t = t + df(__shfl_xor_sync(0xffffffffu, t.hi, o), __shfl_xor_sync(0xffffffffu, t.lo, o));
-        if (lane == 0) ws[k][wid] = t;
-    }
+    for (int k = 0; k < NV; k++) sv[k][threadIdx.x] = v[k];
     __syncthreads();
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int k = 0; k < NV; k++) partials[k * stride + at] = df_to_double(((ws[k][0] + ws[k][1]) + ws[k][2]) + ws[k][3]);
+    if (wid < NV) {
+        const float *q = sv[wid] + lane;
+        const double s = warp_sum(((double)q[0] + (double)q[32]) + ((double)q[64] + (double)q[96]));
+        if (lane == 0) partials[wid * stride + at] = s;
+    }
 }
 
 // the solver scalars from the block partials of a fused launch (one block of CG_FIN_THREADS)
@@ -88,8 +84,10 @@ struct CgVec {
     const double *scal;
 };
 
-// One site of a fused step, its terms of the sums in v. PN: sum |p|^2 in the Mhat step (a nonzero shift)
-template <int PS, int RECON, int MODE, bool PN>
+// One site of a fused step, its terms of the sums in v. PN: sum |p|^2 in the Mhat step (a nonzero shift).
+// TR: FP16 t enters <p, Mhat^dag t_r> = <t, t_r> as it is stored (t_r), which is what the next step applies
+// Mhat^dag to; else |t|^2 before rounding.
+template <int PS, int RECON, int MODE, bool PN, bool TR>
 __device__ __forceinline__ void cg_site(const DslashArgs &a, const CgVec &vec, const int h,
                                         float (&v)[MODE == CNT_CG_MHAT ? 2 : 1]) {
     using T = typename Traits<PS>::real;
@@ -113,8 +111,19 @@ __device__ __forceinline__ void cg_site(const DslashArgs &a, const CgVec &vec, c
         xpay_site<PS>(a, vec.xin, h, acc, xv, o);
         SpinorIO<PS>::store(vec.out, h, a.Vh, o);
         float n0 = 0.f, n1 = 0.f;
+        if constexpr (TR) {
+            float inv;
+            const float m = SpinorIO<PS>::scale(o, inv);
 #pragma unroll
-        for (int c = 0; c < 12; c++) n0 += o[c].re * o[c].re + o[c].im * o[c].im;
+            for (int c = 0; c < 12; c++) {
+                const float2 r = h2f(f2h(o[c].re * inv, o[c].im * inv));
+                n0 += o[c].re * r.x + o[c].im * r.y;
+            }
+            n0 *= m;
+        } else {
+#pragma unroll
+            for (int c = 0; c < 12; c++) n0 += o[c].re * o[c].re + o[c].im * o[c].im;
+        }
         if (PN)
 #pragma unroll
             for (int c = 0; c < 12; c++) n1 += xv[c].re * xv[c].re + xv[c].im * xv[c].im;
@@ -213,7 +222,7 @@ __global__ void __launch_bounds__(128, DslashMinBlocks<PS>::value) k_dslash_cg(c
     float v[NV];
 #pragma unroll
     for (int k = 0; k < NV; k++) v[k] = 0.f;
-    if (h < a.Vh) cg_site<PS, RECON, MODE, PN>(a, CgVec{a.in, a.xin, f.p, a.out, f.xs, f.rs, f.scal}, h, v);
+    if (h < a.Vh) cg_site<PS, RECON, MODE, PN, false>(a, CgVec{a.in, a.xin, f.p, a.out, f.xs, f.rs, f.scal}, h, v);
     block_partials(v, f.partials, gridDim.x, blockIdx.x);
 }
 
@@ -236,9 +245,9 @@ __global__ void __launch_bounds__(128, DslashMinBlocks<PS>::value) k_dslash_batc
 #pragma unroll
     for (int k = 0; k < NV; k++) v[k] = 0.f;
     if (h < U.a.Vh)
-        cg_site<PS, RECON, MODE, true>(
+        cg_site<PS, RECON, MODE, true, true>(
             U.a, CgVec{U.in[r], U.xin[r], sv.p, U.out[r], sv.xs, sv.rs, cg.scal + (size_t)sys * S_NSCAL}, h, v);
-    block_partials_df(v, cg.partials + (size_t)sys * 2 * cg.pstride, cg.pstride, blk);
+    block_partials_fp64(v, cg.partials + (size_t)sys * 2 * cg.pstride, cg.pstride, blk);
 }
 
 template <int PS, int RECON>

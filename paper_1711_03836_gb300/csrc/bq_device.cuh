@@ -230,13 +230,19 @@ struct SpinorIO<BQ_PREC_HALF> {
             s[4 * k + 3] = {d.x, d.y};
         }
     }
-    __device__ static __forceinline__ void store(void *base, int h, int Vh, const cplx<T> s[12]) {
-        uint4 *p = static_cast<uint4 *>(base);
-        float *nrm = reinterpret_cast<float *>(p + (size_t)3 * Vh);
+    // the scale of a site that is stored, and the factor of its components before rounding
+    __device__ static __forceinline__ float scale(const cplx<T> s[12], float &inv) {
         float m = 0.f;
 #pragma unroll
         for (int c = 0; c < 12; c++) m = fmaxf(m, fmaxf(fabsf(s[c].re), fabsf(s[c].im)));
-        float inv = (m > 0.f) ? 1.0f / m : 0.f;
+        inv = (m > 0.f) ? 1.0f / m : 0.f;
+        return m;
+    }
+    __device__ static __forceinline__ void store(void *base, int h, int Vh, const cplx<T> s[12]) {
+        uint4 *p = static_cast<uint4 *>(base);
+        float *nrm = reinterpret_cast<float *>(p + (size_t)3 * Vh);
+        float inv;
+        const float m = scale(s, inv);
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             uint4 v;
