@@ -641,11 +641,23 @@ struct SpinorIO<BQ_PREC_DF64> {
     }
 };
 
-// df64 links: each complex entry as float4 (re.hi, re.lo, im.hi, im.lo), [entry][Vh]
+// d = hi + lo with hi = (float)d and lo = (float)(d - hi): the double's bits rounded to 24 as an integer (ties to
+// even), lo the signed rest of its low 29 bits times hi's power of two. Integer operations in hi's normal range:
+// the two conversions and the subtraction took most of the time of packing double-float fields on the FP64 pipe.
 __device__ __forceinline__ void df_split(double d, float &hi, float &lo) {
-    hi = __double2float_rn(d);
-    lo = __double2float_rn(d - (double)hi);
+    const unsigned h32 = (unsigned)__double2hiint(d), l32 = (unsigned)__double2loint(d);
+    const unsigned a = h32 & 0x7fffffffu, sign = h32 & 0x80000000u;
+    if (a - (897u << 20) >= (253u << 20)) {  // zero, a subnormal float, at or beyond 2^127, not finite
+        hi = __double2float_rn(d);
+        lo = __double2float_rn(d - (double)hi);
+        return;
+    }
+    const unsigned t = __funnelshift_l(l32, a - (896u << 20), 3);
+    const int low = (int)(l32 & 0x1fffffffu), up = low + (int)(t & 1u) > (1 << 28);
+    hi = __uint_as_float((t + up) | sign);
+    lo = __fmul_rn(__fmul_rn(__int2float_rn(low - (up << 29)), 0x1p-52f), __uint_as_float((t & 0x7f800000u) | sign));
 }
+// df64 links: each complex entry as float4 (re.hi, re.lo, im.hi, im.lo), [entry][Vh]
 
 template <int RECON>
 struct LinkIO<BQ_PREC_DF64, RECON> {
