@@ -517,7 +517,8 @@ static int build_units(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int ma
             DslashUnit *u = &tab.units[tab.nunits];
             BQ_TRY(bq_dslash_unit_fill(c, prec, parity, dagger, epi, kk, &u->a));
             u->nr = e - s;
-            u->a.rev = bq_reverse(prec, BQ_RECON_12, epi, c->Vh, u->nr);
+            const int recon = c->links_recon[(prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) ? 3 : prec];
+            u->a.rev = bq_reverse(prec, recon, epi, c->Vh, u->nr);  // the working set of nr right-hand sides
             u->log2R = log2_ceil(u->nr);
             u->interleave = m == -1 ? 1 : m == -2 ? 2 : m <= -3 ? 3 : 0;
             if (prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) {
@@ -554,7 +555,6 @@ static int build_units(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int ma
             tab.block0[tab.nunits + 1] = tab.block0[tab.nunits] + blocks;
             tab.nunits++;
             // links and clover once per site of the unit, spinors per rhs
-            const int recon = c->links_recon[(prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) ? 3 : prec];
             const double shared = 8.0 * link_bytes_per_link(prec, recon) + clover_bytes_per_site(prec);
             const double per_rhs = dslash_site_bytes(prec, recon, epi) - shared;
             bytes += (shared + per_rhs * u->nr) * (double)c->Vh;

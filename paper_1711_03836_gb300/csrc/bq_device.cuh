@@ -307,10 +307,11 @@ __device__ __forceinline__ void reconstruct8(cplx<float> U[9], cplx<float> a1, c
 template <int PREC, int RECON>
 struct LinkIO;
 
-template <int RECON>
-struct LinkIO<BQ_PREC_DOUBLE, RECON> {
+// FP64 links (and their double-float split) are stored with all 18 reals
+template <>
+struct LinkIO<BQ_PREC_DOUBLE, BQ_RECON_18> {
     using T = double;
-    static constexpr int NC = (RECON == 12) ? 6 : 9;
+    static constexpr int NC = 9;
     __device__ static __forceinline__ void load(cplx<T> U[9], const char *blk, int h, int Vh) {
         const double2 *p = reinterpret_cast<const double2 *>(blk);
 #pragma unroll
@@ -318,7 +319,6 @@ struct LinkIO<BQ_PREC_DOUBLE, RECON> {
             double2 v = ldg(p + (size_t)c * Vh + h);
             U[c] = {v.x, v.y};
         }
-        if (RECON == 12) reconstruct_row2(U);
     }
     __device__ static __forceinline__ void store(char *blk, int h, int Vh, const double2 U[9]) {
         double2 *p = reinterpret_cast<double2 *>(blk);
@@ -659,23 +659,12 @@ __device__ __forceinline__ void df_split(double d, float &hi, float &lo) {
 }
 // df64 links: each complex entry as float4 (re.hi, re.lo, im.hi, im.lo), [entry][Vh]
 
-template <int RECON>
-struct LinkIO<BQ_PREC_DF64, RECON> {
-    using T = df;
-    static constexpr int NC = (RECON == 12) ? 6 : 9;
-    __device__ static __forceinline__ void load(cplx<T> U[9], const char *blk, int h, int Vh) {
-        const float4 *p = reinterpret_cast<const float4 *>(blk);
-#pragma unroll
-        for (int c = 0; c < NC; c++) {
-            float4 v = ldg(p + (size_t)c * Vh + h);
-            U[c] = {df(v.x, v.y), df(v.z, v.w)};
-        }
-        if (RECON == 12) reconstruct_row2(U);
-    }
+template <>
+struct LinkIO<BQ_PREC_DF64, BQ_RECON_18> {  // loaded an entry at a time by the lane-pair kernels
     __device__ static __forceinline__ void store(char *blk, int h, int Vh, const double2 U[9]) {
         float4 *p = reinterpret_cast<float4 *>(blk);
 #pragma unroll
-        for (int c = 0; c < NC; c++) {
+        for (int c = 0; c < 9; c++) {
             float4 v;
             df_split(U[c].x, v.x, v.y);
             df_split(U[c].y, v.z, v.w);

@@ -77,7 +77,7 @@ double dslash_site_flops(int epi) { return 1320.0 + (epi != EPI_PLAIN ? 504.0 : 
 
 // links (both parities) and the two clover fields of an operator application against L2
 static bool fields_exceed_l2(const DslashArgs &a, int recon) {
-    return (double)a.Vh * (8.0 * link_bytes_per_link(BQ_PREC_SINGLE, recon) + 2.0 * clover_bytes_per_site(BQ_PREC_SINGLE)) > 129e6;
+    return (double)a.Vh * (8.0 * link_bytes_per_link(BQ_PREC_SINGLE, recon) + 2.0 * clover_bytes_per_site(BQ_PREC_SINGLE)) > BQ_L2_BYTES;
 }
 
 template <int PREC, int RECON, bool STREAM>

@@ -19,6 +19,6 @@ void bq_pair64_launch(const DslashArgs &a, bool dag, int epi, cudaStream_t s);
 // 45 / 108 us FP64; 4096 27 / 30, 27 / 31, 66 / 109; 10368 35 / 31, 35 / 32, 143 / 133 (beyond,
 // the shared-memory exchange and the half-width loads cost more than the idle SMs).
 static inline bool bq_use_split(const bq_ctx *c, int prec) {
-    if (prec == BQ_PREC_DOUBLE) return c->fp64_arith == BQ_FP64_NATIVE && c->Vh <= 16 * 152 * 3;
-    return c->Vh <= 16 * 152 * 2;
+    if (prec == BQ_PREC_DOUBLE) return c->fp64_arith == BQ_FP64_NATIVE && c->Vh <= 16 * BQ_SMS * 3;
+    return c->Vh <= 16 * BQ_SMS * 2;
 }

@@ -262,10 +262,6 @@ template <>
 struct DslashMinBlocks<BQ_PREC_HALF> {
     static constexpr int value = HALF_MIN_BLOCKS;
 };
-template <>
-struct DslashMinBlocks<BQ_PREC_DOUBLE> {  // FP64-unit bound: no cap
-    static constexpr int value = 1;
-};
 // STREAM (FP32): where links and clover of an application exceed L2 (129 MB). 24^3x48 180 -> 176 us,
 // 32^3x64 538 -> 534 us, 48^3x96 with 18-real links 3367 -> 3241 us; L2-resident 16^3x32 31.1 -> 32.3 us.
 template <int PREC, int RECON, bool DAG, int EPI, bool STREAM>
