@@ -500,7 +500,7 @@ static int build_units(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int ma
         const int epi = parity == 1 ? EPI_CLOVINV : EPI_XPAY;
         std::vector<DslashBatchTable> &tabs = w->tables[step];
         tabs.clear();
-        double bytes = 0, flops = 0;
+        double bytes = 0, flops = 0, wset = 0;
         int s = 0;
         while (s < nsys) {
             if (tabs.empty() || tabs.back().nunits == DSLASH_MAX_UNITS) {
@@ -519,6 +519,7 @@ static int build_units(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int ma
             u->nr = e - s;
             const int recon = c->links_recon[(prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) ? 3 : prec];
             u->a.rev = bq_reverse(prec, recon, epi, c->Vh, u->nr);  // the working set of nr right-hand sides
+            wset += bq_working_set(prec, recon, c->Vh, u->nr);
             u->log2R = log2_ceil(u->nr);
             u->interleave = m == -1 ? 1 : m == -2 ? 2 : m <= -3 ? 3 : 0;
             if (prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) {
@@ -561,6 +562,7 @@ static int build_units(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int ma
             flops += dslash_site_flops(epi) * u->nr * (double)c->Vh;
             s = e;
         }
+        for (DslashBatchTable &t : tabs) t.stream = wset > BQ_L2_BYTES;
         plan->bytes_all[step] = bytes;
         plan->flops_all[step] = flops;
     }

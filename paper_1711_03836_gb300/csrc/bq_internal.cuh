@@ -170,15 +170,21 @@ inline size_t links_block_bytes(const bq_ctx *c, int prec) {
 constexpr double BQ_L2_BYTES = 129e6;
 constexpr int BQ_SMS = 152;
 
+// what an operator application on nr right-hand sides goes through: links, both clover fields and four
+// spinors per right-hand side
+inline double bq_working_set(int prec, int recon, int Vh, int nr) {
+    return (double)Vh * (8.0 * link_bytes_per_link(prec, recon) + 2.0 * clover_bytes_per_site(prec) +
+                         4.0 * nr * spinor_bytes_per_site(prec));
+}
+
 // The launches of an operator alternate their direction over the lattice where its working set
-// (links, both clover fields, four spinors per right-hand side) exceeds L2, except in the shared-memory tiles
+// exceeds L2, except in the shared-memory tiles
 // (slower there, bq_tile.cu): the A x - k D step goes from the last site to the first, so that it starts with the part of its input that the D_oe step
 // wrote last and L2 still holds. FP32 Mhat^dag Mhat 24^3x48 191 -> 180 us, 32^3x64 549 -> 538 us, CG
 // iteration 242 -> 230 and 676 -> 664 us; a lattice that fits loses (16^3x32 CG 47.3 -> 49.5 us: its
 // sites change the die between launches).
 inline int bq_reverse(int prec, int recon, int epi, int Vh, int nr) {
-    return epi == EPI_XPAY && (double)Vh * (8.0 * link_bytes_per_link(prec, recon) + 2.0 * clover_bytes_per_site(prec) +
-                                            4.0 * nr * spinor_bytes_per_site(prec)) > BQ_L2_BYTES;
+    return epi == EPI_XPAY && bq_working_set(prec, recon, Vh, nr) > BQ_L2_BYTES;
 }
 
 // one unit of a batched hopping-term launch: a lattice (fields, geometry and
@@ -206,6 +212,7 @@ enum { DSLASH_MAX_UNITS = 16 };
 struct DslashBatchTable {
     int nunits;
     int variant;  // shared-memory tile units: resident blocks per SM the kernel is compiled for (4, 5, 6)
+    int stream;   // and whether FP32 links and clover blocks are staged past L1 (see stage_links)
     int block0[DSLASH_MAX_UNITS + 1];  // first block of each unit; block0[nunits] = grid size
     DslashUnit units[DSLASH_MAX_UNITS];
 };

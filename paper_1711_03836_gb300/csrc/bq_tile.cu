@@ -125,10 +125,12 @@ __device__ __forceinline__ void tile_clover_block(float d[6], cplx<float> o[15],
 }
 
 // the eight links of the tile's sites (forward: U_mu(x) of the output parity;
-// backward: U_mu(x - mu) of the other parity), reconstructed / converted to FP32; FP32 links and
-// clover blocks, staged once per tile, are loaded without a place in L1, which the spinors keep
-// (12 right-hand sides, 24^3x48: 1234 -> 1220 us)
-template <int PREC, int RECON>
+// backward: U_mu(x - mu) of the other parity), reconstructed / converted to FP32. STREAM (FP32): links
+// and clover blocks, staged once per tile, are loaded without a place in L1, which the spinors keep, where
+// the batch's working set exceeds L2 (12 right-hand sides, 24^3x48: 1234 -> 1220 us). Below that it costs:
+// a CG iteration of 2 / 4 / 8 systems at 12^3x24 72 / 86 / 141 us with it off, 82 / 96 / 147 with it on;
+// the lines cross at V/2 = 57 000, 47 000 and 28 000, at 98, 117 and 113 MB.
+template <int PREC, int RECON, bool STREAM>
 __device__ __forceinline__ void stage_links(float4 *sL, const DslashArgs &a, int h0) {
     const char *Lo = a.links + (size_t)a.parity * 4 * a.lblk;
     const char *Li = a.links + (size_t)(1 - a.parity) * 4 * a.lblk;
@@ -139,7 +141,7 @@ __device__ __forceinline__ void stage_links(float4 *sL, const DslashArgs &a, int
         if (h < a.Vh) {
             int hl = h;
             if (d & 1) hl = site_neighbours(a, h).hn[d];
-            if constexpr (PREC == BQ_PREC_SINGLE && RECON != BQ_RECON_8)
+            if constexpr (STREAM)
                 LinkIO<PREC, RECON>::template load<true>(U, ((d & 1) ? Li : Lo) + (size_t)mu * a.lblk, hl, a.Vh);
             else
                 LinkIO<PREC, RECON>::load(U, ((d & 1) ? Li : Lo) + (size_t)mu * a.lblk, hl, a.Vh);
@@ -156,7 +158,7 @@ __device__ __forceinline__ void stage_links(float4 *sL, const DslashArgs &a, int
     }
 }
 
-template <int PREC>
+template <int PREC, bool STREAM>
 __device__ __forceinline__ void stage_clover(float4 *sC, const void *clov, int h0, int Vh) {
     for (int i = threadIdx.x; i < 18 * TILE_SITES; i += blockDim.x) {
         const int k = i / TILE_SITES, lane = i % TILE_SITES;
@@ -164,7 +166,7 @@ __device__ __forceinline__ void stage_clover(float4 *sC, const void *clov, int h
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (h < Vh) {
             if constexpr (PREC == BQ_PREC_SINGLE) {
-                v = ldg_once<true>(static_cast<const float4 *>(clov) + (size_t)k * Vh + h);
+                v = ldg_once<STREAM>(static_cast<const float4 *>(clov) + (size_t)k * Vh + h);
             } else {
                 const uint2 u = ldg(static_cast<const uint2 *>(clov) + (size_t)k * Vh + h);
                 const float2 lo = h2f(u.x), hi = h2f(u.y);
@@ -370,7 +372,7 @@ __device__ __forceinline__ void dslash_site_tile(const DslashArgs &a, const Site
 
 // MB: resident 128-thread blocks per SM the kernel is compiled for (registers
 // per thread 128, 96 or 80); the autotuner picks among the variants
-template <int PREC, int RECON, bool DAG, int EPI, int MB, int CGM = 0>
+template <int PREC, int RECON, bool DAG, int EPI, int MB, bool STREAM, int CGM = 0>
 __global__ void __launch_bounds__(128, MB) k_dslash_tile(const __grid_constant__ DslashBatchTable tab,
                                                          const double *mask, const BatchCg cg) {
     bq_pdl_enter();
@@ -387,8 +389,8 @@ __global__ void __launch_bounds__(128, MB) k_dslash_tile(const __grid_constant__
         for (int r = 0; r < U.nr; r++) any = any || mask[U.sys[r]] != 0.0;
         if (!any) return;
     }
-    stage_links<PREC, RECON>(sL, U.a, h0);
-    if (EPI != EPI_PLAIN) stage_clover<PREC>(sC, U.a.clov, h0, U.a.Vh);
+    stage_links<PREC, RECON, STREAM>(sL, U.a, h0);
+    if (EPI != EPI_PLAIN) stage_clover<PREC, STREAM>(sC, U.a.clov, h0, U.a.Vh);
     __syncthreads();
     const int lane = (int)(threadIdx.x & 31), warp = (int)(threadIdx.x >> 5), nw = (int)(blockDim.x >> 5);
     const int h = h0 + lane;
@@ -415,27 +417,35 @@ __global__ void __launch_bounds__(128, MB) k_dslash_tile(const __grid_constant__
     }
 }
 
-template <int PREC, int RECON, int MB>
+template <int PREC, int RECON, int MB, bool STREAM>
 static void launch_tile_mb(const DslashBatchTable &tab, const double *mask, int nblocks, bool dag, int epi,
                            cudaStream_t s) {
     const BatchCg none{};
     if (dag) {
-        if (epi == EPI_CLOVINV) bq_launch(k_dslash_tile<PREC, RECON, true, EPI_CLOVINV, MB>, nblocks, 128, s, tab, mask, none);
-        else bq_launch(k_dslash_tile<PREC, RECON, true, EPI_XPAY, MB>, nblocks, 128, s, tab, mask, none);
+        if (epi == EPI_CLOVINV) bq_launch(k_dslash_tile<PREC, RECON, true, EPI_CLOVINV, MB, STREAM>, nblocks, 128, s, tab, mask, none);
+        else bq_launch(k_dslash_tile<PREC, RECON, true, EPI_XPAY, MB, STREAM>, nblocks, 128, s, tab, mask, none);
     } else {
-        if (epi == EPI_CLOVINV) bq_launch(k_dslash_tile<PREC, RECON, false, EPI_CLOVINV, MB>, nblocks, 128, s, tab, mask, none);
-        else bq_launch(k_dslash_tile<PREC, RECON, false, EPI_XPAY, MB>, nblocks, 128, s, tab, mask, none);
+        if (epi == EPI_CLOVINV) bq_launch(k_dslash_tile<PREC, RECON, false, EPI_CLOVINV, MB, STREAM>, nblocks, 128, s, tab, mask, none);
+        else bq_launch(k_dslash_tile<PREC, RECON, false, EPI_XPAY, MB, STREAM>, nblocks, 128, s, tab, mask, none);
     }
 }
 
 // batched units carry the clover epilogues only (the solvers and the batched
 // apply run D_oe A_oo^-1 and A x - k D_eo steps); tab.variant = resident blocks
+template <int PREC, int RECON, bool STREAM>
+static void launch_tile_v(const DslashBatchTable &tab, const double *mask, int nblocks, bool dag, int epi,
+                          cudaStream_t s) {
+    if (tab.variant == 6) launch_tile_mb<PREC, RECON, 6, STREAM>(tab, mask, nblocks, dag, epi, s);
+    else if (tab.variant == 5) launch_tile_mb<PREC, RECON, 5, STREAM>(tab, mask, nblocks, dag, epi, s);
+    else launch_tile_mb<PREC, RECON, 4, STREAM>(tab, mask, nblocks, dag, epi, s);
+}
 template <int PREC, int RECON>
 static void launch_tile_pr(const DslashBatchTable &tab, const double *mask, int nblocks, bool dag, int epi,
                            cudaStream_t s) {
-    if (tab.variant == 6) launch_tile_mb<PREC, RECON, 6>(tab, mask, nblocks, dag, epi, s);
-    else if (tab.variant == 5) launch_tile_mb<PREC, RECON, 5>(tab, mask, nblocks, dag, epi, s);
-    else launch_tile_mb<PREC, RECON, 4>(tab, mask, nblocks, dag, epi, s);
+    if constexpr (PREC == BQ_PREC_SINGLE && RECON != BQ_RECON_8) {
+        if (tab.stream) return launch_tile_v<PREC, RECON, true>(tab, mask, nblocks, dag, epi, s);
+    }
+    launch_tile_v<PREC, RECON, false>(tab, mask, nblocks, dag, epi, s);
 }
 
 void bq_tile_launch(int prec, int recon, const DslashBatchTable &tab, const double *mask, int nblocks, bool dag,
@@ -454,24 +464,32 @@ void bq_tile_launch(int prec, int recon, const DslashBatchTable &tab, const doub
 // --------------------------------------------------------------------------
 // CG-fused A x - k D steps of an FP32 batch in the tile mapping
 
-template <int PREC, int RECON, int MB>
+template <int PREC, int RECON, int MB, bool STREAM>
 static void launch_tile_cg_mb(const DslashBatchTable &tab, const double *mask, int nblocks, int mode,
                               const BatchCg &cg, cudaStream_t s) {
     if (mode == CNT_CG_MHAT)
-        k_dslash_tile<PREC, RECON, false, EPI_XPAY, MB, CNT_CG_MHAT><<<nblocks, 128, 0, s>>>(tab, mask, cg);
+        k_dslash_tile<PREC, RECON, false, EPI_XPAY, MB, STREAM, CNT_CG_MHAT><<<nblocks, 128, 0, s>>>(tab, mask, cg);
     else
-        k_dslash_tile<PREC, RECON, true, EPI_XPAY, MB, CNT_CG_MHATDAG><<<nblocks, 128, 0, s>>>(tab, mask, cg);
+        k_dslash_tile<PREC, RECON, true, EPI_XPAY, MB, STREAM, CNT_CG_MHATDAG><<<nblocks, 128, 0, s>>>(tab, mask, cg);
 }
 
-template <int PREC, int RECON>
-static void launch_tile_cg_r(const DslashBatchTable &tab, const double *mask, int nblocks, int mode, const BatchCg &cg,
+template <int PREC, int RECON, bool STREAM>
+static void launch_tile_cg_v(const DslashBatchTable &tab, const double *mask, int nblocks, int mode, const BatchCg &cg,
                              cudaStream_t s) {
     // FP16 t with its norms needs the whole site in registers: at 80 registers (six blocks)
     // it spills about 200 bytes, so that step runs with five at most
     const int mb = (PREC == BQ_PREC_HALF && mode == CNT_CG_MHAT && tab.variant == 6) ? 5 : tab.variant;
-    if (mb == 6) launch_tile_cg_mb<PREC, RECON, 6>(tab, mask, nblocks, mode, cg, s);
-    else if (mb == 5) launch_tile_cg_mb<PREC, RECON, 5>(tab, mask, nblocks, mode, cg, s);
-    else launch_tile_cg_mb<PREC, RECON, 4>(tab, mask, nblocks, mode, cg, s);
+    if (mb == 6) launch_tile_cg_mb<PREC, RECON, 6, STREAM>(tab, mask, nblocks, mode, cg, s);
+    else if (mb == 5) launch_tile_cg_mb<PREC, RECON, 5, STREAM>(tab, mask, nblocks, mode, cg, s);
+    else launch_tile_cg_mb<PREC, RECON, 4, STREAM>(tab, mask, nblocks, mode, cg, s);
+}
+template <int PREC, int RECON>
+static void launch_tile_cg_r(const DslashBatchTable &tab, const double *mask, int nblocks, int mode, const BatchCg &cg,
+                             cudaStream_t s) {
+    if constexpr (PREC == BQ_PREC_SINGLE && RECON != BQ_RECON_8) {
+        if (tab.stream) return launch_tile_cg_v<PREC, RECON, true>(tab, mask, nblocks, mode, cg, s);
+    }
+    launch_tile_cg_v<PREC, RECON, false>(tab, mask, nblocks, mode, cg, s);
 }
 
 template <int PREC>
