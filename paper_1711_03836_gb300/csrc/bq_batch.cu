@@ -739,6 +739,21 @@ static unsigned long long fnv(unsigned long long h, const void *p, size_t n) {
 // --------------------------------------------------------------------------
 // the batched solver core
 
+// Whether the vector work of CG rides on the A x - k D launches of a batch in a tile mapping or
+// block-interleaved (sum_vh: sites of all systems). Tiles and FP16 storage: always (FP16 at 16^3x32, 2 to 12
+// systems: 6 to 12 % of an iteration). Block-interleaved in FP32 only where p, x and r exceed L2 and the
+// passes that the fusion saves go to memory (an iteration of 8 systems at 16^3x32 330 us without, 325 with;
+// at 20^3x40 747, 729; but 2 at 16^3x32 105, 108, 4 at 16^3x20 124, 132, 12 at 12^3x24 173, 178), or where
+// the launch is between half a wave and one (four resident blocks on each SM): its blocks then all run
+// at once, and each ends a little later in place of two further launches (2 at 16^4 62 and 60 us, 6 at
+// 16x6x4x38 50 and 48; on fewer blocks the separate kernels reach more SMs: 2 to 8 at 8^4 40 to 46 and 42 to 47).
+static bool fuse_in_batch(int ps, int mapping, double sum_vh) {
+    if (ps == BQ_PREC_DOUBLE) return false;
+    if (ps == BQ_PREC_HALF || mapping <= -3) return true;
+    const double blocks = sum_vh / 128.0;
+    return 3.0 * spinor_bytes_per_site(ps) * sum_vh > BQ_L2_BYTES || (blocks > 2.0 * BQ_SMS && blocks <= 4.0 * BQ_SMS);
+}
+
 template <int PS, int PR>
 static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double *shifts,
                         const bq_solver_params *sp, bool have_x0, int rhs_per_unit, bq_solver_stats *st) {
@@ -803,9 +818,10 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     }
     // several FP32 / FP16 systems in the shared-memory tile mapping or block-interleaved: the same fusion
     // inside those kernels, one partial per system and tile of 32 sites, or block of 128
-    const bool fuse_batch = nsys > 1 && PS != BQ_PREC_DOUBLE && (mapping <= -3 || mapping == -1);
     BatchCg tcg{};
     double sum_vh = 0.0;
+    for (int i = 0; i < nsys; i++) sum_vh += ctxs[i]->Vh;
+    const bool fuse_batch = nsys > 1 && (mapping <= -3 || mapping == -1) && fuse_in_batch(PS, mapping, sum_vh);
     if (fuse_batch) {
         const int psites = mapping == -1 ? 128 : 32, pstride = (maxVh + psites - 1) / psites;
         const size_t need = (size_t)nsys * 2 * pstride;
@@ -817,7 +833,6 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
             w->fpart_n = need;
         }
         tcg = BatchCg{w->d_sys, w->d_scal, w->d_fpart, pstride, psites};
-        for (int i = 0; i < nsys; i++) sum_vh += ctxs[i]->Vh;
     }
 
     for (int i = 0; i < nsys; i++) {
