@@ -598,63 +598,6 @@ static int mdagm_batch(bq_ctx *c0, int prec, int recon, int first_step, const Un
     return BQ_OK;
 }
 
-// Autotuner of the batched hopping term: times one sloppy Mhat^dag Mhat of the
-// batch (after one warm-up) for each rhs mapping -- block-interleaved units,
-// warp-per-rhs units and warp-interleaved units of 2, 4 and 8 -- and keeps the fastest for this batch
-// (same contexts, same number of systems, same precision) on later calls; the
-// last few batch signatures are remembered.
-static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int *mapping) {
-    BatchWork *w = c0->batch;
-    unsigned long long sig = 1469598103934665603ull ^ (unsigned long long)nsys ^ ((unsigned long long)ps << 40);
-    int maxrun = 1, run = 1;
-    for (int i = 0; i < nsys; i++) {
-        sig = (sig ^ (unsigned long long)(uintptr_t)ctxs[i]) * 1099511628211ull;
-        if (i > 0) run = (ctxs[i] == ctxs[i - 1]) ? run + 1 : 1;
-        maxrun = run > maxrun ? run : maxrun;
-    }
-    for (int e = 0; e < BatchWork::TUNE_CACHE; e++)
-        if (w->tuned_sig[e] == sig) {
-            *mapping = w->tuned_mapping[e];
-            return BQ_OK;
-        }
-    int cand[8] = {-1, -2, 2, 4, 8};
-    int ncand = 2;
-    for (int k = 2; k < 5; k++)
-        if (cand[k] <= maxrun) cand[ncand++] = cand[k];
-    if (ps != BQ_PREC_DOUBLE)
-        for (int m = -3; m >= -5; m--) cand[ncand++] = m;
-    double *h_on = w->h_flags;
-    for (int i = 0; i < nsys; i++) h_on[i] = 1.0;
-    BQ_CUDA_TRY(cudaMemcpyAsync(w->d_flags, h_on, sizeof(double) * nsys, cudaMemcpyHostToDevice, c0->stream));
-    const int recon = ctxs[0]->links_recon[ps];
-    float best = 1e30f;
-    int best_m = -1;
-    for (int k = 0; k < ncand; k++) {
-        UnitPlan plan;
-        BQ_TRY(build_units(c0, nsys, ctxs, ps, cand[k], &plan));
-        BQ_TRY(mdagm_batch(c0, ps, recon, 0, &plan, nsys, w->d_flags, 1.0));  // warm-up
-        float ms = 1e30f;
-        for (int rep = 0; rep < 2; rep++) {  // the better of two timed applications
-            BQ_CUDA_TRY(cudaEventRecord(w->t0, c0->stream));
-            BQ_TRY(mdagm_batch(c0, ps, recon, 0, &plan, nsys, w->d_flags, 1.0));
-            BQ_CUDA_TRY(cudaEventRecord(w->t1, c0->stream));
-            BQ_CUDA_TRY(cudaEventSynchronize(w->t1));
-            float t = 0.f;
-            BQ_CUDA_TRY(cudaEventElapsedTime(&t, w->t0, w->t1));
-            ms = t < ms ? t : ms;
-        }
-        if (ms < best) {
-            best = ms;
-            best_m = cand[k];
-        }
-    }
-    w->tuned_sig[w->tuned_next] = sig;
-    w->tuned_mapping[w->tuned_next] = best_m;
-    w->tuned_next = (w->tuned_next + 1) % BatchWork::TUNE_CACHE;
-    *mapping = best_m;
-    return BQ_OK;
-}
-
 // --------------------------------------------------------------------------
 // CUDA graph of the iteration body
 
@@ -736,6 +679,85 @@ static unsigned long long fnv(unsigned long long h, const void *p, size_t n) {
     return h;
 }
 
+// Autotuner of the batched hopping term: times what the caller runs (after one
+// warm-up) for each rhs mapping -- block-interleaved units, warp-per-rhs units,
+// warp-interleaved units of 2, 4 and 8, and the tiles -- and keeps the fastest for this batch
+// (same caller, same contexts, same number of systems, same precision) on later calls; the
+// last few batch signatures are remembered. use(m) sets up mapping m, run() queues the work:
+// a CG iteration for the solver (the vector work rides on the hopping launches in some mappings
+// only; by Mhat^dag Mhat alone, eight systems at 16^3x32 with 18-real links took block-interleaved
+// units, 334 us an iteration, where tiles take 307), Mhat^dag Mhat for the block multishift. `graphs`: as
+// a captured graph, where the caller runs that (the launch gaps of a stream, about 2 us for every launch
+// without programmatic dependence, count against the fused steps).
+template <typename Use, typename Run>
+static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int caller, bool graphs, Use use, Run run,
+                        int *mapping) {
+    BatchWork *w = c0->batch;
+    unsigned long long sig = 1469598103934665603ull ^ (unsigned long long)nsys ^ ((unsigned long long)ps << 40) ^
+                             ((unsigned long long)caller << 48);
+    int maxrun = 1, len = 1;
+    for (int i = 0; i < nsys; i++) {
+        sig = (sig ^ (unsigned long long)(uintptr_t)ctxs[i]) * 1099511628211ull;
+        if (i > 0) len = (ctxs[i] == ctxs[i - 1]) ? len + 1 : 1;
+        maxrun = len > maxrun ? len : maxrun;
+    }
+    for (int e = 0; e < BatchWork::TUNE_CACHE; e++)
+        if (w->tuned_sig[e] == sig) {
+            *mapping = w->tuned_mapping[e];
+            return BQ_OK;
+        }
+    int cand[8] = {-1, -2, 2, 4, 8};
+    int ncand = 2;
+    for (int k = 2; k < 5; k++)
+        if (cand[k] <= maxrun) cand[ncand++] = cand[k];
+    if (ps != BQ_PREC_DOUBLE)
+        for (int m = -3; m >= -5; m--) cand[ncand++] = m;
+    double *h_on = w->h_flags;
+    for (int i = 0; i < nsys; i++) h_on[i] = 1.0;
+    BQ_CUDA_TRY(cudaMemcpyAsync(w->d_flags, h_on, sizeof(double) * nsys, cudaMemcpyHostToDevice, c0->stream));
+    float best = 1e30f;
+    int best_m = -1;
+    for (int k = 0; k < ncand; k++) {
+        BQ_TRY(use(cand[k]));
+        BQ_TRY(run());  // warm-up
+        GraphRun gr;
+        auto body = [&](double) { return run(); };
+        if (graphs) {
+            const int st = capture_iterations(c0, 1, body, &gr);
+            if (st != BQ_OK) {
+                drop_graph(c0, &gr);
+                return st;
+            }
+        }
+        float ms = 1e30f;
+        for (int rep = 0; rep < 2; rep++) {  // the better of two
+            BQ_CUDA_TRY(cudaEventRecord(w->t0, c0->stream));
+            if (gr.exec) {
+                BQ_CUDA_TRY(cudaGraphLaunch(gr.exec, c0->stream));
+                credit_replay(c0, gr, 1.0);
+            } else {
+                BQ_TRY(run());
+            }
+            BQ_CUDA_TRY(cudaEventRecord(w->t1, c0->stream));
+            BQ_CUDA_TRY(cudaEventSynchronize(w->t1));
+            float t = 0.f;
+            BQ_CUDA_TRY(cudaEventElapsedTime(&t, w->t0, w->t1));
+            ms = t < ms ? t : ms;
+            if (gr.exec && c0->timing) BQ_TRY(bq_fold_slots(c0, gr.slot0, gr.slot0 + gr.nslots));
+        }
+        drop_graph(c0, &gr);
+        if (ms < best) {
+            best = ms;
+            best_m = cand[k];
+        }
+    }
+    w->tuned_sig[w->tuned_next] = sig;
+    w->tuned_mapping[w->tuned_next] = best_m;
+    w->tuned_next = (w->tuned_next + 1) % BatchWork::TUNE_CACHE;
+    *mapping = best_m;
+    return BQ_OK;
+}
+
 // --------------------------------------------------------------------------
 // the batched solver core
 
@@ -774,14 +796,7 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
         hs[i] = SysVec{sl->b, sl->x, sl->r, sl->t, sl->rs, sl->xs, sl->p, sl->Ap, sl->Vh};
         hscal[(size_t)i * S_NSCAL + S_SIGMA] = shifts ? shifts[i] : sp->shift;
     }
-    UnitPlan plan;
-    int mapping = rhs_per_unit ? rhs_per_unit : c0->batch_mapping;
-    if (nsys > 1 && mapping == 0) BQ_TRY(tune_mapping(c0, nsys, ctxs, PS, &mapping));
-    BQ_TRY(build_units(c0, nsys, ctxs, PS, mapping, &plan));
-    c0->batch_mapping_used = nsys > 1 ? mapping : 0;
     BQ_CUDA_TRY(cudaMemcpyAsync(w->d_sys, hs.data(), sizeof(SysVec) * nsys, cudaMemcpyHostToDevice, s));
-    BQ_CUDA_TRY(cudaMemcpyAsync(w->d_scal, hscal.data(), sizeof(double) * S_NSCAL * nsys, cudaMemcpyHostToDevice, s));
-    BQ_CUDA_TRY(cudaStreamSynchronize(s));
     int status = BQ_OK;
 
     double *active = w->h_flags, *update = w->h_flags + nsys;
@@ -818,11 +833,16 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     }
     // several FP32 / FP16 systems in the shared-memory tile mapping or block-interleaved: the same fusion
     // inside those kernels, one partial per system and tile of 32 sites, or block of 128
+    UnitPlan plan;
     BatchCg tcg{};
+    bool fuse_batch = false;
     double sum_vh = 0.0;
     for (int i = 0; i < nsys; i++) sum_vh += ctxs[i]->Vh;
-    const bool fuse_batch = nsys > 1 && (mapping <= -3 || mapping == -1) && fuse_in_batch(PS, mapping, sum_vh);
-    if (fuse_batch) {
+    // the launch tables of a mapping, and what its iterations need besides
+    auto use_mapping = [&](int mapping) -> int {
+        BQ_TRY(build_units(c0, nsys, ctxs, PS, mapping, &plan));
+        fuse_batch = nsys > 1 && (mapping <= -3 || mapping == -1) && fuse_in_batch(PS, mapping, sum_vh);
+        if (!fuse_batch) return BQ_OK;
         const int psites = mapping == -1 ? 128 : 32, pstride = (maxVh + psites - 1) / psites;
         const size_t need = (size_t)nsys * 2 * pstride;
         if (w->fpart_n < need) {
@@ -833,44 +853,8 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
             w->fpart_n = need;
         }
         tcg = BatchCg{w->d_sys, w->d_scal, w->d_fpart, pstride, psites};
-    }
-
-    for (int i = 0; i < nsys; i++) {
-        active[i] = 1.0;
-        update[i] = have_x0 ? 1.0 : 0.0;
-        memset(&st[i], 0, sizeof st[i]);
-    }
-    BQ_TRY(upload_flags());
-    if (have_x0) {
-        BQ_TRY(mdagm_batch(c0, BQ_PREC_DOUBLE, recon_d, 4, &plan, nsys, d_update, 1.0));
-        for (int i = 0; i < nsys; i++) {
-            update[i] = 0.0;
-            st[i].dslash_calls = 4;
-        }
-        BQ_TRY(upload_flags());
-    }
-    kb_init<PS, PR><<<G, RED_THREADS, 0, s>>>(ba_act, have_x0 ? 1 : 0);
-    BQ_COUNT(c0);
-    BQ_LAUNCH_CHECK();
-    BQ_TRY(read_scal());
-    std::vector<double> bb(nsys), maxrr(nsys), rrtrue(nsys);
-    int nactive = 0;
-    for (int i = 0; i < nsys; i++) {
-        const double *sc = w->h_scal + (size_t)i * S_NSCAL;
-        bb[i] = sc[S_BB];
-        rrtrue[i] = maxrr[i] = sc[S_RR];
-        if (bb[i] == 0.0 || rrtrue[i] <= sp->tol * sp->tol * bb[i]) {
-            active[i] = 0.0;
-            st[i].converged = 1;
-            st[i].true_residual = bb[i] == 0.0 ? 0.0 : sqrt(rrtrue[i] / bb[i]);
-        } else {
-            nactive++;
-        }
-    }
-    BQ_TRY(upload_flags());
-    const double delta = (PS == BQ_PREC_DOUBLE) ? 0.0 : sp->delta;
-    const int check = sp->check_every > 0 ? sp->check_every : 1;
-    int it = 0;
+        return BQ_OK;
+    };
     // one iteration of the whole batch, queued on c0->stream
     auto body = [&](double frac) -> int {
         kb_update_p<PS, PR><<<GP, RED_THREADS, 0, c0->stream>>>(ba_act);
@@ -910,6 +894,51 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
         BQ_LAUNCH_CHECK();
         return BQ_OK;
     };
+    // (the autotuner's iterations leave nothing but the sloppy vectors, which kb_init sets anew)
+    int mapping = rhs_per_unit ? rhs_per_unit : c0->batch_mapping;
+    if (nsys > 1 && mapping == 0)
+        BQ_TRY(tune_mapping(c0, nsys, ctxs, PS, 0, c0->use_graphs, use_mapping, [&] { return body(1.0); }, &mapping));
+    BQ_TRY(use_mapping(mapping));
+    c0->batch_mapping_used = nsys > 1 ? mapping : 0;
+    BQ_CUDA_TRY(cudaMemcpyAsync(w->d_scal, hscal.data(), sizeof(double) * S_NSCAL * nsys, cudaMemcpyHostToDevice, s));
+    BQ_CUDA_TRY(cudaStreamSynchronize(s));
+
+    for (int i = 0; i < nsys; i++) {
+        active[i] = 1.0;
+        update[i] = have_x0 ? 1.0 : 0.0;
+        memset(&st[i], 0, sizeof st[i]);
+    }
+    BQ_TRY(upload_flags());
+    if (have_x0) {
+        BQ_TRY(mdagm_batch(c0, BQ_PREC_DOUBLE, recon_d, 4, &plan, nsys, d_update, 1.0));
+        for (int i = 0; i < nsys; i++) {
+            update[i] = 0.0;
+            st[i].dslash_calls = 4;
+        }
+        BQ_TRY(upload_flags());
+    }
+    kb_init<PS, PR><<<G, RED_THREADS, 0, s>>>(ba_act, have_x0 ? 1 : 0);
+    BQ_COUNT(c0);
+    BQ_LAUNCH_CHECK();
+    BQ_TRY(read_scal());
+    std::vector<double> bb(nsys), maxrr(nsys), rrtrue(nsys);
+    int nactive = 0;
+    for (int i = 0; i < nsys; i++) {
+        const double *sc = w->h_scal + (size_t)i * S_NSCAL;
+        bb[i] = sc[S_BB];
+        rrtrue[i] = maxrr[i] = sc[S_RR];
+        if (bb[i] == 0.0 || rrtrue[i] <= sp->tol * sp->tol * bb[i]) {
+            active[i] = 0.0;
+            st[i].converged = 1;
+            st[i].true_residual = bb[i] == 0.0 ? 0.0 : sqrt(rrtrue[i] / bb[i]);
+        } else {
+            nactive++;
+        }
+    }
+    BQ_TRY(upload_flags());
+    const double delta = (PS == BQ_PREC_DOUBLE) ? 0.0 : sp->delta;
+    const int check = sp->check_every > 0 ? sp->check_every : 1;
+    int it = 0;
     // check_every iterations captured once as a CUDA graph on a private stream
     // and launched on the library stream; the capture's counter increments
     // describe one launch of the graph
@@ -1254,8 +1283,12 @@ static int ms_block_run(bq_ctx *c0, int nrhs, int n, const double *shifts, int b
     }
     UnitPlan plan;
     int mapping = c0->batch_mapping ? c0->batch_mapping : -1;
-    if (nrhs > 1 && c0->batch_mapping == 0) BQ_TRY(tune_mapping(c0, nrhs, ctxs.data(), PS, &mapping));
-    BQ_TRY(build_units(c0, nrhs, ctxs.data(), PS, mapping, &plan));
+    auto use_mapping = [&](int m) -> int { return build_units(c0, nrhs, ctxs.data(), PS, m, &plan); };
+    const int recon_t = c0->links_recon[PS];
+    if (nrhs > 1 && c0->batch_mapping == 0)
+        BQ_TRY(tune_mapping(c0, nrhs, ctxs.data(), PS, 1, false, use_mapping,
+                            [&] { return mdagm_batch(c0, PS, recon_t, 0, &plan, nrhs, w->d_flags, 1.0); }, &mapping));
+    BQ_TRY(use_mapping(mapping));
     c0->batch_mapping_used = nrhs > 1 ? mapping : 0;
     BQ_CUDA_TRY(cudaMemcpyAsync(w->d_sys, hs.data(), sizeof(SysVec) * nrhs, cudaMemcpyHostToDevice, s));
     BQ_CUDA_TRY(cudaMemcpyAsync(w->d_scal, hscal.data(), sizeof(double) * S_NSCAL * nrhs, cudaMemcpyHostToDevice, s));
@@ -1494,7 +1527,9 @@ extern "C" int bq_apply_mdagm_batch(bq_ctx *const *ctxs, int nsys, void *const *
         // tiles where their staging pays: eight right-hand sides per lattice on average. 24^3x48 FP32 with
         // 4 / 8 / 12 right-hand sides 499 / 928 / 1414 us block-interleaved, 567 / 898 / 1256 us in tiles;
         // FP16 456 / 880 / 1327 against 492 / 756 / 1030 (five resident blocks); four different lattices
-        // of one right-hand side each 343 us in tiles (three of four warps idle), 130 us block-interleaved
+        // of one right-hand side each 343 us in tiles (three of four warps idle), 130 us block-interleaved.
+        // Seven right-hand sides block-interleaved against tiles: 8^4 22 / 40 us, 16^3x32 169 / 214, 24^3x48
+        // 814 / 864, 32^4 1303 / 1353
         int runs = 1;
         for (int i = 1; i < nsys; i++) runs += ctxs[i] != ctxs[i - 1];
         mapping = (prec == BQ_PREC_DOUBLE || nsys < 8 * runs) ? -1 : prec == BQ_PREC_HALF ? -4 : -3;
