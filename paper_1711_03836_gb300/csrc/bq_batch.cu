@@ -679,19 +679,18 @@ static unsigned long long fnv(unsigned long long h, const void *p, size_t n) {
     return h;
 }
 
-// Autotuner of the batched hopping term: times what the caller runs (after one
-// warm-up) for each rhs mapping -- block-interleaved units, warp-per-rhs units,
+// Autotuner of the batched hopping term: times what the caller runs for each rhs mapping -- block-interleaved units, warp-per-rhs units,
 // warp-interleaved units of 2, 4 and 8, and the tiles -- and keeps the fastest for this batch
 // (same caller, same contexts, same number of systems, same precision) on later calls; the
 // last few batch signatures are remembered. use(m) sets up mapping m, run() queues the work:
 // a CG iteration for the solver (the vector work rides on the hopping launches in some mappings
 // only; by Mhat^dag Mhat alone, eight systems at 16^3x32 with 18-real links took block-interleaved
-// units, 334 us an iteration, where tiles take 307), Mhat^dag Mhat for the block multishift. `graphs`: as
-// a captured graph, where the caller runs that (the launch gaps of a stream, about 2 us for every launch
-// without programmatic dependence, count against the fused steps).
+// units, 334 us an iteration, where tiles take 307), Mhat^dag Mhat for the block multishift. run() gives
+// how many more ordinary launches than with separate vector kernels it made: in a stream each leaves
+// a gap of about 2.3 us that the captured graph of the solver does not have (capturing every candidate
+// instead took 0.1 to 0.4 ms each, 3 of the 39 ms of a first solve of ten shifts at 16^3x32).
 template <typename Use, typename Run>
-static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int caller, bool graphs, Use use, Run run,
-                        int *mapping) {
+static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int caller, Use use, Run run, int *mapping) {
     BatchWork *w = c0->batch;
     unsigned long long sig = 1469598103934665603ull ^ (unsigned long long)nsys ^ ((unsigned long long)ps << 40) ^
                              ((unsigned long long)caller << 48);
@@ -719,33 +718,18 @@ static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int c
     int best_m = -1;
     for (int k = 0; k < ncand; k++) {
         BQ_TRY(use(cand[k]));
-        BQ_TRY(run());  // warm-up
-        GraphRun gr;
-        auto body = [&](double) { return run(); };
-        if (graphs) {
-            const int st = capture_iterations(c0, 1, body, &gr);
-            if (st != BQ_OK) {
-                drop_graph(c0, &gr);
-                return st;
-            }
-        }
         float ms = 1e30f;
         for (int rep = 0; rep < 2; rep++) {  // the better of two
+            int gaps = 0;
             BQ_CUDA_TRY(cudaEventRecord(w->t0, c0->stream));
-            if (gr.exec) {
-                BQ_CUDA_TRY(cudaGraphLaunch(gr.exec, c0->stream));
-                credit_replay(c0, gr, 1.0);
-            } else {
-                BQ_TRY(run());
-            }
+            BQ_TRY(run(&gaps));
             BQ_CUDA_TRY(cudaEventRecord(w->t1, c0->stream));
             BQ_CUDA_TRY(cudaEventSynchronize(w->t1));
             float t = 0.f;
             BQ_CUDA_TRY(cudaEventElapsedTime(&t, w->t0, w->t1));
+            t -= 2.3e-3f * gaps;
             ms = t < ms ? t : ms;
-            if (gr.exec && c0->timing) BQ_TRY(bq_fold_slots(c0, gr.slot0, gr.slot0 + gr.nslots));
         }
-        drop_graph(c0, &gr);
         if (ms < best) {
             best = ms;
             best_m = cand[k];
@@ -897,7 +881,12 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     // (the autotuner's iterations leave nothing but the sloppy vectors, which kb_init sets anew)
     int mapping = rhs_per_unit ? rhs_per_unit : c0->batch_mapping;
     if (nsys > 1 && mapping == 0)
-        BQ_TRY(tune_mapping(c0, nsys, ctxs, PS, 0, c0->use_graphs, use_mapping, [&] { return body(1.0); }, &mapping));
+        BQ_TRY(tune_mapping(c0, nsys, ctxs, PS, 0, use_mapping,
+                            [&](int *gaps) {
+                                *gaps = fuse_batch && c0->use_graphs ? 2 : 0;
+                                return body(1.0);
+                            },
+                            &mapping));
     BQ_TRY(use_mapping(mapping));
     c0->batch_mapping_used = nsys > 1 ? mapping : 0;
     BQ_CUDA_TRY(cudaMemcpyAsync(w->d_scal, hscal.data(), sizeof(double) * S_NSCAL * nsys, cudaMemcpyHostToDevice, s));
@@ -1071,6 +1060,7 @@ int bq_batch_prepare(int nsys, bq_ctx *const *ctxs, int ps) {
         BQ_TRY(bq_prepare_clover(c, BQ_PREC_DOUBLE));
         BQ_TRY(bq_prepare_links(c, ps));
         BQ_TRY(bq_prepare_clover(c, ps));
+        BQ_TRY(bq_fields_written(c));
         // field preparation ran on this context's stream; the batch runs on ctx[0]'s
         if (c->stream != ctxs[0]->stream) {
             c->read_elsewhere = 1;
@@ -1286,8 +1276,9 @@ static int ms_block_run(bq_ctx *c0, int nrhs, int n, const double *shifts, int b
     auto use_mapping = [&](int m) -> int { return build_units(c0, nrhs, ctxs.data(), PS, m, &plan); };
     const int recon_t = c0->links_recon[PS];
     if (nrhs > 1 && c0->batch_mapping == 0)
-        BQ_TRY(tune_mapping(c0, nrhs, ctxs.data(), PS, 1, false, use_mapping,
-                            [&] { return mdagm_batch(c0, PS, recon_t, 0, &plan, nrhs, w->d_flags, 1.0); }, &mapping));
+        BQ_TRY(tune_mapping(c0, nrhs, ctxs.data(), PS, 1, use_mapping,
+                            [&](int *) { return mdagm_batch(c0, PS, recon_t, 0, &plan, nrhs, w->d_flags, 1.0); },
+                            &mapping));
     BQ_TRY(use_mapping(mapping));
     c0->batch_mapping_used = nrhs > 1 ? mapping : 0;
     BQ_CUDA_TRY(cudaMemcpyAsync(w->d_sys, hs.data(), sizeof(SysVec) * nrhs, cudaMemcpyHostToDevice, s));

@@ -238,6 +238,7 @@ int bq_dslash_unit_fill(bq_ctx *c, int prec, int out_parity, int dagger, int epi
     const int fs = field_store(c, prec);
     BQ_TRY(bq_prepare_links(c, fs));
     if (epi != EPI_PLAIN) BQ_TRY(bq_prepare_clover(c, fs));
+    BQ_TRY(bq_fields_written(c));
     a->out = nullptr;
     a->in = nullptr;
     a->xin = nullptr;

@@ -392,7 +392,7 @@ extern "C" int bq_set_u1(bq_ctx *c, const double *A, int where) {
 
 // REBUILD: 12-real FP64 links, third row = conj(row 0 x row 1), rebuilt here once and stored
 // (the FP64 kernels are bound by arithmetic: rebuilding it at every hop cost the double-float
-// kernel 40 % and the FP64-unit one 20 %)
+// kernel 40 % and the FP64-unit one 20 %; stored, it takes 48 bytes a link more)
 template <int PREC, int RECON, bool REBUILD = false>
 __global__ void k_pack_links(char *dst, size_t blk, const double2 *U, const double *A, double charge, Geo g,
                              int *flag) {
@@ -428,6 +428,8 @@ __global__ void k_pack_links(char *dst, size_t blk, const double2 *U, const doub
 // a launch with programmatic dependence on it can only start after that.
 __global__ void k_fields_written() {}
 int bq_fields_written(bq_ctx *c) {
+    if (!c->fields_fresh) return BQ_OK;
+    c->fields_fresh = 0;
     k_fields_written<<<1, 1, 0, c->stream>>>();
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
@@ -472,9 +474,9 @@ int bq_prepare_links(bq_ctx *c, int prec) {
         if (rebuild) PACK(BQ_PREC_DF64, 18, true); else PACK(BQ_PREC_DF64, 18);
     }
 #undef PACK
+    c->fields_fresh = 1;
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
-    BQ_TRY(bq_fields_written(c));
     if (recon == BQ_RECON_8) {
         int flag = 0;
         BQ_CUDA_TRY(cudaMemcpyAsync(&flag, c->dev_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -889,9 +891,9 @@ int bq_prepare_clover(bq_ctx *c, int prec) {
         k_convert_clover<BQ_PREC_DF64><<<grid, 128, 0, c->stream>>>(c->clov[prec], (const double2 *)c->clov_master, c->Vh, 4);
     else
         k_convert_clover<BQ_PREC_HALF><<<grid, 128, 0, c->stream>>>(c->clov[prec], (const double2 *)c->clov_master, c->Vh, 4);
+    c->fields_fresh = 1;
     BQ_LAUNCH_CHECK();
     BQ_COUNT(c);
-    BQ_TRY(bq_fields_written(c));
     c->clov_valid[prec] = 1;
     return BQ_OK;
 }

@@ -39,7 +39,9 @@ void bq_set_error(const char *fmt, ...);
 // the SMs of the running kernel leave an uneven distribution behind (FP64, 12^4: 158 -> 307 us).
 // Links and clover blocks are read through the read-only path, whose loads may be scheduled ahead
 // of bq_pdl_enter(): after the kernels that write them, bq_fields_written() keeps every later
-// launch, by whichever context or thread, behind their end.
+// launch, by whichever context or thread, behind their end. Every operator call has it between
+// the preparation of its fields and its first launch; a call that is refused in between leaves it to the
+// context's next one.
 template <typename... P, typename... A>
 inline void bq_launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args) {
     cudaLaunchAttribute at;
@@ -95,6 +97,7 @@ struct bq_ctx {
     char *links[BQ_NFIELD];
     int links_recon[BQ_NFIELD];
     int links_valid[BQ_NFIELD];
+    int fields_fresh;              // links or clover blocks written since bq_fields_written
     double *clov_master;           // FP64 packed, [parity][inverse] blocks of 72*Vh reals
     int clov_master_valid;
     int clov_user;                 // clov_master holds a caller-supplied field (bq_set_clover)
@@ -141,7 +144,7 @@ int bq_time_end(bq_ctx *c, int slot);
 // field preparation (bq_fields.cu)
 int bq_prepare_links(bq_ctx *c, int prec);
 int bq_prepare_clover(bq_ctx *c, int prec);
-int bq_fields_written(bq_ctx *c);  // see bq_launch
+int bq_fields_written(bq_ctx *c);  // after these and before a launch by bq_launch that reads the fields
 // A place for split links in memory that holds no valid field (p null: there is none), or where the split of
 // U_canon lies already. build: the clover term is about to be built, so that the blocks of its inverse hold nothing.
 PairLinks bq_split_place(const bq_ctx *c, bool build);
@@ -264,12 +267,13 @@ void bq_interleaved_cg_launch(int prec, int recon, const DslashBatchTable &tab, 
 int bq_cg_finish_batch(bq_ctx *c, int mode, const BatchCg &cg, const double *mask, int nsys);
 
 // The CG vector work fused into the two A x - k D launches of one CG iteration
-// on Mhat^dag Mhat + sigma (single system, FP32 or FP16-storage inner iteration; bq_cgfuse.cu).
+// on Mhat^dag Mhat + sigma (one system: FP32 or FP16-storage inner iteration, bq_cgfuse.cu; any storage
+// on a small lattice, FP64 on the FP64 units, bq_split.cu).
 // scal: the system's solver scalars (S_* slots of bq_reduce.cuh); partials: 2 doubles
-// per 128-site block of the launch (2 * ceil(V/2 / 128))
+// per block of the launch (128 sites, on a small lattice 16)
 struct CgFuse {
     const void *p;  // search direction, precision ps
-    void *xs, *rs;  // iterated solution and residual, FP32
+    void *xs, *rs;  // iterated solution and residual: FP32, or FP64 with an FP64 p
     double *scal;
     double *partials;
     int with_pnorm;  // sum |p|^2 too (the shift is nonzero); the eight-thread kernels read the shift instead
