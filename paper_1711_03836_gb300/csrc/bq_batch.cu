@@ -517,7 +517,7 @@ static int build_units(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int ma
             DslashUnit *u = &tab.units[tab.nunits];
             BQ_TRY(bq_dslash_unit_fill(c, prec, parity, dagger, epi, kk, &u->a));
             u->nr = e - s;
-            const int recon = c->links_recon[(prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) ? 3 : prec];
+            const int recon = c->links_recon[bq_field_store(c, prec)];
             u->a.rev = bq_reverse(prec, recon, epi, c->Vh, u->nr);  // the working set of nr right-hand sides
             wset += bq_working_set(prec, recon, c->Vh, u->nr);
             u->log2R = log2_ceil(u->nr);
@@ -686,8 +686,8 @@ static unsigned long long fnv(unsigned long long h, const void *p, size_t n) {
 // a CG iteration for the solver (the vector work rides on the hopping launches in some mappings
 // only; by Mhat^dag Mhat alone, eight systems at 16^3x32 with 18-real links took block-interleaved
 // units, 334 us an iteration, where tiles take 307), Mhat^dag Mhat for the block multishift. run() gives
-// how many more ordinary launches than with separate vector kernels it made: in a stream each leaves
-// a gap of about 2.3 us that the captured graph of the solver does not have (capturing every candidate
+// how many more ordinary launches than with separate vector kernels it made: in a stream each costs
+// about 1.2 us that it does not in the captured graph of the solver (capturing every candidate
 // instead took 0.1 to 0.4 ms each, 3 of the 39 ms of a first solve of ten shifts at 16^3x32).
 template <typename Use, typename Run>
 static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int caller, Use use, Run run, int *mapping) {
@@ -727,7 +727,7 @@ static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int c
             BQ_CUDA_TRY(cudaEventSynchronize(w->t1));
             float t = 0.f;
             BQ_CUDA_TRY(cudaEventElapsedTime(&t, w->t0, w->t1));
-            t -= 2.3e-3f * gaps;
+            t -= 1.2e-3f * gaps;
             ms = t < ms ? t : ms;
         }
         if (ms < best) {
@@ -766,7 +766,7 @@ static int cg_batch_run(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const double 
     BatchWork *w = c0->batch;
     cudaStream_t s = c0->stream;
     const int recon_s = ctxs[0]->links_recon[PS];
-    const int recon_d = ctxs[0]->links_recon[ctxs[0]->fp64_arith == BQ_FP64_DF64 ? 3 : BQ_PREC_DOUBLE];
+    const int recon_d = ctxs[0]->links_recon[bq_field_store(ctxs[0], BQ_PREC_DOUBLE)];
     int maxVh = 0;
     for (int i = 0; i < nsys; i++) maxVh = ctxs[i]->Vh > maxVh ? ctxs[i]->Vh : maxVh;
     const dim3 G(red_grid(maxVh), nsys);
@@ -1036,7 +1036,7 @@ static int cg_batch_dispatch(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, const do
 }
 
 // check a batch: same sloppy recon and FP64 arithmetic everywhere; fields prepared
-int bq_batch_prepare(int nsys, bq_ctx *const *ctxs, int ps) {
+int bq_batch_prepare(int nsys, bq_ctx *const *ctxs, int ps, bool fp64) {
     for (int i = 0; i < nsys; i++) {
         bq_ctx *c = ctxs[i];
         if (!c) {
@@ -1056,10 +1056,12 @@ int bq_batch_prepare(int nsys, bq_ctx *const *ctxs, int ps) {
             bq_set_error("batched CG: all contexts must be on one device");
             return BQ_ERR_ARG;
         }
-        BQ_TRY(bq_prepare_links(c, BQ_PREC_DOUBLE));
-        BQ_TRY(bq_prepare_clover(c, BQ_PREC_DOUBLE));
-        BQ_TRY(bq_prepare_links(c, ps));
-        BQ_TRY(bq_prepare_clover(c, ps));
+        // all fields that the launches read: later ones would be packed on a stream that the batch is not on
+        for (int prec : {fp64 ? (int)BQ_PREC_DOUBLE : ps, ps}) {
+            const int fs = bq_field_store(c, prec);
+            BQ_TRY(bq_prepare_links(c, fs));
+            BQ_TRY(bq_prepare_clover(c, fs));
+        }
         BQ_TRY(bq_fields_written(c));
         // field preparation ran on this context's stream; the batch runs on ctx[0]'s
         if (c->stream != ctxs[0]->stream) {
@@ -1510,7 +1512,7 @@ extern "C" int bq_apply_mdagm_batch(bq_ctx *const *ctxs, int nsys, void *const *
                 return BQ_ERR_ARG;
             }
     }
-    BQ_TRY(bq_batch_prepare(nsys, ctxs, prec));
+    BQ_TRY(bq_batch_prepare(nsys, ctxs, prec, false));
     bq_ctx *c0 = ctxs[0];
     BQ_TRY(bq_batch_reserve(c0, nsys, ctxs, prec, prec));
     int mapping = c0->batch_mapping;
@@ -1528,7 +1530,7 @@ extern "C" int bq_apply_mdagm_batch(bq_ctx *const *ctxs, int nsys, void *const *
     UnitPlan plan;
     BQ_TRY(build_units(c0, nsys, ctxs, prec, mapping, &plan, in, out));
     c0->batch_mapping_used = nsys > 1 ? mapping : 0;
-    const int recon = ctxs[0]->links_recon[(prec == BQ_PREC_DOUBLE && c0->fp64_arith == BQ_FP64_DF64) ? 3 : prec];
+    const int recon = ctxs[0]->links_recon[bq_field_store(ctxs[0], prec)];
     return mdagm_batch(c0, prec, recon, 0, &plan, nsys, nullptr, 1.0);
 }
 

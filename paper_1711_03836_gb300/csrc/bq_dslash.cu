@@ -100,14 +100,9 @@ static void launch_dslash_pr(const DslashArgs &a, bool dag, int epi, unsigned gr
     launch_dslash_prs<PREC, RECON, false>(a, dag, epi, grid, s);
 }
 
-// storage of the links and clover a launch at precision prec reads
-static int field_store(const bq_ctx *c, int prec) {
-    return (prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) ? (int)BQ_PREC_DF64 : prec;
-}
-
 int bq_dslash_launch(bq_ctx *c, int prec, void *out, const void *in, int out_parity, int dagger, int epi,
                      const void *xin, double k, int fmt) {
-    const int fs = field_store(c, prec);
+    const int fs = bq_field_store(c, prec);
     DslashArgs a;
     BQ_TRY(bq_dslash_unit_fill(c, prec, out_parity, dagger, epi, k, &a));
     a.out = out;
@@ -235,7 +230,7 @@ static void launch_batch_pr(const DslashBatchTable &tab, const double *mask, int
 // Fill the lattice-level part of a unit for one launch type (fields of c at
 // precision prec, output parity, adjoint, epilogue); the rhs pointers are the caller's.
 int bq_dslash_unit_fill(bq_ctx *c, int prec, int out_parity, int dagger, int epi, double k, DslashArgs *a) {
-    const int fs = field_store(c, prec);
+    const int fs = bq_field_store(c, prec);
     BQ_TRY(bq_prepare_links(c, fs));
     if (epi != EPI_PLAIN) BQ_TRY(bq_prepare_clover(c, fs));
     BQ_TRY(bq_fields_written(c));
@@ -296,7 +291,7 @@ int bq_dslash_batch_launch(bq_ctx *c, int prec, int recon, const DslashBatchTabl
 }
 
 int bq_clover_launch(bq_ctx *c, int prec, void *out, const void *in, int parity, int inverse) {
-    const int fs = field_store(c, prec);
+    const int fs = bq_field_store(c, prec);
     BQ_TRY(bq_prepare_clover(c, fs));
     const void *cl = clover_ptr(c, fs, parity, inverse);
     unsigned grid = (unsigned)((c->Vh + 127) / 128);

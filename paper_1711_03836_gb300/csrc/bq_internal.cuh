@@ -163,6 +163,10 @@ inline const char *clover_ptr(const bq_ctx *c, int prec, int parity, int inverse
     return c->clov[prec] + (size_t)(parity * 2 + inverse) * clover_bytes_per_site(prec) * c->Vh;
 }
 inline const char *links_ptr(const bq_ctx *c, int prec) { return c->links[prec]; }
+// storage of the links and clover a launch at precision prec reads
+inline int bq_field_store(const bq_ctx *c, int prec) {
+    return (prec == BQ_PREC_DOUBLE && c->fp64_arith == BQ_FP64_DF64) ? (int)BQ_PREC_DF64 : prec;
+}
 inline size_t links_block_bytes(const bq_ctx *c, int prec) {
     return link_bytes_per_link(prec, c->links_recon[prec]) * (size_t)c->Vh;
 }
@@ -286,7 +290,8 @@ int bq_dslash_cg_launch(bq_ctx *c, int ps, void *out, const void *in, const void
                         const CgFuse &f);
 
 // batched solver (bq_batch.cu)
-int bq_batch_prepare(int nsys, bq_ctx *const *ctxs, int ps);  // fields of every system at FP64 and ps
+// fields of every system at ps and, for a solver, in FP64
+int bq_batch_prepare(int nsys, bq_ctx *const *ctxs, int ps, bool fp64 = true);
 int bq_batch_reserve(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int pr);
 void *bq_batch_slot_b(bq_ctx *c0, int s);
 void *bq_batch_slot_x(bq_ctx *c0, int s);
