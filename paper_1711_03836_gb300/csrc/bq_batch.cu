@@ -687,7 +687,7 @@ static unsigned long long fnv(unsigned long long h, const void *p, size_t n) {
 // only; by Mhat^dag Mhat alone, eight systems at 16^3x32 with 18-real links took block-interleaved
 // units, 334 us an iteration, where tiles take 307), Mhat^dag Mhat for the block multishift. run() gives
 // how many more ordinary launches than with separate vector kernels it made: in a stream each costs
-// about 1.2 us that it does not in the captured graph of the solver (capturing every candidate
+// about 1.7 us that it does not in the captured graph of the solver (capturing every candidate
 // instead took 0.1 to 0.4 ms each, 3 of the 39 ms of a first solve of ten shifts at 16^3x32).
 template <typename Use, typename Run>
 static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int caller, Use use, Run run, int *mapping) {
@@ -727,7 +727,7 @@ static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int c
             BQ_CUDA_TRY(cudaEventSynchronize(w->t1));
             float t = 0.f;
             BQ_CUDA_TRY(cudaEventElapsedTime(&t, w->t0, w->t1));
-            t -= 1.2e-3f * gaps;
+            t -= 1.7e-3f * gaps;
             ms = t < ms ? t : ms;
         }
         if (ms < best) {
@@ -746,18 +746,20 @@ static int tune_mapping(bq_ctx *c0, int nsys, bq_ctx *const *ctxs, int ps, int c
 // the batched solver core
 
 // Whether the vector work of CG rides on the A x - k D launches of a batch in a tile mapping or
-// block-interleaved (sum_vh: sites of all systems). Tiles and FP16 storage: always (FP16 at 16^3x32, 2 to 12
-// systems: 6 to 12 % of an iteration). Block-interleaved in FP32 only where p, x and r exceed L2 and the
-// passes that the fusion saves go to memory (an iteration of 8 systems at 16^3x32 330 us without, 325 with;
-// at 20^3x40 747, 729; but 2 at 16^3x32 105, 108, 4 at 16^3x20 124, 132, 12 at 12^3x24 173, 178), or where
-// the launch is between half a wave and one (four resident blocks on each SM): its blocks then all run
-// at once, and each ends a little later in place of two further launches (2 at 16^4 62 and 60 us, 6 at
-// 16x6x4x38 50 and 48; on fewer blocks the separate kernels reach more SMs: 2 to 8 at 8^4 40 to 46 and 42 to 47).
+// block-interleaved (sum_vh: sites of all systems). Tiles: always. Block-interleaved not on fewer blocks than
+// half a wave (four resident blocks on each SM), where the separate kernels reach more SMs (FP32, 2 to 8
+// systems at 8^4 40 to 46 us an iteration without, 42 to 47 with it; FP16, 4 at 16x6x4x38 41.0 and 41.7).
+// FP16 storage: everywhere else (2 to 12 systems at 16^3x32 6 to 12 % of an iteration). FP32: up to one wave,
+// as its blocks then all run at once and each ends a little later in place of two further launches (2 at
+// 16^4 62 and 60 us, 6 at 16x6x4x38 50 and 48), and where p, x and r exceed L2, so that the passes saved go to
+// memory (8 at 16^3x32 330 and 325, at 20^3x40 747 and 729; in between 2 at 16^3x32 105 and 108, 4 at 16^3x20
+// 124 and 132, 12 at 12^3x24 173 and 178).
 static bool fuse_in_batch(int ps, int mapping, double sum_vh) {
     if (ps == BQ_PREC_DOUBLE) return false;
-    if (ps == BQ_PREC_HALF || mapping <= -3) return true;
+    if (mapping <= -3) return true;
     const double blocks = sum_vh / 128.0;
-    return 3.0 * spinor_bytes_per_site(ps) * sum_vh > BQ_L2_BYTES || (blocks > 2.0 * BQ_SMS && blocks <= 4.0 * BQ_SMS);
+    if (blocks <= 2.0 * BQ_SMS) return false;
+    return ps == BQ_PREC_HALF || blocks <= 4.0 * BQ_SMS || 3.0 * spinor_bytes_per_site(ps) * sum_vh > BQ_L2_BYTES;
 }
 
 template <int PS, int PR>
