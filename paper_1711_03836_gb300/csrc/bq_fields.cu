@@ -188,7 +188,6 @@ extern "C" int bq_set_recon(bq_ctx *c, int prec, int recon) {
     if (c->recon[prec] != recon) {
         c->recon[prec] = recon;
         c->links_valid[prec] = 0;
-        if (prec == BQ_PREC_DOUBLE) c->links_valid[BQ_PREC_DF64] = 0;
     }
     return BQ_OK;
 }
@@ -443,8 +442,10 @@ int bq_prepare_links(bq_ctx *c, int prec) {
     }
     const bool fp64 = prec == BQ_PREC_DF64 || prec == BQ_PREC_DOUBLE;  // df64 pairs follow the FP64 setting
     const int recon = fp64 ? BQ_RECON_18 : c->recon[prec];
-    if (c->links_valid[prec] && c->links_recon[prec] == recon) return BQ_OK;
-    const bool rebuild = fp64 && c->recon[BQ_PREC_DOUBLE] == BQ_RECON_12;
+    const int setting = c->recon[fp64 ? (int)BQ_PREC_DOUBLE : prec];
+    if (c->links_valid[prec] && c->links_setting[prec] == setting) return BQ_OK;
+    c->links_valid[prec] = 0;
+    const bool rebuild = fp64 && setting == BQ_RECON_12;
     size_t blk = link_bytes_per_link(prec, recon) * (size_t)c->Vh;
     if (c->links[prec] && c->links_recon[prec] != recon) {
         cudaFree(c->links[prec]);
@@ -452,6 +453,7 @@ int bq_prepare_links(bq_ctx *c, int prec) {
     }
     BQ_TRY(bq_alloc((void **)&c->links[prec], blk * 8));
     c->links_recon[prec] = recon;
+    c->links_setting[prec] = setting;
     Geo g = geo_of(c);
     unsigned grid = grid_for(c->V, 128);
     double q = c->params.charge;

@@ -96,6 +96,7 @@ struct bq_ctx {
     // derived native fields, rebuilt lazily
     char *links[BQ_NFIELD];
     int links_recon[BQ_NFIELD];
+    int links_setting[BQ_NFIELD];  // bq_set_recon's value when they were packed (FP64: 12 means a rebuilt third row)
     int links_valid[BQ_NFIELD];
     int fields_fresh;              // links or clover blocks written since bq_fields_written
     double *clov_master;           // FP64 packed, [parity][inverse] blocks of 72*Vh reals
