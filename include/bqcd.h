@@ -102,7 +102,8 @@ typedef struct {
  * the CG vector work fused in: 3 = t = Mhat p with |t|^2 and |p|^2 (so
  * <p, Ap> = |t|^2 + shift |p|^2), 4 = Mhat^dag t with the x and r updates and
  * |r|^2 (Ap itself is not stored). Batches in a tile mapping count the same steps
- * there; block-interleaved batches (mapping -1) count them as epilogue 2.
+ * there; block-interleaved batches (mapping -1), which run them where that is
+ * faster, count them as epilogue 2, with their vector work in fused_bytes[.][2].
  * Bytes and flops are ALGORITHMIC per launch: 8 links + 1 input + 1 output
  * spinor per output site, plus the clover blocks (and the x spinor) the fused
  * epilogue reads; 1320 flops per site for D_hop, +504 per clover apply,
@@ -138,7 +139,8 @@ int bq_set_params(bq_ctx *ctx, const bq_params *p);
  * U00 and U20; the rest rebuilt from unitarity and det U = 1, with two sine /
  * cosine evaluations, two square roots and one reciprocal per link). For
  * BQ_PREC_DOUBLE the third row of BQ_RECON_12 is rebuilt once, when the links are
- * packed, and kept with the other two. 12 and 8
+ * packed, and kept with the other two (576 bytes per lattice site with either
+ * setting). 12 and 8
  * are valid for SU(3) links only, so they are refused while a U(1) field is
  * set; 8 is singular where |U00| = 1, so the link packing (on the first
  * operator call) fails with BQ_ERR_ARG if a link has |U01|^2 + |U02|^2 < 1e-6

@@ -1,6 +1,9 @@
 // bq_cgfuse.cu -- one CG iteration on Mhat^dag Mhat + sigma (Section 3: cg)
 // with its vector work folded into the two hopping-term launches that end in
-// A x - k D (single system, FP32 or FP16-storage inner iteration).
+// A x - k D: one system with an FP32 or FP16-storage inner iteration, or a batch
+// of them block-interleaved (one thread per site, blocks of 128 sites). The same
+// steps for batches in tiles are in bq_tile.cu, for one system on a small lattice
+// (FP32, FP16 storage, FP64 on the FP64 units) in bq_split.cu.
 //
 // Of the four launches of Ap = (Mhat^dag Mhat + sigma) p the second produces
 // t = Mhat p = A_ee p - k D_eo A_oo^{-1} D_oe p and the fourth Mhat^dag t. As

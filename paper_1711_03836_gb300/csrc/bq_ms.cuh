@@ -211,7 +211,8 @@ __device__ __forceinline__ void ms_coef_body(const double *hist, double *coef, i
 
 // X_k += A_k P_k + sum_i W_{k,i} R_i and P_k = g_k P_k + sum_i C_{k,i} R_i for every shift,
 // groups of GROUP shifts per pass (the residuals are read once per group; ten in FP32, 80 registers of
-// sums); one thread per site and storage chunk (a float4 of two complex components for FP32, a
+// sums: against eight to a group and coefficients in FP64 whole solves of 1, 2, 4, 6, 8, 10, 12 and 16 shifts
+// take 16, 10, 12, 13, 15, 14, 12 and 12 % less at 16^3x32); one thread per site and storage chunk (a float4 of two complex components for FP32, a
 // double2 for FP64); coefficients in shared memory in the vectors' type: converting each from FP64
 // at its use kept the FP64 pipe busy for 430 of the 513 us of a 32-iteration chunk of ten shifts at 16^3x32
 
