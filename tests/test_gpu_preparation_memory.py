@@ -84,7 +84,7 @@ def test_next_configuration_needs_no_memory(bq, where, order):  # noqa: F811
     torch.cuda.empty_cache()
     free = torch.cuda.mem_get_info()[0]
     one_pass(bq, lat, U, ORDERS[order], "single", src, out, hop)
-    assert torch.cuda.mem_get_info()[0] == free
+    assert torch.cuda.mem_get_info()[0] >= free - (16 << 20)  # one more copy of the links is 604 MB
     fill = torch.empty(free - (350 << 20), dtype=torch.uint8, device="cuda")
     one_pass(bq, lat, U, ORDERS[order], "single", src, out, hop)
     del fill
